@@ -106,6 +106,7 @@ template <typename T> struct Dot;
 template <> struct Dot<double> {
   double s;
   __device__ __forceinline__ Dot() : s(0.0) {}
+  __device__ __forceinline__ Dot(double c, double x) : s(c * x) {}
   __device__ __forceinline__ void add(double c, double x) { s = fma(c, x, s); }
   __device__ __forceinline__ double get() const { return s; }
   __device__ __forceinline__ double raw() const { return s; }
@@ -114,6 +115,7 @@ template <> struct Dot<double> {
 template <> struct Dot<float> {
   float s;
   __device__ __forceinline__ Dot() : s(0.f) {}
+  __device__ __forceinline__ Dot(float c, float x) : s(c * x) {}
   __device__ __forceinline__ void add(float c, float x) { s = fmaf(c, x, s); }
   __device__ __forceinline__ float get() const { return s; }
   __device__ __forceinline__ float raw() const { return s; }
@@ -122,6 +124,11 @@ template <> struct Dot<float> {
 template <> struct Dot<df32> {
   float s, e;
   __device__ __forceinline__ Dot() : s(0.f), e(0.f) {}
+  // The first term by itself: 4 instructions instead of 12.
+  __device__ __forceinline__ Dot(df32 c, df32 x) {
+    s = __fmul_rn(c.hi, x.hi);
+    e = __fmaf_rn(c.lo, x.hi, __fmaf_rn(c.hi, x.lo, __fmaf_rn(c.hi, x.hi, -s)));
+  }
   __device__ __forceinline__ void add(df32 c, df32 x) {
     const float p = __fmul_rn(c.hi, x.hi);
     float err = __fmaf_rn(c.hi, x.hi, -p);
@@ -141,6 +148,62 @@ template <> struct Dot<df32> {
   // (|e| > |s|) an unevaluated pair whose sum is the dot product to the same absolute error.
   __device__ __forceinline__ df32 raw() const { return fast_two_sum(s, e); }
 };
+
+// Sum of products with a bound known beforehand: Bound collects b >= sum_i |c_i x_i|, Acc then adds
+// the terms.  double and float: the bound is empty and the sum is the FMA chain of Dot.  df32: the
+// leading parts are summed on top of an offset m = 2.125 b, so the running value a stays within
+// [1.1 b, 3.2 b]; there both a' - a (a' = fl(a + c x), one FMA) and the final a - m are exact (their
+// operands lie on the grid of the smaller one and differ by less than 2^24 of its steps), so the
+// rounding error of every step is one more FMA, c x - (a' - a) -- a two_sum whose three-operation
+// error term is free of the operands' order (Rump, Ogita & Oishi 2008, "Accurate floating-point
+// summation": extraction against a large constant).  7 FP32 instructions per term (the bound
+// included) and 4 at the end, where Dot takes 12 and 3; the offset costs at most two bits of the
+// error term, which is kept to 2^-24 of one grid step (about 2^-48 of b).
+template <typename T> struct Bound {
+  __device__ __forceinline__ void add(T, T) {}
+};
+template <> struct Bound<df32> {
+  float b;
+  __device__ __forceinline__ Bound() : b(0.f) {}
+  __device__ __forceinline__ void add(df32 c, df32 x) { b = __fmaf_rn(::fabsf(c.hi), ::fabsf(x.hi), b); }
+};
+
+template <typename T> struct Acc {
+  T s;
+  __device__ __forceinline__ explicit Acc(const Bound<T> &) : s(0) {}
+  __device__ __forceinline__ void add(T c, T x) { s = fma(c, x, s); }
+  __device__ __forceinline__ T raw() const { return s; }
+};
+template <> struct Acc<df32> {
+  float a, m, e;
+  __device__ __forceinline__ explicit Acc(const Bound<df32> &b) : e(0.f) { a = m = __fmul_rn(2.125f, b.b); }
+  __device__ __forceinline__ void add(df32 c, df32 x) {
+    const float t = __fmaf_rn(c.hi, x.hi, a);
+    float r = __fmaf_rn(c.hi, x.hi, -__fsub_rn(t, a));
+    r = __fmaf_rn(c.hi, x.lo, r);
+    r = __fmaf_rn(c.lo, x.hi, r);
+    a = t;
+    e = __fadd_rn(e, r);
+  }
+  __device__ __forceinline__ df32 raw() const { return fast_two_sum(__fsub_rn(a, m), e); }
+};
+
+// a0 b0 + a1 b1 + a2 b2.  df32: the leading products by two two_sums, every error in one term
+// (31 FP32 instructions; three Dot terms started from zero take 39).
+__device__ __forceinline__ double dot3(double a0, double b0, double a1, double b1, double a2, double b2) {
+  return fma(a2, b2, fma(a1, b1, a0 * b0));
+}
+__device__ __forceinline__ float dot3(float a0, float b0, float a1, float b1, float a2, float b2) {
+  return fmaf(a2, b2, fmaf(a1, b1, a0 * b0));
+}
+__device__ __forceinline__ df32 dot3(df32 a0, df32 b0, df32 a1, df32 b1, df32 a2, df32 b2) {
+  const float p0 = __fmul_rn(a0.hi, b0.hi), p1 = __fmul_rn(a1.hi, b1.hi), p2 = __fmul_rn(a2.hi, b2.hi);
+  const float e0 = __fmaf_rn(a0.lo, b0.hi, __fmaf_rn(a0.hi, b0.lo, __fmaf_rn(a0.hi, b0.hi, -p0)));
+  const float e1 = __fmaf_rn(a1.lo, b1.hi, __fmaf_rn(a1.hi, b1.lo, __fmaf_rn(a1.hi, b1.hi, -p1)));
+  const float e2 = __fmaf_rn(a2.lo, b2.hi, __fmaf_rn(a2.hi, b2.lo, __fmaf_rn(a2.hi, b2.hi, -p2)));
+  const df32 s = two_sum(p0, p1), t = two_sum(s.hi, p2);
+  return fast_two_sum(t.hi, __fadd_rn(__fadd_rn(__fadd_rn(e0, e1), __fadd_rn(e2, s.lo)), t.lo));
+}
 
 __device__ __forceinline__ df32 fabs(df32 x) { return x.hi < 0.f ? -x : x; }
 __device__ __forceinline__ bool operator<(df32 x, df32 y) { return x.hi < y.hi || (x.hi == y.hi && x.lo < y.lo); }

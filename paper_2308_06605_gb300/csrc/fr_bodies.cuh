@@ -301,11 +301,21 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   // FP32 viscous branch: Q minus the element's first point, in FP32, in the upper half of the
   // gradient buffer (the FP32 gradient uses only its lower half).
   TG *sQg = kPert ? reinterpret_cast<TG *>(sQ + 5 * Np) + 15 * Np : nullptr;   // [5][Np]
+  // Double-float viscous branch: sQ itself holds the perturbation (only the gradient reads it).
+  constexpr bool kPertDf = std::is_same<TG, df32>::value;
   const PhysT<T> &ph = phys_of<T>(dph);
   const PhysT<TG> &phg = phys_of<TG>(dph);
   const BasisT<T> &B = basis_ref<N, T, VC>(dph);
-  // Sums of products end with Dot::raw(): the compensated sum s + e renormalised by one
-  // fast_two_sum only (an error of the order of 2^-48 of the sum of the terms' magnitudes).
+  // Sums of products end with raw(): the compensated sum renormalised by one fast_two_sum only (an
+  // error of the order of 2^-48 of the sum of the terms' magnitudes).  The gradient and the gradient
+  // traces use the cheaper bounded sums (Acc); in double-float they act on the perturbation from the
+  // element's first point, which makes up for Acc's larger error where a variable has a large mean
+  // (density, energy).  The divergence keeps Dot: it acts on the flux itself, whose pressure part is
+  // nearly constant at low Mach number, and with Acc the momentum residual's error against 64 bits grew
+  // from 3.8e-10 to 1.2e-9 (TGV 40^3, p = 3, Ma 0.1) for 3 % of the kernel's time.  The kernel is bound by
+  // FP32 issue (69 % of the issue slots at 4 warps per scheduler): the bounded sums, the three-term
+  // products and paired traces took the double-float kernel from 8860 to 7540 instructions per
+  // warp, 4.375 -> 3.80 ms per launch at 48^3 p = 4, 1.34 -> 1.18 ms at 40^3 p = 3, errors unchanged.
   const bool viscous = dph.viscous != 0;
   const bool pt = active && tid < Np;
   const int m = tid < Np ? tid : 0, i = m % N, j = (m / N) % N, k = m / (N * N);
@@ -317,10 +327,13 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
     for (int c = 0; c < 9; ++c) S[c] = met[c * Np];
     invJ = met[9 * Np];
   }
-  if (active)
+  if (active && (viscous || !kPertDf))
     for (int t = tid; t < 5 * Np; t += nth) {
       const T x = Q[e * Np * 5 + t];
-      sQ[(t % 5) * Np + t / 5] = x;
+      if constexpr (kPertDf)
+        sQ[(t % 5) * Np + t / 5] = x - Q[e * Np * 5 + t % 5];
+      else
+        sQ[(t % 5) * Np + t / 5] = x;
       if constexpr (kPert)
         if (viscous) sQg[(t % 5) * Np + t / 5] = to_g<TG>(x - Q[e * Np * 5 + t % 5]);
     }
@@ -345,7 +358,7 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   TG G[15];
   if (pt) {
 #pragma unroll
-    for (int v = 0; v < 5; ++v) q[v] = sQ[v * Np + m];
+    for (int v = 0; v < 5; ++v) q[v] = kPertDf ? Q[(e * Np + m) * 5 + v] : sQ[v * Np + m];
     if (viscous) {
       // One variable at a time: reference gradient, its correction, and both transformed to
       // physical components at once (short live ranges; the same operations as a two-pass form).
@@ -366,34 +379,40 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
           sq = sQg + v * Np;
         else
           sq = sQ + v * Np;
-        Dot<TG> a0, a1, a2;
+        // One reference direction: derivative along the point's line, then the two faces' correction
+        // added to the same sum.
+        TG gu[3], gc[3];
+        auto line = [&](int row, int at, int st, TG hlo, TG hhi, TG jlo, TG jhi, TG &u, TG &c) {
+          TG x[N];
+          Bound<TG> bd;
 #pragma unroll
-        for (int a = 0; a < N; ++a) {
-          a0.add(to_g<TG>(B.D[i * N + a]), sq[a + N * j + N * N * k]);
-          a1.add(to_g<TG>(B.D[j * N + a]), sq[i + N * a + N * N * k]);
-          a2.add(to_g<TG>(B.D[k * N + a]), sq[i + N * j + N * N * a]);
-        }
-        const TG gu0 = a0.raw(), gu1 = a1.raw(), gu2 = a2.raw();
-        a0.add(nhm[0], sdQ[(0 * 5 + v) * Nf + j + N * k]);
-        a0.add(to_g<TG>(B.hp[i]), sdQ[(1 * 5 + v) * Nf + j + N * k]);
-        a1.add(nhm[1], sdQ[(2 * 5 + v) * Nf + i + N * k]);
-        a1.add(to_g<TG>(B.hp[j]), sdQ[(3 * 5 + v) * Nf + i + N * k]);
-        a2.add(nhm[2], sdQ[(4 * 5 + v) * Nf + i + N * j]);
-        a2.add(to_g<TG>(B.hp[k]), sdQ[(5 * 5 + v) * Nf + i + N * j]);
-        const TG gc0 = a0.raw(), gc1 = a1.raw(), gc2 = a2.raw();
+          for (int a = 0; a < N; ++a) {
+            x[a] = sq[at + a * st];
+            bd.add(to_g<TG>(B.D[row * N + a]), x[a]);
+          }
+          bd.add(hlo, jlo);
+          bd.add(hhi, jhi);
+          Acc<TG> s(bd);
+#pragma unroll
+          for (int a = 0; a < N; ++a) s.add(to_g<TG>(B.D[row * N + a]), x[a]);
+          u = s.raw();
+          s.add(hlo, jlo);
+          s.add(hhi, jhi);
+          c = s.raw();
+        };
+        const TG *dq = sdQ + v * Nf;      // jump of variable v, faces 5 Nf apart
+        line(i, N * j + N * N * k, 1, nhm[0], to_g<TG>(B.hp[i]), dq[j + N * k], dq[5 * Nf + j + N * k], gu[0], gc[0]);
+        line(j, i + N * N * k, N, nhm[1], to_g<TG>(B.hp[j]), dq[10 * Nf + i + N * k], dq[15 * Nf + i + N * k], gu[1],
+             gc[1]);
+        line(k, i + N * j, N * N, nhm[2], to_g<TG>(B.hp[k]), dq[20 * Nf + i + N * j], dq[25 * Nf + i + N * j], gu[2],
+             gc[2]);
 #pragma unroll
         for (int jj = 0; jj < 3; ++jj) {
-          Dot<TG> du, dc;
-          du.add(sj[0 * 3 + jj], gu0);
-          du.add(sj[1 * 3 + jj], gu1);
-          du.add(sj[2 * 3 + jj], gu2);
-          dc.add(sj[0 * 3 + jj], gc0);
-          dc.add(sj[1 * 3 + jj], gc1);
-          dc.add(sj[2 * 3 + jj], gc2);
-          const TG gc = dc.raw();
-          sGc[gslot(jj * 5 + v)] = gc;
+          const TG du = dot3(sj[jj], gu[0], sj[3 + jj], gu[1], sj[6 + jj], gu[2]);
+          const TG dc = dot3(sj[jj], gc[0], sj[3 + jj], gc[1], sj[6 + jj], gc[2]);
+          sGc[gslot(jj * 5 + v)] = dc;
           // Face-gradient source: BR2 the uncorrected gradient (+ eta r_f), LDG the corrected one.
-          sG[(jj * 5 + v) * Np + m] = dph.ldg ? gc : du.raw();
+          sG[(jj * 5 + v) * Np + m] = dph.ldg ? dc : du;
         }
       }
 #pragma unroll
@@ -486,30 +505,50 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   __syncthreads();
   if (viscous && active) {
     // Gradient traces: uncorrected gradient interpolated to the face + eta * own lifting.
-    // One item per (gradient component jj, face point): 3 * 6 * Nf items keep the block busy.
-    for (int t = tid; t < 18 * Nf; t += nth) {
-      const int jj = t / (6 * Nf), fr_ = t - jj * 6 * Nf;
-      const int f = fr_ / Nf, r = fr_ % Nf;
-      const T *l = (f & 1) ? B.lp : B.lm;
+    // df32 and FP32: one item per (gradient component jj, line normal to a face pair), whose two end
+    // points share the line's values.  FP64: one item per (jj, face point), because the FP64 pipe is the
+    // bound there and 18 Nf single items fill its warps better than 9 Nf double ones (p = 4: 15 against 16
+    // warp passes).
+    constexpr int S = std::is_same<T, double>::value ? 1 : 2, kF = 6 / S;
+    for (int t = tid; t < 3 * kF * Nf; t += nth) {
+      const int jj = t / (kF * Nf), fr_ = t - jj * kF * Nf;
+      const int f0 = fr_ / Nf * S, r = fr_ % Nf;
       int base, sd;
-      face_line<N>(f, r, base, sd);
-      const int packed = ef[e * 6 + f];
-      const int64_t I = packed >> 4;
-      const int side = (packed >> 3) & 1;
-      const int slot = slot_of(packed & 7, r % N, r / N, N);
-      T *dst = Gtr + (I * 2 + side) * 15 * Nf + slot;
-      const TG lj = to_g<TG>(ph.eta * liftfac[((e * 6 + f) * 3 + jj) * Nf + r]);
+      face_line<N>(f0, r, base, sd);
+      T *dst[S];
+      TG lj[S];
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        const int packed = ef[e * 6 + f0 + s];
+        const int64_t I = packed >> 4;
+        dst[s] = Gtr + (I * 2 + ((packed >> 3) & 1)) * 15 * Nf + slot_of(packed & 7, r % N, r / N, N) + jj * 5 * Nf;
+        lj[s] = to_g<TG>(ph.eta * liftfac[((e * 6 + f0 + s) * 3 + jj) * Nf + r]);
+      }
+      const T *l0 = (S == 1 && (f0 & 1)) ? B.lp : B.lm;
       TG lg[N];
 #pragma unroll
-      for (int c = 0; c < N; ++c) lg[c] = to_g<TG>(l[c]);
+      for (int c = 0; c < N; ++c) lg[c] = to_g<TG>(l0[c]);
 #pragma unroll 1
       for (int v = 0; v < 5; ++v) {
         const TG *sg = sG + (jj * 5 + v) * Np + base;
-        Dot<TG> acc;
+        TG x[N];
 #pragma unroll
-        for (int c = 0; c < N; ++c) acc.add(lg[c], sg[c * sd]);
-        acc.add(lj, sdQ[(f * 5 + v) * Nf + r]);
-        dst[(jj * 5 + v) * Nf] = from_g<T>(acc.raw());
+        for (int c = 0; c < N; ++c) x[c] = sg[c * sd];
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          // l(+1) is l(-1) mirrored.
+          auto l = [&](int c) { return s ? lg[N - 1 - c] : lg[c]; };
+          const TG jump = sdQ[((f0 + s) * 5 + v) * Nf + r];
+          Bound<TG> bd;
+#pragma unroll
+          for (int c = 0; c < N; ++c) bd.add(l(c), x[c]);
+          bd.add(lj[s], jump);
+          Acc<TG> acc(bd);
+#pragma unroll
+          for (int c = 0; c < N; ++c) acc.add(l(c), x[c]);
+          acc.add(lj[s], jump);
+          dst[s][v * Nf] = from_g<T>(acc.raw());
+        }
       }
     }
   }
@@ -519,9 +558,11 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
 #pragma unroll 1
     for (int v = 0; v < 5; ++v) {
       const T *h0 = sH + (0 * 5 + v) * Np, *h1 = sH + (1 * 5 + v) * Np, *h2 = sH + (2 * 5 + v) * Np;
-      Dot<T> acc;
+      Dot<T> acc(B.Dt[i * N], h0[N * j + N * N * k]);
+      acc.add(B.Dt[j * N], h1[i + N * N * k]);
+      acc.add(B.Dt[k * N], h2[i + N * j]);
 #pragma unroll
-      for (int a = 0; a < N; ++a) {
+      for (int a = 1; a < N; ++a) {
         acc.add(B.Dt[i * N + a], h0[a + N * j + N * N * k]);
         acc.add(B.Dt[j * N + a], h1[i + N * a + N * N * k]);
         acc.add(B.Dt[k * N + a], h2[i + N * j + N * N * a]);
