@@ -107,7 +107,9 @@ template <> struct Dot<double> {
   double s;
   __device__ __forceinline__ Dot() : s(0.0) {}
   __device__ __forceinline__ Dot(double c, double x) : s(c * x) {}
+  __device__ __forceinline__ explicit Dot(double x) : s(x) {}
   __device__ __forceinline__ void add(double c, double x) { s = fma(c, x, s); }
+  __device__ __forceinline__ void plus(double x) { s += x; }
   __device__ __forceinline__ double get() const { return s; }
   __device__ __forceinline__ double raw() const { return s; }
 };
@@ -116,7 +118,9 @@ template <> struct Dot<float> {
   float s;
   __device__ __forceinline__ Dot() : s(0.f) {}
   __device__ __forceinline__ Dot(float c, float x) : s(c * x) {}
+  __device__ __forceinline__ explicit Dot(float x) : s(x) {}
   __device__ __forceinline__ void add(float c, float x) { s = fmaf(c, x, s); }
+  __device__ __forceinline__ void plus(float x) { s += x; }
   __device__ __forceinline__ float get() const { return s; }
   __device__ __forceinline__ float raw() const { return s; }
 };
@@ -124,6 +128,7 @@ template <> struct Dot<float> {
 template <> struct Dot<df32> {
   float s, e;
   __device__ __forceinline__ Dot() : s(0.f), e(0.f) {}
+  __device__ __forceinline__ explicit Dot(df32 x) : s(x.hi), e(x.lo) {}
   // The first term by itself: 4 instructions instead of 12.
   __device__ __forceinline__ Dot(df32 c, df32 x) {
     s = __fmul_rn(c.hi, x.hi);
@@ -139,6 +144,11 @@ template <> struct Dot<df32> {
     const float r = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(p, bb));
     s = t;
     e = __fadd_rn(e, __fadd_rn(r, err));
+  }
+  __device__ __forceinline__ void plus(df32 x) {
+    const df32 t = two_sum(s, x.hi);
+    s = t.hi;
+    e = __fadd_rn(e, __fadd_rn(t.lo, x.lo));
   }
   __device__ __forceinline__ df32 get() const {
     const df32 r = two_sum(s, e);
@@ -204,6 +214,21 @@ __device__ __forceinline__ df32 dot3(df32 a0, df32 b0, df32 a1, df32 b1, df32 a2
   const df32 s = two_sum(p0, p1), t = two_sum(s.hi, p2);
   return fast_two_sum(t.hi, __fadd_rn(__fadd_rn(__fadd_rn(e0, e1), __fadd_rn(e2, s.lo)), t.lo));
 }
+
+// c + a b (df32: 15 FP32 instructions, against 18 for the product and the sum by themselves).
+__device__ __forceinline__ double muladd(double c, double a, double b) { return fma(a, b, c); }
+__device__ __forceinline__ float muladd(float c, float a, float b) { return fmaf(a, b, c); }
+__device__ __forceinline__ df32 muladd(df32 c, df32 a, df32 b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  const float e = __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.hi, b.hi, -p)));
+  const df32 s = two_sum(c.hi, p);
+  return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(c.lo, e)));
+}
+
+// x times a power of two (exact).
+__device__ __forceinline__ double scale2(double x, float f) { return x * (double)f; }
+__device__ __forceinline__ float scale2(float x, float f) { return x * f; }
+__device__ __forceinline__ df32 scale2(df32 x, float f) { return df(__fmul_rn(x.hi, f), __fmul_rn(x.lo, f)); }
 
 __device__ __forceinline__ df32 fabs(df32 x) { return x.hi < 0.f ? -x : x; }
 __device__ __forceinline__ bool operator<(df32 x, df32 y) { return x.hi < y.hi || (x.hi == y.hi && x.lo < y.lo); }

@@ -348,10 +348,10 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
       const T *oth = Qtr + (I * 2 + (1 - side)) * 5 * Nf + slot;
       // Q^I - Q_own.  BR2: (other - own)/2 (a boundary's other slot holds 2 Q^I - Q-).  LDG: 0 on
       // the side that supplies Q^I, other - own on the other; boundaries as BR2.
-      T w = ph.half;
-      if (dph.ldg && I < n_interior) w = side == (if_up[I] ? 0 : 1) ? ph.zero : ph.one;
+      float w = 0.5f;
+      if (dph.ldg && I < n_interior) w = side == (if_up[I] ? 0 : 1) ? 0.f : 1.f;
 #pragma unroll
-      for (int v = 0; v < 5; ++v) sdQ[(f * 5 + v) * Nf + r] = to_g<TG>(w * (oth[v * Nf] - own[v * Nf]));
+      for (int v = 0; v < 5; ++v) sdQ[(f * 5 + v) * Nf + r] = to_g<TG>(scale2(oth[v * Nf] - own[v * Nf], w));
     }
   }
   __syncthreads();
@@ -470,14 +470,14 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
     if (pt) rho_nu = q[0] * from_double<T>((double)red[10 * Np]);
   }
   if (pt) {
-    // Transformed fluxes per reference direction from the contravariant velocity.
+    // Physical flux (symmetric momentum tensor and energy vector), then its three transforms.
     const T ri = ph.one / q[0];
     const T u[3] = {q[1] * ri, q[2] * ri, q[3] * ri};
-    const T p = ph.gm1 * (q[4] - ph.half * (q[1] * u[0] + q[2] * u[1] + q[3] * u[2]));
-    T tau[3][3], hq[3];
+    const T p = ph.gm1 * (q[4] - scale2(dot3(q[1], u[0], q[2], u[1], q[3], u[2]), 0.5f));
+    T tau[6], hq[3], mom[6], en[3];
     if (viscous) {
       if constexpr (kPert) {
-        TG qg[5], ug[3], taug[3][3], hqg[3];
+        TG qg[5], ug[3], taug[6], hqg[3];
 #pragma unroll
         for (int v = 0; v < 5; ++v) qg[v] = to_g<TG>(q[v]);
         const TG rig = phg.one / qg[0];
@@ -485,19 +485,18 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
         for (int c = 0; c < 3; ++c) ug[c] = qg[1 + c] * rig;
         viscous_stress<TG>(qg, ug, rig, G, phg, visc_with(phg, to_g<TG>(rho_nu), dph), taug, hqg);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          hq[a] = from_g<T>(hqg[a]);
+        for (int a = 0; a < 3; ++a) hq[a] = from_g<T>(hqg[a]);
 #pragma unroll
-          for (int b2 = 0; b2 < 3; ++b2) tau[a][b2] = from_g<T>(taug[a][b2]);
-        }
+        for (int a = 0; a < 6; ++a) tau[a] = from_g<T>(taug[a]);
       } else {
         viscous_stress<T>(q, u, ri, G, ph, visc_with(ph, rho_nu, dph), tau, hq);
       }
     }
+    physical_flux<T>(q, u, p, viscous, tau, hq, mom, en);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       T f[5];
-      contravariant_flux<T>(q, u, p, S + 3 * d, viscous, tau, hq, f);
+      transformed_flux<T>(q, mom, en, S + 3 * d, f);
 #pragma unroll
       for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
     }

@@ -143,10 +143,10 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
       const T *own = Qtr + (I * 2 + side) * 5 * Nf + slot;
       const T *oth = Qtr + (I * 2 + (1 - side)) * 5 * Nf + slot;
       // Q^I - Q_own: BR2 (other - own)/2; LDG 0 on the supplying side, other - own on the other.
-      T w = ph.half;
-      if (dph.ldg && I < n_interior) w = side == (if_up[I] ? 0 : 1) ? ph.zero : ph.one;
+      float w = 0.5f;
+      if (dph.ldg && I < n_interior) w = side == (if_up[I] ? 0 : 1) ? 0.f : 1.f;
 #pragma unroll
-      for (int v = 0; v < 5; ++v) sdQ[(f * 5 + v) * Nf + r] = w * (oth[v * Nf] - own[v * Nf]);
+      for (int v = 0; v < 5; ++v) sdQ[(f * 5 + v) * Nf + r] = scale2(oth[v * Nf] - own[v * Nf], w);
     }
   }
   __syncthreads();
@@ -230,16 +230,17 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
       }
     }
     {
-      // Transformed fluxes per reference direction from the contravariant velocity.
+      // Physical flux, then its three transforms.
       const T ri = ph.one / qv[0];
       const T u[3] = {qv[1] * ri, qv[2] * ri, qv[3] * ri};
-      const T p = ph.gm1 * (qv[4] - ph.half * (qv[1] * u[0] + qv[2] * u[1] + qv[3] * u[2]));
-      T tau[3][3], hq[3];
+      const T p = ph.gm1 * (qv[4] - scale2(dot3(qv[1], u[0], qv[2], u[1], qv[3], u[2]), 0.5f));
+      T tau[6], hq[3], mom[6], en[3];
       if (viscous) viscous_stress<T>(qv, u, ri, G, ph, visc_of(ph), tau, hq);
+      physical_flux<T>(qv, u, p, viscous, tau, hq, mom, en);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         T f[5];
-        contravariant_flux<T>(qv, u, p, S + 3 * d, viscous, tau, hq, f);
+        transformed_flux<T>(qv, mom, en, S + 3 * d, f);
 #pragma unroll
         for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
       }
