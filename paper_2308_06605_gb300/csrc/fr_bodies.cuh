@@ -471,7 +471,7 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   }
   if (pt) {
     // Physical flux (symmetric momentum tensor and energy vector), then its three transforms.
-    const T ri = ph.one / q[0];
+    const T ri = reciprocal(q[0]);
     const T u[3] = {q[1] * ri, q[2] * ri, q[3] * ri};
     const T p = ph.gm1 * (q[4] - scale2(dot3(q[1], u[0], q[2], u[1], q[3], u[2]), 0.5f));
     T tau[6], hq[3], mom[6], en[3];
@@ -480,7 +480,7 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
         TG qg[5], ug[3], taug[6], hqg[3];
 #pragma unroll
         for (int v = 0; v < 5; ++v) qg[v] = to_g<TG>(q[v]);
-        const TG rig = phg.one / qg[0];
+        const TG rig = reciprocal(qg[0]);
 #pragma unroll
         for (int c = 0; c < 3; ++c) ug[c] = qg[1 + c] * rig;
         viscous_stress<TG>(qg, ug, rig, G, phg, visc_with(phg, to_g<TG>(rho_nu), dph), taug, hqg);
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(volume_threads<N>(), volume_min_blocks_v<N, T,
 // 3. Common normal flux at the flux points of two-sided interfaces (Rusanov + BR2).  The
 // inviscid part (pressure/energy recovery) is FP64 in both paths.
 // ------------------------------------------------------------------------------------------
-template <int N, typename T, bool FP32V = false>
+template <int N, typename T, bool FP32V, bool ROE>
 __device__ __forceinline__ void iface_body(int64_t t, const T *__restrict__ Qtr, const T *__restrict__ Gtr,
                                            const T *__restrict__ normals, T *__restrict__ FI, int64_t n_if,
                                            const DevPhys &dph, const int32_t *__restrict__ if_elem,
@@ -623,7 +623,7 @@ __device__ __forceinline__ void iface_body(int64_t t, const T *__restrict__ Qtr,
 #pragma unroll
   for (int c = 0; c < 3; ++c) nT[c] = normals[(I * 4 + c) * Nf + q];
   T F[5];
-  if (dph.inviscid == FR_ROE) {
+  if constexpr (ROE) {
     double a[5], b[5], nd[3], Fd[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
@@ -639,81 +639,64 @@ __device__ __forceinline__ void iface_body(int64_t t, const T *__restrict__ Qtr,
     T fL[5], fR[5], sL, sR;
     normal_inviscid(qL, nT, nn, dph, fL, sL);
     normal_inviscid(qR, nT, nn, dph, fR, sR);
-    const T hl = ph.half * fmax(sL, sR);
+    const T ms = -fmax(sL, sR);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) F[v] = ph.half * (fL[v] + fR[v]) - hl * (qR[v] - qL[v]);
+    for (int v = 0; v < 5; ++v) F[v] = scale2(muladd(fL[v] + fR[v], ms, qR[v] - qL[v]), 0.5f);
   }
-  if constexpr (!std::is_same<typename GradOf<T, FP32V>::type, T>::value) {
-    if (dph.viscous) {
-      // FR_PREC_MIXED_VF32: the whole viscous part in FP32 (the gradient traces written by the
-      // volume kernel's FP32 branch are exact FP32 values).
-      using TG = typename GradOf<T, FP32V>::type;
-      const PhysT<TG> &phg = phys_of<TG>(dph);
-      TG qg[5], Gg[15], ng[3], Fv[3][5];
-      const int sup = (dph.ldg && if_up[I]) ? 0 : 1;
+  if (dph.viscous) {
+    // BR2: the mean state and gradient (their sums, see viscous_normal); LDG: the supplying side's
+    // solution and the other side's gradient.  FR_PREC_MIXED_VF32 forms the whole viscous part in FP32
+    // (the gradient traces written by the volume kernel's FP32 branch are exact FP32 values).
+    using TG = typename GradOf<T, FP32V>::type;
+    const PhysT<TG> &phg = phys_of<TG>(dph);
+    const int sup = (dph.ldg && if_up[I]) ? 0 : 1;
+    TG qc[5], ng[3], tn[3], en;
 #pragma unroll
-      for (int v = 0; v < 5; ++v)
-        qg[v] = dph.ldg ? to_g<TG>(sup == 0 ? qL[v] : qR[v]) : phg.half * (to_g<TG>(qL[v]) + to_g<TG>(qR[v]));
+    for (int v = 0; v < 5; ++v)
+      qc[v] = dph.ldg ? to_g<TG>(sup == 0 ? qL[v] : qR[v]) : to_g<TG>(qL[v]) + to_g<TG>(qR[v]);
 #pragma unroll
-      for (int c = 0; c < 15; ++c) {
-        const TG g0 = to_g<TG>(Gtr[(I * 2 + 0) * 15 * Nf + c * Nf + q]);
-        const TG g1 = to_g<TG>(Gtr[(I * 2 + 1) * 15 * Nf + c * Nf + q]);
-        Gg[c] = dph.ldg ? (sup == 0 ? g1 : g0) : phg.half * (g0 + g1);
-      }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) ng[c] = to_g<TG>(nT[c]);
-      TG rho_nu = phg.zero;
-      if (dph.closure) rho_nu = qg[0] * (TG)(0.5 * ((double)nu[if_elem[2 * I]] + (double)nu[if_elem[2 * I + 1]]));
-      viscous_flux<TG>(qg, Gg, phg, visc_with(phg, rho_nu, dph), Fv);
-#pragma unroll
-      for (int v = 0; v < 5; ++v) F[v] -= from_g<T>(Fv[0][v] * ng[0] + Fv[1][v] * ng[1] + Fv[2][v] * ng[2]);
-      if (dph.ldg) {
-        const T tn = ph.tau * nn;
-#pragma unroll
-        for (int v = 0; v < 5; ++v) F[v] += tn * (qL[v] - qR[v]);
-      }
-    }
-  } else if (dph.viscous) {
-    T qc[5], G[15];
+    for (int c = 0; c < 3; ++c) ng[c] = to_g<TG>(nT[c]);
+    TG rho_nu = phg.zero;
+    if (dph.closure)
+      rho_nu = scale2(qc[0], dph.ldg ? 1.f : 0.5f) *
+               from_double<TG>(0.5 * ((double)nu[if_elem[2 * I]] + (double)nu[if_elem[2 * I + 1]]));
+    const Visc<TG> vc = visc_with(phg, rho_nu, dph);
+    const T *g0 = Gtr + (I * 2 + 0) * 15 * Nf + q, *g1 = g0 + 15 * Nf;
     if (dph.ldg) {
-      // LDG: the supplying side's solution, the other side's gradient.
-      const int sup = if_up[I] ? 0 : 1;
-#pragma unroll
-      for (int v = 0; v < 5; ++v) qc[v] = sup == 0 ? qL[v] : qR[v];
-#pragma unroll
-      for (int c = 0; c < 15; ++c) G[c] = Gtr[(I * 2 + (1 - sup)) * 15 * Nf + c * Nf + q];
+      const T *gs = sup == 0 ? g1 : g0;
+      viscous_normal<TG>(qc, [&](int c) { return to_g<TG>(gs[c * Nf]); }, ng, phg, vc, tn, en);
     } else {
-#pragma unroll
-      for (int v = 0; v < 5; ++v) qc[v] = ph.half * (qL[v] + qR[v]);
-#pragma unroll
-      for (int c = 0; c < 15; ++c)
-        G[c] = ph.half * (Gtr[(I * 2 + 0) * 15 * Nf + c * Nf + q] + Gtr[(I * 2 + 1) * 15 * Nf + c * Nf + q]);
+      viscous_normal<TG>(qc, [&](int c) { return to_g<TG>(g0[c * Nf]) + to_g<TG>(g1[c * Nf]); }, ng, phg, vc, tn, en);
     }
-    T rho_nu = ph.zero;
-    if (dph.closure) rho_nu = qc[0] * from_double<T>(0.5 * ((double)nu[if_elem[2 * I]] + (double)nu[if_elem[2 * I + 1]]));
-    T Fv[3][5];
-    viscous_flux<T>(qc, G, ph, visc_with(ph, rho_nu, dph), Fv);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) F[v] -= Fv[0][v] * nT[0] + Fv[1][v] * nT[1] + Fv[2][v] * nT[2];
+    for (int v = 0; v < 3; ++v) F[1 + v] -= from_g<T>(tn[v]);
+    F[4] -= from_g<T>(en);
     if (dph.ldg) {
-      const T tn = ph.tau * nn;
+      const T tp = ph.tau * nn;
 #pragma unroll
-      for (int v = 0; v < 5; ++v) F[v] += tn * (qL[v] - qR[v]);
+      for (int v = 0; v < 5; ++v) F[v] = muladd(F[v], tp, qL[v] - qR[v]);
     }
   }
 #pragma unroll
   for (int v = 0; v < 5; ++v) FI[(I * 5 + v) * Nf + q] = F[v];
 }
 
-// 5 resident blocks of 128 threads (96 registers, a few spills): the double-float interface
-// kernel measured 4 % faster than with 128 registers and 4 blocks; the FP64 one is unchanged.
-template <int N, typename T, bool FP32V = false>
-__global__ void __launch_bounds__(128, 5) k_iface_flux(const T *__restrict__ Qtr, const T *__restrict__ Gtr,
+// 5 resident blocks of 128 threads (96 registers, no spills with the Rusanov flux; the Roe flux is an
+// instantiation of its own, which would otherwise set the registers of both), 6 with the FP32 viscous
+// part.  Measured at 5 / 6 blocks: double-float 48^3 p = 4 0.682 / 0.747 ms, FP64 32^3 p = 4 0.843 / 0.857
+// ms, FP32 viscous 40^3 p = 3 0.231 / 0.220 ms.  Before the viscous flux was formed along the normal and
+// the Roe branch split off: 0.869, 1.072 and 0.232 ms (memory floor 0.48 ms at 48^3; FP64 is bound by its
+// pipe: 185 operations per point instead of 240, Roe 330 instead of 500).
+template <bool FP32V>
+constexpr int iface_blocks() { return FP32V ? 6 : 5; }
+
+template <int N, typename T, bool FP32V, bool ROE>
+__global__ void __launch_bounds__(128, iface_blocks<FP32V>()) k_iface_flux(const T *__restrict__ Qtr, const T *__restrict__ Gtr,
                              const T *__restrict__ normals, T *__restrict__ FI, int64_t n_if, DevPhys dph,
                              const int32_t *__restrict__ if_elem, const float *__restrict__ nu,
                              const int8_t *__restrict__ if_up) {
-  iface_body<N, T, FP32V>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, Qtr, Gtr, normals, FI, n_if, dph, if_elem,
-                          nu, if_up);
+  iface_body<N, T, FP32V, ROE>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, Qtr, Gtr, normals, FI, n_if, dph,
+                               if_elem, nu, if_up);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -834,17 +817,16 @@ __device__ __forceinline__ void bc_flux_body(int64_t t, const T *__restrict__ Qt
   }
   if (dph.viscous) {
     const PhysT<T> &ph = phys_of<T>(dph);
-    T G[15], qiT[5];
-#pragma unroll
-    for (int c = 0; c < 15; ++c) G[c] = Gtr[(I * 2 + 0) * 15 * Nf + c * Nf + q];
+    T qiT[5], tn[3], en;
 #pragma unroll
     for (int v = 0; v < 5; ++v) qiT[v] = from_double<T>(qi[v]);
     T rho_nu = ph.zero;
     if (dph.closure) rho_nu = qiT[0] * from_double<T>((double)nu[if_elem[2 * I]]);
-    T Fv[3][5];
-    viscous_flux<T>(qiT, G, ph, visc_with(ph, rho_nu, dph), Fv);
+    const T *g0 = Gtr + (I * 2 + 0) * 15 * Nf + q;
+    viscous_normal<T>(qiT, [&](int c) { return g0[c * Nf]; }, nT, ph, visc_with(ph, rho_nu, dph), tn, en);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) F[v] -= Fv[0][v] * nT[0] + Fv[1][v] * nT[1] + Fv[2][v] * nT[2];
+    for (int v = 0; v < 3; ++v) F[1 + v] -= tn[v];
+    F[4] -= en;
     if (dph.ldg) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) F[v] += from_double<T>(dph.ldg_tau * nn * (qm[v] - qi[v]));
@@ -925,14 +907,14 @@ __device__ __forceinline__ bool unused_tri_slot(int64_t t, int64_t first, int64_
   return if_tri[first + t / Nf] && (int)(t % Nf) >= Nt;
 }
 
-template <int N, typename T>
-__global__ void k_iface_flux_tri(const T *__restrict__ Qtr, const T *__restrict__ Gtr, const T *__restrict__ normals,
+template <int N, typename T, bool ROE>
+__global__ void __launch_bounds__(128, iface_blocks<false>()) k_iface_flux_tri(const T *__restrict__ Qtr, const T *__restrict__ Gtr, const T *__restrict__ normals,
                                  T *__restrict__ FI, int64_t n_if, DevPhys dph, const int32_t *__restrict__ if_elem,
                                  const float *__restrict__ nu, const int8_t *__restrict__ if_tri,
                                  const int8_t *__restrict__ if_up) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (unused_tri_slot<N>(t, 0, n_if, if_tri)) return;
-  iface_body<N, T>(t, Qtr, Gtr, normals, FI, n_if, dph, if_elem, nu, if_up);
+  iface_body<N, T, false, ROE>(t, Qtr, Gtr, normals, FI, n_if, dph, if_elem, nu, if_up);
 }
 
 template <int N, typename T>
@@ -1023,7 +1005,10 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const BatchCase 
     }
     case TASK_IFACE:
       if (m.if_tri && unused_tri_slot<N>(idx, 0, m.n_interior, m.if_tri)) break;
-      iface_body<N, T>(idx, Qtr, Gtr, nrm, FI, m.n_interior, c.ph, m.if_elem, m.nu, m.if_up);
+      if (c.ph.inviscid == FR_ROE)
+        iface_body<N, T, false, true>(idx, Qtr, Gtr, nrm, FI, m.n_interior, c.ph, m.if_elem, m.nu, m.if_up);
+      else
+        iface_body<N, T, false, false>(idx, Qtr, Gtr, nrm, FI, m.n_interior, c.ph, m.if_elem, m.nu, m.if_up);
       break;
     case TASK_BC_FLUX:
       if (m.if_tri && unused_tri_slot<N>(idx, m.n_interior, m.n_if - m.n_interior, m.if_tri)) break;

@@ -114,15 +114,18 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
   if (phases & 4) {
     const int64_t n = m.n_interior * Nf;
     FR_EV_BEGIN(2);
+    const bool roe = ph.inviscid == FR_ROE;
     if (n > 0 && !tri) {
-      auto ik = k_iface_flux<N, T, false>;
+      auto ik = roe ? k_iface_flux<N, T, false, true> : k_iface_flux<N, T, false, false>;
       if constexpr (std::is_same<T, df32>::value)
-        if (m.vf32) ik = k_iface_flux<N, T, true>;
+        if (m.vf32) ik = roe ? k_iface_flux<N, T, true, true> : k_iface_flux<N, T, true, false>;
       ik<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(Qtr, Gtr, nrm, FI, m.n_interior, ph, m.if_elem, m.nu, m.if_up);
     }
-    if (n > 0 && tri)
-      k_iface_flux_tri<N, T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(Qtr, Gtr, nrm, FI, m.n_interior, ph,
-                                                                         m.if_elem, m.nu, m.if_tri, m.if_up);
+    if (n > 0 && tri) {
+      auto ik = roe ? k_iface_flux_tri<N, T, true> : k_iface_flux_tri<N, T, false>;
+      ik<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(Qtr, Gtr, nrm, FI, m.n_interior, ph, m.if_elem, m.nu, m.if_tri,
+                                                      m.if_up);
+    }
     const int64_t nb = (m.n_if - m.n_interior) * Nf;
     if (nb > 0 && !tri)
       k_bc_flux<N, T><<<(unsigned)((nb + 127) / 128), 128, 0, st>>>(Qtr, Gtr, nrm, m.if_bc, m.bcs, FI, m.n_interior,

@@ -40,24 +40,18 @@ __device__ __forceinline__ void normal_inviscid(const double q[5], const double 
 __device__ __forceinline__ void normal_inviscid(const df32 q[5], const df32 n[3], df32 nn, const DevPhys &dph,
                                                 df32 out[5], df32 &un_abs_plus_c_n) {
   const PhysT<df32> &ph = dph.f;
-  const df32 ri = ph.one / q[0];
+  const df32 ri = reciprocal(q[0]);
   const df32 u[3] = {q[1] * ri, q[2] * ri, q[3] * ri};
-  Dot<df32> mu, unn;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    mu.add(q[1 + c], u[c]);
-    unn.add(u[c], n[c]);
-  }
-  const double pd = (dph.gamma - 1.0) * (to_double(q[4]) - 0.5 * to_double(mu.get()));
+  const double pd = (dph.gamma - 1.0) *
+                    (to_double(q[4]) - 0.5 * to_double(dot3(q[1], u[0], q[2], u[1], q[3], u[2])));
   const df32 p = df_from(pd);
-  const df32 un = unn.get();
+  const df32 un = dot3(u[0], n[0], u[1], n[1], u[2], n[2]);
   out[0] = q[0] * un;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    Dot<df32> f;
-    f.add(q[1 + c], un);
+    Dot<df32> f(q[1 + c], un);
     f.add(p, n[c]);
-    out[1 + c] = f.get();
+    out[1 + c] = f.raw();
   }
   out[4] = (q[4] + p) * un;
   un_abs_plus_c_n = fabs(un) + sqrt(ph.gamma * p * ri) * nn;
@@ -77,50 +71,53 @@ __device__ __forceinline__ void normal_inviscid(const double q[5], const double 
 // d = 0.1 c becomes (lambda^2 + d^2) / (2 d).
 __device__ __forceinline__ void roe_flux(const double qL[5], const double qR[5], const double n[3], double nn,
                                          double g, double F[5]) {
-  double fL[5], fR[5], sL, sR;
-  normal_inviscid(qL, n, nn, g, fL, sL);
-  normal_inviscid(qR, n, nn, g, fR, sR);
-  const double inn = 1.0 / nn;
+  // Five reciprocals and three square roots: on this FP64 pipe a division costs about ten additions.
+  const double inn = 1.0 / nn, iL = 1.0 / qL[0], iR = 1.0 / qR[0];
   const double nh[3] = {n[0] * inn, n[1] * inn, n[2] * inn};
   const double rL = qL[0], rR = qR[0];
-  const double uL[3] = {qL[1] / rL, qL[2] / rL, qL[3] / rL}, uR[3] = {qR[1] / rR, qR[2] / rR, qR[3] / rR};
+  const double uL[3] = {qL[1] * iL, qL[2] * iL, qL[3] * iL}, uR[3] = {qR[1] * iR, qR[2] * iR, qR[3] * iR};
   const double pL = (g - 1.0) * (qL[4] - 0.5 * (qL[1] * uL[0] + qL[2] * uL[1] + qL[3] * uL[2]));
   const double pR = (g - 1.0) * (qR[4] - 0.5 * (qR[1] * uR[0] + qR[2] * uR[1] + qR[3] * uR[2]));
-  const double HL = (qL[4] + pL) / rL, HR = (qR[4] + pR) / rR;
+  const double eL = qL[4] + pL, eR = qR[4] + pR;
   const double sl = sqrt(rL), sr = sqrt(rR), w = 1.0 / (sl + sr);
-  const double r = sl * sr;
-  double u[3], du[3], q2 = 0.0, un = 0.0, dun = 0.0;
+  const double r = sl * sr, wl = sl * w, wr = sr * w;
+  double u[3], du[3], q2 = 0.0, un = 0.0, dun = 0.0, nL = 0.0, nR = 0.0;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    u[c] = (sl * uL[c] + sr * uR[c]) * w;
+    u[c] = wl * uL[c] + wr * uR[c];
     du[c] = uR[c] - uL[c];
     q2 += u[c] * u[c];
     un += u[c] * nh[c];
     dun += du[c] * nh[c];
+    nL += uL[c] * n[c];
+    nR += uR[c] * n[c];
   }
-  const double H = (sl * HL + sr * HR) * w;
-  const double c2 = (g - 1.0) * (H - 0.5 * q2), c = sqrt(c2);
-  const double dp = pR - pL, dr = rR - rL;
-  const double a1 = (dp - r * c * dun) / (2.0 * c2), a2 = dr - dp / c2, a3 = (dp + r * c * dun) / (2.0 * c2);
-  const double d = 0.1 * c;
-  auto fix = [d](double lam) {
+  const double H = wl * (eL * iL) + wr * (eR * iR);
+  const double c2 = (g - 1.0) * (H - 0.5 * q2), c = sqrt(c2), ic2 = 1.0 / c2;
+  const double dp = pR - pL, dr = rR - rL, rcd = r * c * dun, h2 = 0.5 * ic2;
+  const double a1 = (dp - rcd) * h2, a2 = dr - dp * ic2, a3 = (dp + rcd) * h2;
+  // Harten's fix with d = 0.1 c: (lam^2 + d^2) / (2 d), 1 / (2 d) = 5 / c = 5 c / c^2.
+  const double d = 0.1 * c, i2d = 5.0 * c * ic2;
+  auto fix = [d, i2d](double lam) {
     const double a = fabs(lam);
-    return a < d ? (lam * lam + d * d) / (2.0 * d) : a;
+    return a < d ? (lam * lam + d * d) * i2d : a;
   };
   const double l1 = fix(un - c) * a1, l2 = fabs(un), l3 = fix(un + c) * a3;
-  double sh[3], ush = 0.0;
+  const double la = l1 + l3, lc = (l3 - l1) * c, m2 = l2 * a2, mr = l2 * r;
+  double D[5], ush = 0.0;
+  D[0] = la + m2;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    sh[k] = r * (du[k] - dun * nh[k]);
-    ush += u[k] * sh[k];
+    const double sh = du[k] - dun * nh[k];     // shear, times r
+    ush += u[k] * sh;
+    D[1 + k] = D[0] * u[k] + lc * nh[k] + mr * sh;
   }
-  double D[5];
-  D[0] = l1 + l2 * a2 + l3;
+  D[4] = la * H + lc * un + m2 * 0.5 * q2 + mr * ush;
+  const double ps = pL + pR;
+  F[0] = 0.5 * (rL * nL + rR * nR - nn * D[0]);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) D[1 + k] = l1 * (u[k] - c * nh[k]) + l3 * (u[k] + c * nh[k]) + l2 * (a2 * u[k] + sh[k]);
-  D[4] = l1 * (H - c * un) + l3 * (H + c * un) + l2 * (a2 * 0.5 * q2 + ush);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) F[v] = 0.5 * (fL[v] + fR[v]) - 0.5 * nn * D[v];
+  for (int k = 0; k < 3; ++k) F[1 + k] = 0.5 * (qL[1 + k] * nL + qR[1 + k] * nR + ps * n[k] - nn * D[1 + k]);
+  F[4] = 0.5 * (eL * nL + eR * nR - nn * D[4]);
 }
 
 // Transport coefficients of one viscous-flux evaluation (molecular, or with an eddy viscosity).
@@ -142,42 +139,54 @@ __device__ __forceinline__ Visc<T> visc_with(const PhysT<T> &ph, T rho_nu, const
   return Visc<T>{mu, ph.m2mu3 + from_double<T>(-2.0 / 3.0) * rho_nu, ph.kappa + from_double<T>(dph.cp_prt) * rho_nu};
 }
 
-// Viscous flux F_v[j][v] (j = direction) of state q with gradient G[j*5 + v] = dQ_v/dx_j.
-template <typename T>
-__device__ __forceinline__ void viscous_flux(const T q[5], const T *G, const PhysT<T> &ph, const Visc<T> &vc,
-                                             T Fv[3][5]) {
-  const T ri = ph.one / q[0];
+// Viscous flux through the normal n: tn = tau . n and en = u . tn + kappa dT/dn, of the state q and
+// gradient g(j * 5 + v) = dQ_v/dx_j.  Both enter through their ratio only (and u, E/rho), so a pair of
+// sides passes the sums of its states and gradients, and no factor 1/2 is spent on the mean.  The
+// columns of the gradient are read one at a time (five values live) and the 3 x 3 stress is never
+// formed: 80 FP64 operations with the sums, where the full flux and its projection take 190.
+template <typename T, typename GetG>
+__device__ __forceinline__ void viscous_normal(const T q[5], GetG g, const T n[3], const PhysT<T> &ph,
+                                               const Visc<T> &vc, T tn[3], T &en) {
+  const T ri = reciprocal(q[0]);
   const T u[3] = {q[1] * ri, q[2] * ri, q[3] * ri};
   const T eo = q[4] * ri;
-  T du[3][3];   // du[i][j] = du_i/dx_j
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) du[i][j] = (G[j * 5 + 1 + i] - u[i] * G[j * 5]) * ri;
-  T dT[3];
-#pragma unroll
-  for (int j = 0; j < 3; ++j)
-    dT[j] = ph.cT * ((G[j * 5 + 4] - eo * G[j * 5]) * ri - (u[0] * du[0][j] + u[1] * du[1][j] + u[2] * du[2][j]));
-  const T lam = vc.m2mu3 * (du[0][0] + du[1][1] + du[2][2]);
+  T z[3], div;        // z[j] = sum_i n_i rho du_i/dx_j
+  Dot<T> w[3], h;     // w[i] = sum_j n_j rho du_i/dx_j, h = sum_j n_j (dE/dx_j - E/rho drho/dx_j)
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    T t[3];
+    const T g0 = g(j * 5);
+    T a[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) a[i] = muladd(g(j * 5 + 1 + i), -u[i], g0);
+    z[j] = dot3(n[0], a[0], n[1], a[1], n[2], a[2]);
+    const T e = muladd(g(j * 5 + 4), -eo, g0);
+    if (j == 0) {
+      div = a[0];
+      h = Dot<T>(n[0], e);
+    } else {
+      div = div + a[j];
+      h.add(n[j], e);
+    }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      t[i] = vc.mu * (du[i][j] + du[j][i]);
-      if (i == j) t[i] = t[i] + lam;
+      if (j == 0)
+        w[i] = Dot<T>(n[0], a[i]);
+      else
+        w[i].add(n[j], a[i]);
     }
-    Fv[j][0] = ph.zero;
-    Fv[j][1] = t[0];
-    Fv[j][2] = t[1];
-    Fv[j][3] = t[2];
-    Fv[j][4] = u[0] * t[0] + u[1] * t[1] + u[2] * t[2] + vc.kappa * dT[j];
   }
+  const T t = vc.mu * ri, ld = vc.m2mu3 * ri * div;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const T wi = w[i].raw();
+    h.add(-u[i], wi);
+    tn[i] = muladd(t * (wi + z[i]), ld, n[i]);
+  }
+  en = muladd(dot3(u[0], tn[0], u[1], tn[1], u[2], tn[2]), vc.kappa * (ph.cT * ri), h.raw());
 }
 
 // Viscous stress tau = mu (du_i/dx_j + du_j/dx_i) + delta_ij lambda div u, packed (xx, yy, zz, xy,
-// xz, yz), and heat-flux term hq[j] = kappa dT/dx_j of state q with gradient G[j*5 + v] = dQ_v/dx_j (the
-// entries of viscous_flux).  Works on rho du_i/dx_j = G[j][1+i] - u_i G[j][0] and puts the factor 1/rho
+// xz, yz), and heat-flux term hq[j] = kappa dT/dx_j of state q with gradient G[j*5 + v] = dQ_v/dx_j.  Works on rho du_i/dx_j = G[j][1+i] - u_i G[j][0] and puts the factor 1/rho
 // into the coefficients: 40 FP64 operations, 450 FP32 instructions in double-float (57 and 700 with
 // du_i/dx_j itself).
 template <typename T>

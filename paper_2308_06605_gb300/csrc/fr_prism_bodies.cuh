@@ -231,7 +231,7 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
     }
     {
       // Physical flux, then its three transforms.
-      const T ri = ph.one / qv[0];
+      const T ri = reciprocal(qv[0]);
       const T u[3] = {qv[1] * ri, qv[2] * ri, qv[3] * ri};
       const T p = ph.gm1 * (qv[4] - scale2(dot3(qv[1], u[0], qv[2], u[1], qv[3], u[2]), 0.5f));
       T tau[6], hq[3], mom[6], en[3];
