@@ -360,52 +360,65 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
 #pragma unroll
     for (int v = 0; v < 5; ++v) q[v] = kPertDf ? Q[(e * Np + m) * 5 + v] : sQ[v * Np + m];
     if (viscous) {
-      // One variable at a time: reference gradient, its correction, and both transformed to
-      // physical components at once (short live ranges; the same operations as a two-pass form).
       TG sj[9];   // S[d][jj] / |J|
 #pragma unroll
       for (int c = 0; c < 9; ++c) sj[c] = to_g<TG>(S[c] * invJ);
-      const TG nhm[3] = {-to_g<TG>(B.hm[i]), -to_g<TG>(B.hm[j]), -to_g<TG>(B.hm[k])};
-      // The variable loop stays rolled (a smaller instruction footprint): the corrected gradient
-      // goes through shared memory, in this thread's own entries of the transformed-flux buffer,
-      // which only this thread writes later (R gradient values of type TG per entry of type T).
+      // The reference gradient, uncorrected and corrected, goes through shared memory, in this thread's
+      // own entries of the gradient and transformed-flux buffers, which only this thread writes before
+      // the next barrier (R gradient values of type TG per entry of type T).
       constexpr int R = sizeof(T) / sizeof(TG);
       TG *sGc = reinterpret_cast<TG *>(sH);
       auto gslot = [&](int c) { return ((c / R) * Np + m) * R + c % R; };
+      const TG *sq;
+      if constexpr (kPert)
+        sq = sQg;
+      else
+        sq = sQ;
+      // One reference direction at a time: its row of D (indexed by the lane's own i, j or k, so every
+      // read of it from constant memory is a divergent one) is loaded once for the five variables.  With the
+      // variables outside, the three rows were re-read for each of them (address-divergence unit 37 %
+      // busy): double-float 48^3 p = 4 3.43 -> 3.27 ms per launch, 20^3 p = 7 1.56 -> 1.25 ms, 28^3 p = 5 1.30 ->
+      // 1.17 ms; FP64 unchanged.  At p = 7 the five variables are unrolled (one block per SM: more loads in
+      // flight; 1.270 -> 1.248 ms), below they stay rolled.
 #pragma unroll 1
-      for (int v = 0; v < 5; ++v) {
-        const TG *sq;
-        if constexpr (kPert)
-          sq = sQg + v * Np;
-        else
-          sq = sQ + v * Np;
-        // One reference direction: derivative along the point's line, then the two faces' correction
-        // added to the same sum.
-        TG gu[3], gc[3];
-        auto line = [&](int row, int at, int st, TG hlo, TG hhi, TG jlo, TG jhi, TG &u, TG &c) {
+      for (int d = 0; d < 3; ++d) {
+        const int row = d == 0 ? i : (d == 1 ? j : k), st = axis_stride<N>(d), at = m - row * st;
+        const int r = d == 0 ? j + N * k : (d == 1 ? i + N * k : i + N * j);
+        TG c[N];
+#pragma unroll
+        for (int a = 0; a < N; ++a) c[a] = to_g<TG>(B.D[row * N + a]);
+        const TG hlo = -to_g<TG>(B.hm[row]), hhi = to_g<TG>(B.hp[row]);
+        const TG *dq = sdQ + d * 10 * Nf + r;
+#pragma unroll(N == 8 ? 5 : 1)
+        for (int v = 0; v < 5; ++v) {
+          // Derivative along the point's line, then the two faces' correction added to the same sum.
+          const TG jlo = dq[v * Nf], jhi = dq[(5 + v) * Nf];
           TG x[N];
           Bound<TG> bd;
 #pragma unroll
           for (int a = 0; a < N; ++a) {
-            x[a] = sq[at + a * st];
-            bd.add(to_g<TG>(B.D[row * N + a]), x[a]);
+            x[a] = sq[v * Np + at + a * st];
+            bd.add(c[a], x[a]);
           }
           bd.add(hlo, jlo);
           bd.add(hhi, jhi);
           Acc<TG> s(bd);
 #pragma unroll
-          for (int a = 0; a < N; ++a) s.add(to_g<TG>(B.D[row * N + a]), x[a]);
-          u = s.raw();
+          for (int a = 0; a < N; ++a) s.add(c[a], x[a]);
+          sG[(d * 5 + v) * Np + m] = s.raw();
           s.add(hlo, jlo);
           s.add(hhi, jhi);
-          c = s.raw();
-        };
-        const TG *dq = sdQ + v * Nf;      // jump of variable v, faces 5 Nf apart
-        line(i, N * j + N * N * k, 1, nhm[0], to_g<TG>(B.hp[i]), dq[j + N * k], dq[5 * Nf + j + N * k], gu[0], gc[0]);
-        line(j, i + N * N * k, N, nhm[1], to_g<TG>(B.hp[j]), dq[10 * Nf + i + N * k], dq[15 * Nf + i + N * k], gu[1],
-             gc[1]);
-        line(k, i + N * j, N * N, nhm[2], to_g<TG>(B.hp[k]), dq[20 * Nf + i + N * j], dq[25 * Nf + i + N * j], gu[2],
-             gc[2]);
+          sGc[gslot(d * 5 + v)] = s.raw();
+        }
+      }
+#pragma unroll 1
+      for (int v = 0; v < 5; ++v) {
+        TG gu[3], gc[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          gu[d] = sG[(d * 5 + v) * Np + m];
+          gc[d] = sGc[gslot(d * 5 + v)];
+        }
 #pragma unroll
         for (int jj = 0; jj < 3; ++jj) {
           const TG du = dot3(sj[jj], gu[0], sj[3 + jj], gu[1], sj[6 + jj], gu[2]);
@@ -571,25 +584,20 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   }
 }
 
-// Resident blocks at p = 5 and 6: 3 blocks of 224 and (double-float) 2 of 352 threads at 80
-// registers, with some spills, measured faster than the register-limited 2 and 1 (double-float
-// p = 6: 9.16 -> 7.73 ms per launch at 40^3; p = 5: 8.80 -> 8.61 ms at 48^3; FP64 p = 5: 25.63 ->
-// 25.26 ms; FP64 p = 6 unchanged at 2 blocks, so it keeps 1).
+// Resident blocks per order and arithmetic, each measured (GB300).  p = 5 and 6: 3 blocks of 224 and
+// (double-float) 2 of 352 threads at 80 registers, with some spills, beat the register-limited 2 and
+// 1; FP64 p = 6 keeps 1 block.  Double-float at p = 2, 3, 4: 20, 10 and 5 blocks (96 registers, no
+// spills) beat 16, 8 and 4, since the gradient holds one row of D instead of three: 40^3 p = 2 0.485 -> 0.463
+// ms per launch, 40^3 p = 3 1.023 -> 0.985 ms, 48^3 p = 4 3.27 -> 3.09 ms.  With the viscous branch in FP32 the
+// same counts (6 and 12 at p = 4 and 3 measure the same).
 template <int N, typename T>
 constexpr int volume_min_blocks_of() {
-  return N == 6 ? 3 : ((N == 7 && !std::is_same<T, double>::value) ? 2 : volume_min_blocks<N>());
-}
-
-// With the viscous branch in FP32 (96 registers, no spills) the kernels of p = 3 and 4 fit 10 and
-// 5 blocks per SM, which hides more of their load latency (p = 4: 6.44 -> 5.96 ms per launch at
-// 64^3; p = 3: 3.27 -> 3.00 ms); the double-float ones measured slower at those counts.
-template <int N, typename T, bool FP32V>
-constexpr int volume_min_blocks_v() {
-  return (FP32V && N == 5) ? 5 : ((FP32V && N == 4) ? 10 : volume_min_blocks_of<N, T>());
+  if (std::is_same<T, double>::value) return N == 6 ? 3 : volume_min_blocks<N>();
+  return N == 3 ? 20 : (N == 4 ? 10 : (N == 5 ? 5 : (N == 6 ? 3 : (N == 7 ? 2 : volume_min_blocks<N>()))));
 }
 
 template <int N, typename T, bool FP32V = false>
-__global__ void __launch_bounds__(volume_threads<N>(), volume_min_blocks_v<N, T, FP32V>())
+__global__ void __launch_bounds__(volume_threads<N>(), volume_min_blocks_of<N, T>())
     k_volume(const T *__restrict__ Q, const T *__restrict__ metrics, const int32_t *__restrict__ ef,
              const T *__restrict__ Qtr, const T *__restrict__ liftfac, T *__restrict__ Gtr, T *__restrict__ Rpart,
              DevPhys dph, const double *__restrict__ hel, float *__restrict__ nu_out,
