@@ -856,22 +856,17 @@ __global__ void k_bc_flux(const T *__restrict__ Qtr, const T *__restrict__ Gtr, 
 // ------------------------------------------------------------------------------------------
 // 4. Correction by the common flux, scaling, and output / RK44 stage update (FP64).
 // ------------------------------------------------------------------------------------------
-template <int N, typename T, bool VC = false>
-__device__ __forceinline__ void correct_body(int64_t t, const T *__restrict__ Rpart, const T *__restrict__ FI,
-                                             const int32_t *__restrict__ ef, const T *__restrict__ metrics,
-                                             int64_t E, int mode, int stage, double dt, double *__restrict__ Rout,
-                                             double *__restrict__ Q, T *__restrict__ Qc, double *__restrict__ Un,
-                                             T *__restrict__ Unc, double *__restrict__ acc, int *__restrict__ flag,
-                                             const DevPhys &dph) {
-  constexpr int Np = N * N * N, Nf = N * N;
-  if (t >= E * Np) return;
-  const int64_t e = t / Np;
-  const int m = (int)(t % Np), i = m % N, j = (m / N) % N, k = m / (N * N);
+// Bracket of Eq. 3 at point m of element e: the partial residual rp (5 values) plus the lifted common
+// fluxes of the six faces.
+template <int N, typename T, bool VC>
+__device__ __forceinline__ void correct_bracket(int64_t e, int m, const T *rp, const T *__restrict__ FI,
+                                                const int32_t *__restrict__ ef, const DevPhys &dph, T rv[5]) {
+  constexpr int Nf = N * N;
+  const int i = m % N, j = (m / N) % N, k = m / (N * N);
   const BasisT<T> &B = basis_ref<N, T, VC>(dph);
-  const PhysT<T> &ph = phys_of<T>(dph);
   Dot<T> r[5];
 #pragma unroll
-  for (int v = 0; v < 5; ++v) r[v].add(ph.one, Rpart[t * 5 + v]);
+  for (int v = 0; v < 5; ++v) r[v] = Dot<T>(rp[v]);
   // Faces: (weight, local flux point (a, b)).
   const int fa[6] = {j, j, i, i, i, i};
   const int fb[6] = {k, k, k, k, j, j};
@@ -887,23 +882,48 @@ __device__ __forceinline__ void correct_body(int64_t t, const T *__restrict__ Rp
 #pragma unroll
     for (int v = 0; v < 5; ++v) r[v].add(w, src[v * Nf]);
   }
-  const T s = -metrics[(e * 10 + 9) * Np + m];
-  T rv[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) rv[v] = r[v].get();
-  finish_point<T>(t, rv, s, mode, stage, dt, Rout, Q, Qc, Un, Unc, acc, flag, dph);
 }
 
-// 6 resident blocks (40 registers): the double-float kernel measured 2.62 -> 2.55 ms per launch at
-// 64^3, p = 4 (its FP64 RK update and its loads overlap better across more warps); FP64 unchanged.
+// Thread per point (batched stage).
 template <int N, typename T>
-__global__ void __launch_bounds__(256, 6) k_correct(const T *__restrict__ Rpart, const T *__restrict__ FI, const int32_t *__restrict__ ef,
-                          const T *__restrict__ metrics, int64_t E, int mode, int stage, double dt,
-                          double *__restrict__ Rout, double *__restrict__ Q, T *__restrict__ Qc,
+__device__ __forceinline__ void correct_body(int64_t t, const T *__restrict__ Rpart, const T *__restrict__ FI,
+                                             const int32_t *__restrict__ ef, const T *__restrict__ metrics,
+                                             int64_t E, const StageCoef &sc, double *__restrict__ Rout,
+                                             double *__restrict__ Q, T *__restrict__ Qc, double *__restrict__ Un,
+                                             T *__restrict__ Unc, double *__restrict__ acc, int *__restrict__ flag,
+                                             const DevPhys &dph) {
+  constexpr int Np = N * N * N;
+  if (t >= E * Np) return;
+  const int64_t e = t / Np;
+  const int m = (int)(t % Np);
+  T rv[5];
+  correct_bracket<N, T, false>(e, m, Rpart + t * 5, FI, ef, dph, rv);
+  finish_point<T>(t, rv, -metrics[(e * 10 + 9) * Np + m], sc, Rout, Q, Qc, Un, Unc, acc, flag, dph);
+}
+
+template <int N, typename T, bool VC, bool SRC>
+__global__ void __launch_bounds__(kCorrectThreads, 6) k_correct(const T *__restrict__ Rpart, const T *__restrict__ FI,
+                          const int32_t *__restrict__ ef, const T *__restrict__ metrics, int64_t E,
+                          StageCoef sc, double *__restrict__ Rout, double *__restrict__ Q, T *__restrict__ Qc,
                           double *__restrict__ Un, T *__restrict__ Unc, double *__restrict__ acc,
                           int *__restrict__ flag, DevPhys dph) {
-  correct_body<N, T>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, Rpart, FI, ef, metrics, E, mode, stage, dt, Rout,
-                     Q, Qc, Un, Unc, acc, flag, dph);
+  extern __shared__ double sm_raw[];
+  constexpr int Np = N * N * N;
+  T *sr = reinterpret_cast<T *>(sm_raw);
+  const int64_t first = (int64_t)blockIdx.x * kCorrectThreads;
+  const int n = (int)(E * Np - first < kCorrectThreads ? E * Np - first : kCorrectThreads);
+  stage_partial<T>(sr, Rpart, first, n);
+  T rv[5], s{};
+  if ((int)threadIdx.x < n) {
+    const int64_t t = first + threadIdx.x, e = t / Np;
+    const int m = (int)(t % Np);
+    correct_bracket<N, T, VC>(e, m, sr + threadIdx.x * 5, FI, ef, dph, rv);
+    s = -metrics[(e * 10 + 9) * Np + m];
+  }
+  finish_block<T, SRC>(first, n, sr, sm_raw + 5 * kCorrectThreads, rv, s, sc, Rout, Q, Qc, Un, Unc, acc, flag,
+                  dph);
 }
 
 // Meshes with prisms: a triangular interface uses only the first N(N+1)/2 of its N^2 slots;
@@ -1040,13 +1060,13 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const BatchCase 
       break;
     }
     case TASK_PRISM_CORRECT:
-      prism_correct_body<N, T>(idx, Rpart + pts, FI, m.ef_p, pmet, ptab, m.tri_slot, m.Ep, m.E * m.Np, MODE_RK, L.stage,
-                               L.dts[tk.cs], nullptr, m.Q, m.mixed ? reinterpret_cast<T *>(m.Qc) : nullptr, m.Un,
+      prism_correct_body<N, T>(idx, Rpart + pts, FI, m.ef_p, pmet, ptab, m.tri_slot, m.Ep, m.E * m.Np,
+                               stage_coef(MODE_RK, L.stage, L.dts[tk.cs]), nullptr, m.Q, m.mixed ? reinterpret_cast<T *>(m.Qc) : nullptr, m.Un,
                                reinterpret_cast<T *>(m.Unc), m.acc, &L.sync->nonfinite, c.ph);
       break;
     case TASK_CORRECT:
       correct_body<N, T>(tk.begin + threadIdx.x < tk.end ? tk.begin + threadIdx.x : (int64_t)1 << 62, Rpart, FI, m.ef,
-                         met, m.E, MODE_RK, L.stage, L.dts[tk.cs], nullptr, m.Q,
+                         met, m.E, stage_coef(MODE_RK, L.stage, L.dts[tk.cs]), nullptr, m.Q,
                          m.mixed ? reinterpret_cast<T *>(m.Qc) : nullptr, m.Un, reinterpret_cast<T *>(m.Unc), m.acc,
                          &L.sync->nonfinite, c.ph);
       break;

@@ -49,15 +49,28 @@ __global__ void __launch_bounds__(prism_threads<N>(), prism_min_blocks<N, T>())
                           Gtr, Rpart, dph, if_up, n_interior);
 }
 
-template <int N, typename T>
-__global__ void k_prism_correct(const T *__restrict__ Rpart, const T *__restrict__ FI, const int32_t *__restrict__ ef_p,
-                                const T *__restrict__ metrics, const T *__restrict__ tab,
-                                const int32_t *__restrict__ tri_slot, int64_t Ep, int64_t first_point, int mode,
-                                int stage, double dt, double *__restrict__ Rout, double *__restrict__ Q,
-                                T *__restrict__ Qc, double *__restrict__ Un, T *__restrict__ Unc,
-                                double *__restrict__ acc, int *__restrict__ flag, DevPhys dph) {
-  prism_correct_body<N, T>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, Rpart, FI, ef_p, metrics, tab, tri_slot, Ep,
-                           first_point, mode, stage, dt, Rout, Q, Qc, Un, Unc, acc, flag, dph);
+template <int N, typename T, bool SRC>
+__global__ void __launch_bounds__(kCorrectThreads)
+    k_prism_correct(const T *__restrict__ Rpart, const T *__restrict__ FI, const int32_t *__restrict__ ef_p,
+                    const T *__restrict__ metrics, const T *__restrict__ tab, const int32_t *__restrict__ tri_slot,
+                    int64_t Ep, int64_t first_point, StageCoef sc, double *__restrict__ Rout,
+                    double *__restrict__ Q, T *__restrict__ Qc, double *__restrict__ Un, T *__restrict__ Unc,
+                    double *__restrict__ acc, int *__restrict__ flag, DevPhys dph) {
+  extern __shared__ double sm_raw[];
+  constexpr int Np = N * (N + 1) / 2 * N;
+  T *sr = reinterpret_cast<T *>(sm_raw);
+  const int64_t first = (int64_t)blockIdx.x * kCorrectThreads;
+  const int n = (int)(Ep * Np - first < kCorrectThreads ? Ep * Np - first : kCorrectThreads);
+  stage_partial<T>(sr, Rpart, first, n);
+  T rv[5], s{};
+  if ((int)threadIdx.x < n) {
+    const int64_t t = first + threadIdx.x, e = t / Np;
+    const int m = (int)(t % Np);
+    prism_correct_bracket<N, T>(e, m, sr + threadIdx.x * 5, FI, ef_p, tab, tri_slot, rv);
+    s = -metrics[(e * 10 + 9) * Np + m];
+  }
+  finish_block<T, SRC>(first_point + first, n, sr, sm_raw + 5 * kCorrectThreads, rv, s, sc, Rout, Q, Qc, Un,
+                  Unc, acc, flag, dph);
 }
 
 // dt bound per prism: cfl h / ((2p + 1) max(|u| + c)) over its points (FP64 state).
@@ -100,8 +113,9 @@ static cudaError_t prism_phase_impl(const DevMesh &m, const DevPhys &ph, int pha
                                                                           Gtr, Rpart, ph, m.if_up, m.n_interior);
   } else if (phase == 3) {
     const int64_t n = m.Ep * Np;
-    k_prism_correct<N, T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-        Rpart, FI, m.ef_p, met, tab, m.tri_slot, m.Ep, m.E * m.Np, mode, stage, dt, Rout, m.Q,
+    auto ck = has_source(ph) ? k_prism_correct<N, T, true> : k_prism_correct<N, T, false>;
+    ck<<<(unsigned)((n + kCorrectThreads - 1) / kCorrectThreads), kCorrectThreads, correct_smem(ph), st>>>(
+        Rpart, FI, m.ef_p, met, tab, m.tri_slot, m.Ep, m.E * m.Np, stage_coef(mode, stage, dt), Rout, m.Q,
         m.mixed ? reinterpret_cast<T *>(m.Qc) : nullptr, m.Un, reinterpret_cast<T *>(m.Unc), m.acc, m.flag, ph);
   }
   return cudaGetLastError();

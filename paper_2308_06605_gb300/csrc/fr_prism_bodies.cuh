@@ -314,23 +314,15 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
 // 4. Correction by the common flux, scaling and output / RK44 update.  Thread per prism point.
 // ------------------------------------------------------------------------------------------
 template <int N, typename T>
-__device__ __forceinline__ void prism_correct_body(int64_t t, const T *__restrict__ Rpart, const T *__restrict__ FI,
-                                                   const int32_t *__restrict__ ef_p, const T *__restrict__ metrics,
-                                                   const T *__restrict__ tab, const int32_t *__restrict__ tri_slot,
-                                                   int64_t Ep, int64_t first_point, int mode, int stage, double dt,
-                                                   double *__restrict__ Rout, double *__restrict__ Q,
-                                                   T *__restrict__ Qc, double *__restrict__ Un, T *__restrict__ Unc,
-                                                   double *__restrict__ acc, int *__restrict__ flag,
-                                                   const DevPhys &dph) {
-  constexpr int Nt = N * (N + 1) / 2, Np = Nt * N, Nf = N * N;
+__device__ __forceinline__ void prism_correct_bracket(int64_t e, int m, const T *rp, const T *__restrict__ FI,
+                                                      const int32_t *__restrict__ ef_p, const T *__restrict__ tab,
+                                                      const int32_t *__restrict__ tri_slot, T rv[5]) {
+  constexpr int Nt = N * (N + 1) / 2, Nf = N * N;
   constexpr PrismTab L = prism_tab(N);
-  if (t >= Ep * Np) return;
-  const int64_t e = t / Np;
-  const int m = (int)(t % Np), q = m % Nt, k = m / Nt;
-  const PhysT<T> &ph = phys_of<T>(dph);
+  const int q = m % Nt, k = m / Nt;
   Dot<T> r[5];
 #pragma unroll
-  for (int v = 0; v < 5; ++v) r[v].add(ph.one, Rpart[t * 5 + v]);
+  for (int v = 0; v < 5; ++v) r[v] = Dot<T>(rp[v]);
 #pragma unroll
   for (int f = 0; f < 2; ++f) {
     const int packed = ef_p[e * 5 + f];
@@ -357,11 +349,28 @@ __device__ __forceinline__ void prism_correct_body(int64_t t, const T *__restric
       for (int v = 0; v < 5; ++v) r[v].add(w, src[v * Nf + slot]);
     }
   }
-  const T s = -metrics[(e * 10 + 9) * Np + m];
-  T rv[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) rv[v] = r[v].get();
-  finish_point<T>(first_point + t, rv, s, mode, stage, dt, Rout, Q, Qc, Un, Unc, acc, flag, dph);
+}
+
+// Thread per point (batched stage).
+template <int N, typename T>
+__device__ __forceinline__ void prism_correct_body(int64_t t, const T *__restrict__ Rpart, const T *__restrict__ FI,
+                                                   const int32_t *__restrict__ ef_p, const T *__restrict__ metrics,
+                                                   const T *__restrict__ tab, const int32_t *__restrict__ tri_slot,
+                                                   int64_t Ep, int64_t first_point, const StageCoef &sc,
+                                                   double *__restrict__ Rout, double *__restrict__ Q,
+                                                   T *__restrict__ Qc, double *__restrict__ Un, T *__restrict__ Unc,
+                                                   double *__restrict__ acc, int *__restrict__ flag,
+                                                   const DevPhys &dph) {
+  constexpr int Np = N * (N + 1) / 2 * N;
+  if (t >= Ep * Np) return;
+  const int64_t e = t / Np;
+  const int m = (int)(t % Np);
+  T rv[5];
+  prism_correct_bracket<N, T>(e, m, Rpart + t * 5, FI, ef_p, tab, tri_slot, rv);
+  finish_point<T>(first_point + t, rv, -metrics[(e * 10 + 9) * Np + m], sc, Rout, Q, Qc, Un, Unc, acc,
+                  flag, dph);
 }
 
 }  // namespace

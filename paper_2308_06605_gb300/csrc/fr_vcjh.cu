@@ -23,16 +23,6 @@ __global__ void __launch_bounds__(volume_threads<N>(), volume_min_blocks<N>())
 }
 
 template <int N, typename T>
-__global__ void k_correct_vc(const T *__restrict__ Rpart, const T *__restrict__ FI, const int32_t *__restrict__ ef,
-                             const T *__restrict__ metrics, int64_t E, int mode, int stage, double dt,
-                             double *__restrict__ Rout, double *__restrict__ Q, T *__restrict__ Qc,
-                             double *__restrict__ Un, T *__restrict__ Unc, double *__restrict__ acc,
-                             int *__restrict__ flag, DevPhys dph) {
-  correct_body<N, T, true>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, Rpart, FI, ef, metrics, E, mode, stage,
-                           dt, Rout, Q, Qc, Un, Unc, acc, flag, dph);
-}
-
-template <int N, typename T>
 static cudaError_t vcjh_phase_impl(const DevMesh &m, const DevPhys &ph, int phase, int mode, int stage, double dt,
                                    double *Rout, cudaStream_t st) {
   constexpr int Np = N * N * N, Nf = N * N;
@@ -52,9 +42,10 @@ static cudaError_t vcjh_phase_impl(const DevMesh &m, const DevPhys &ph, int phas
         m.h, m.nu, m.if_up, m.n_interior);
   } else if (phase == 3) {
     const int64_t n = E * Np;
-    k_correct_vc<N, T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-        Rpart, FI, m.ef, met, E, mode, stage, dt, Rout, m.Q, m.mixed ? reinterpret_cast<T *>(m.Qc) : nullptr, m.Un,
-        reinterpret_cast<T *>(m.Unc), m.acc, m.flag, ph);
+    auto ck = has_source(ph) ? k_correct<N, T, true, true> : k_correct<N, T, true, false>;
+    ck<<<(unsigned)((n + kCorrectThreads - 1) / kCorrectThreads), kCorrectThreads, correct_smem(ph), st>>>(
+        Rpart, FI, m.ef, met, E, stage_coef(mode, stage, dt), Rout, m.Q,
+        m.mixed ? reinterpret_cast<T *>(m.Qc) : nullptr, m.Un, reinterpret_cast<T *>(m.Unc), m.acc, m.flag, ph);
   } else {
     return cudaErrorInvalidValue;
   }
