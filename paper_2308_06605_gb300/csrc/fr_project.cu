@@ -2,10 +2,12 @@
 // runs at low order and switches to a higher one; the state is carried over by the L2 projection
 // onto the target space in reference coordinates: Legendre modal coefficients on each hexahedron
 // axis (truncated or zero-padded), the orthonormal triangle modes times Legendre on the prism.
-// A one-off operation: one thread per target point, FP64, 1D operators from the host.
+// FP64, one axis at a time through shared memory, operators from the host as kernel parameters.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -37,38 +39,117 @@ void line_transfer(int p, int q, std::vector<double> &T) {
   }
 }
 
-// Hexahedra: out(i, j, k) = sum L[i][a] L[j][b] L[k][c] in(a, b, c); prisms:
-// out(t, k) = sum L[k][c] Tt[t][s] in(s, c).  Np/Nq: points per element of source / target.
-__global__ void k_project(const double *__restrict__ src, double *__restrict__ dst, const double *__restrict__ L,
-                          const double *__restrict__ Tt, int64_t n_elem, int Ns, int Nd, int Nts, int Ntd, int prism) {
-  const int Nq = prism ? Ntd * Nd : Nd * Nd * Nd, Np = prism ? Nts * Ns : Ns * Ns * Ns;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_elem * Nq) return;
-  const int64_t e = t / Nq;
-  const int m = (int)(t % Nq);
-  const double *in = src + e * Np * 5;
-  double acc[5] = {0, 0, 0, 0, 0};
-  if (!prism) {
-    const int i = m % Nd, j = (m / Nd) % Nd, k = m / (Nd * Nd);
-    for (int c = 0; c < Ns; ++c)
-      for (int b = 0; b < Ns; ++b) {
-        const double wbc = L[k * Ns + c] * L[j * Ns + b];
-        for (int a = 0; a < Ns; ++a) {
-          const double w = wbc * L[i * Ns + a];
-          const double *q = in + (a + Ns * (b + Ns * c)) * 5;
-          for (int v = 0; v < 5; ++v) acc[v] += w * q[v];
-        }
-      }
-  } else {
-    const int tt = m % Ntd, k = m / Ntd;
-    for (int c = 0; c < Ns; ++c)
-      for (int s = 0; s < Nts; ++s) {
-        const double w = L[k * Ns + c] * Tt[tt * Nts + s];
-        const double *q = in + (s + Nts * c) * 5;
-        for (int v = 0; v < 5; ++v) acc[v] += w * q[v];
-      }
+// Operators of one projection, passed by value as a kernel parameter (no device allocation or copy).
+struct LineOp {
+  double L[kMaxN * kMaxN];                          // [Nd][Ns]
+};
+constexpr int kMaxNt = kMaxN * (kMaxN + 1) / 2;
+struct PrismOp {
+  double L[kMaxN * kMaxN], T[kMaxNt * kMaxNt];      // line [Nd][Ns], triangle [Ntd][Nts]
+};
+
+// The projected state starts a new step: Q and U_n, and on the mixed path their double-float copies.
+struct StateOut {
+  double *Q, *Un;
+  df32 *Qc, *Unc;                                   // null on the FP64 path
+  __device__ __forceinline__ void put(int64_t o, double x) const {
+    Q[o] = x;
+    Un[o] = x;
+    if (Qc) Qc[o] = Unc[o] = df_from(x);
   }
-  for (int v = 0; v < 5; ++v) dst[(e * Nq + m) * 5 + v] = acc[v];
+};
+
+// One axis of ns -> ND values: item = lo + INNER (i + ND o), lo running over the values in front of the
+// axis (variables and faster axes), o over those behind it; in has the axis at c INNER within blocks of
+// ns INNER.  The target size is a template parameter, so the index arithmetic divides by constants.
+template <int ND, int INNER>
+__device__ __forceinline__ double along(const double *M, const double *in, int item, int ns) {
+  const int lo = item % INNER, r = item / INNER, i = r % ND, o = r / ND;
+  const double *x = in + o * ns * INNER + lo, *w = M + i * ns;
+  double acc = w[0] * x[0];
+  for (int c = 1; c < ns; ++c) acc = fma(w[c], x[c * INNER], acc);
+  return acc;
+}
+
+constexpr int kProjectThreads = 256;
+
+// Hexahedra, epb elements per block, one axis after the other through shared memory: out(i, j, k) =
+// sum_c L[k][c] sum_b L[j][b] sum_a L[i][a] in(a, b, c).  Bound by the FP64 pipe and then by memory: the
+// direct triple sum takes 160 operations per target point at p = 2 -> 4, the three passes 30.  GB300, 32^3
+// elements p = 2 -> 4, the whole call: 1.30 ms with the triple sum, device allocations for the operators
+// and the registers set by further copies -> PROJUS.
+template <int Nd>
+__global__ void __launch_bounds__(kProjectThreads)
+    k_project_hex(const double *__restrict__ src, StateOut out, const __grid_constant__ LineOp op, int64_t E, int Ns, int epb) {
+  extern __shared__ double sm[];
+  __shared__ double L[kMaxN * kMaxN];
+  const int n0 = Ns * Ns * Ns * 5, n1 = Nd * Ns * Ns * 5, n2 = Nd * Nd * Ns * 5, n3 = Nd * Nd * Nd * 5;
+  const int64_t e0 = (int64_t)blockIdx.x * epb;
+  const int ne = (int)(E - e0 < epb ? E - e0 : epb);
+  double *a = sm, *b = sm + (size_t)epb * (n0 > n2 ? n0 : n2);
+  for (int i = threadIdx.x; i < Ns * Nd; i += kProjectThreads) L[i] = op.L[i];
+  for (int i = threadIdx.x; i < ne * n0; i += kProjectThreads) a[i] = src[e0 * n0 + i];
+  __syncthreads();
+  for (int i = threadIdx.x; i < ne * n1; i += kProjectThreads) b[i] = along<Nd, 5>(L, a, i, Ns);
+  __syncthreads();
+  for (int i = threadIdx.x; i < ne * n2; i += kProjectThreads) a[i] = along<Nd, 5 * Nd>(L, b, i, Ns);
+  __syncthreads();
+  for (int i = threadIdx.x; i < ne * n3; i += kProjectThreads)
+    out.put(e0 * n3 + i, along<Nd, 5 * Nd * Nd>(L, a, i, Ns));
+}
+
+// Prisms: out(t, k) = sum_c L[k][c] sum_s T[t][s] in(s, c).
+template <int Nd>
+__global__ void __launch_bounds__(kProjectThreads)
+    k_project_prism(const double *__restrict__ src, StateOut out, const __grid_constant__ PrismOp op, int64_t E, int Ns,
+                    int epb) {
+  extern __shared__ double sm[];
+  constexpr int Ntd = Nd * (Nd + 1) / 2;
+  const int Nts = Ns * (Ns + 1) / 2;
+  const int n0 = Nts * Ns * 5, n1 = Ntd * Ns * 5, n2 = Ntd * Nd * 5;
+  const int64_t e0 = (int64_t)blockIdx.x * epb;
+  const int ne = (int)(E - e0 < epb ? E - e0 : epb);
+  double *T = sm, *L = T + Nts * Ntd, *a = L + Ns * Nd, *b = a + (size_t)epb * n0;
+  for (int i = threadIdx.x; i < Ns * Nd; i += kProjectThreads) L[i] = op.L[i];
+  for (int i = threadIdx.x; i < Nts * Ntd; i += kProjectThreads) T[i] = op.T[i];
+  for (int i = threadIdx.x; i < ne * n0; i += kProjectThreads) a[i] = src[e0 * n0 + i];
+  __syncthreads();
+  for (int i = threadIdx.x; i < ne * n1; i += kProjectThreads) b[i] = along<Ntd, 5>(T, a, i, Nts);
+  __syncthreads();
+  for (int i = threadIdx.x; i < ne * n2; i += kProjectThreads)
+    out.put(e0 * n2 + i, along<Nd, 5 * Ntd>(L, b, i, Ns));
+}
+
+// Elements per block: about four items per thread at the larger of the two orders, which also keeps the
+// block's shared memory below 48 KB.
+int project_epb(int values) { return std::min(16, std::max(1, 4 * kProjectThreads / values)); }
+
+template <int Nd>
+cudaError_t launch_project(const DevMesh &a, const DevMesh &b, const std::vector<double> &L,
+                           const std::vector<double> &Tt, cudaStream_t st) {
+  df32 *Qc = b.mixed ? reinterpret_cast<df32 *>(b.Qc) : nullptr, *Unc = b.mixed ? reinterpret_cast<df32 *>(b.Unc) : nullptr;
+  if (a.E > 0) {
+    LineOp op;
+    std::memcpy(op.L, L.data(), L.size() * sizeof(double));
+    const int epb = project_epb(std::max(a.Np, b.Np) * 5);
+    const size_t n0 = (size_t)a.Np, n1 = (size_t)b.N * a.N * a.N, n2 = (size_t)b.N * b.N * a.N;
+    const size_t smem = sizeof(double) * 5 * epb * (std::max(n0, n2) + n1);
+    k_project_hex<Nd><<<(unsigned)((a.E + epb - 1) / epb), kProjectThreads, smem, st>>>(
+        a.Q, StateOut{b.Q, b.Un, Qc, Unc}, op, a.E, a.N, epb);
+  }
+  if (a.Ep > 0) {
+    PrismOp op;
+    std::memcpy(op.L, L.data(), L.size() * sizeof(double));
+    std::memcpy(op.T, Tt.data(), Tt.size() * sizeof(double));
+    const int epb = project_epb(std::max(a.Npp, b.Npp) * 5);
+    const size_t smem = sizeof(double) * ((size_t)a.Nt * b.Nt + a.N * b.N + 5 * (size_t)epb * a.N * (a.Nt + b.Nt));
+    const int64_t os = a.E * a.Np * 5, od = b.E * b.Np * 5;
+    cudaError_t e = cudaFuncSetAttribute(k_project_prism<Nd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_project_prism<Nd><<<(unsigned)((a.Ep + epb - 1) / epb), kProjectThreads, smem, st>>>(
+        a.Q + os, StateOut{b.Q + od, b.Un + od, Qc ? Qc + od : nullptr, Unc ? Unc + od : nullptr}, op, a.Ep, a.N, epb);
+  }
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -103,30 +184,20 @@ extern "C" fr_status fr_project_state(fr_mesh *src, fr_mesh *dst) {
   line_transfer(a.p, b.p, L);
   if (a.Ep > 0 && !tri_transfer(a.p, b.p, Tt))
     return frx_mesh_fail(dst, FR_EMESH, "fr_project_state: triangle transfer failed");
-  double *dL = nullptr, *dT = nullptr;
-  cudaError_t e = cudaMalloc((void **)&dL, L.size() * sizeof(double));
-  if (e == cudaSuccess && !Tt.empty()) e = cudaMalloc((void **)&dT, Tt.size() * sizeof(double));
-  if (e == cudaSuccess) e = cudaStreamSynchronize(sa);   // the source state is complete
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dL, L.data(), L.size() * sizeof(double), cudaMemcpyHostToDevice, sb);
-  if (e == cudaSuccess && dT) e = cudaMemcpyAsync(dT, Tt.data(), Tt.size() * sizeof(double), cudaMemcpyHostToDevice, sb);
-  if (e == cudaSuccess && a.E > 0) {
-    const int64_t n = b.E * b.Np;
-    k_project<<<(unsigned)((n + 255) / 256), 256, 0, sb>>>(a.Q, b.Q, dL, nullptr, a.E, a.N, b.N, 0, 0, 0);
-    e = cudaGetLastError();
+  cudaError_t e = sa == sb ? cudaSuccess : cudaStreamSynchronize(sa);   // the source state is complete
+  if (e == cudaSuccess) {
+    switch (b.N) {
+      case 2: e = launch_project<2>(a, b, L, Tt, sb); break;
+      case 3: e = launch_project<3>(a, b, L, Tt, sb); break;
+      case 4: e = launch_project<4>(a, b, L, Tt, sb); break;
+      case 5: e = launch_project<5>(a, b, L, Tt, sb); break;
+      case 6: e = launch_project<6>(a, b, L, Tt, sb); break;
+      case 7: e = launch_project<7>(a, b, L, Tt, sb); break;
+      case 8: e = launch_project<8>(a, b, L, Tt, sb); break;
+      default: e = cudaErrorInvalidValue;
+    }
   }
-  if (e == cudaSuccess && a.Ep > 0) {
-    const int64_t n = b.Ep * b.Npp;
-    k_project<<<(unsigned)((n + 255) / 256), 256, 0, sb>>>(a.Q + a.E * a.Np * 5, b.Q + b.E * b.Np * 5, dL, dT, a.Ep,
-                                                           a.N, b.N, a.Nt, b.Nt, 1);
-    e = cudaGetLastError();
-  }
-  // The projected state starts a new step, as after fr_set_state.
-  const size_t bytes = ((size_t)b.E * b.Np + (size_t)b.Ep * b.Npp) * 5 * sizeof(double);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(b.Un, b.Q, bytes, cudaMemcpyDeviceToDevice, sb);
-  if (e == cudaSuccess) e = launch_state_copy(b, sb);
   if (e == cudaSuccess) e = cudaStreamSynchronize(sb);
-  if (dL) cudaFree(dL);
-  if (dT) cudaFree(dT);
   if (e != cudaSuccess) return frx_mesh_fail(dst, FR_ECUDA, std::string("fr_project_state: ") + cudaGetErrorString(e));
   return FR_OK;
 }
