@@ -81,8 +81,9 @@ void prism18_geometry(const CurvedOps &o, const TriBasis &tb, const double (*X)[
 
 // Offsets (in values) of the per-mesh prism operator table for line order N (Nt = N(N+1)/2):
 // Dr, Ds (triangle derivatives), Drt, Dst (with the own-flux correction of the quadrilateral
-// faces folded in), E [3][N][Nt], LQ [3][Nt][N], D1, D1t [N][N] (line derivative, plain and with
-// the own-flux correction of the triangular faces), then l(-1), l(+1), h-, h+ [N] each.
+// faces folded in), E [3], LQ [3], D1, D1t [N][N] (line derivative, plain and with the own-flux correction of
+// the triangular faces), then l(-1), l(+1), h-, h+ [N] each.  The triangle operators are stored with the
+// output index fastest (Dr[j][q], E[e][j][a], LQ[e][a][q]): consecutive threads own consecutive outputs.
 struct PrismTab {
   int Nt, Dr, Ds, Drt, Dst, E, LQ, D1, D1t, lm, lp, hm, hp, size;
 };

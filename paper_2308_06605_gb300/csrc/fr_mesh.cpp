@@ -844,10 +844,11 @@ fr_status build_host_mesh(const fr_mesh_desc *desc, HostMesh &m, std::string &er
     const PrismTab L = prism_tab(N);
     m.ptab.assign(L.size, 0.0);
     double *t = m.ptab.data();
-    for (int i = 0; i < Nt * Nt; ++i) {
-      t[L.Dr + i] = tb.Dr[i];
-      t[L.Ds + i] = tb.Ds[i];
-    }
+    for (int i = 0; i < Nt; ++i)
+      for (int j = 0; j < Nt; ++j) {
+        t[L.Dr + j * Nt + i] = tb.Dr[(size_t)i * Nt + j];
+        t[L.Ds + j * Nt + i] = tb.Ds[(size_t)i * Nt + j];
+      }
     // Own-flux correction of the quadrilateral faces (reference normals (0,-1,0), (1,1,0),
     // (-1,0,0) for edges 0, 1, 2): Drt = Dr - LQ1 E1 + LQ2 E2, Dst = Ds + LQ0 E0 - LQ1 E1.
     for (int i = 0; i < Nt; ++i)
@@ -858,12 +859,15 @@ fr_status build_host_mesh(const fr_mesh_desc *desc, HostMesh &m, std::string &er
           for (int a = 0; a < N; ++a) acc += (long double)tb.LQ[e][(size_t)i * N + a] * tb.E[e][(size_t)a * Nt + j];
           c[e] = acc;
         }
-        t[L.Drt + i * Nt + j] = (double)((long double)tb.Dr[(size_t)i * Nt + j] - c[1] + c[2]);
-        t[L.Dst + i * Nt + j] = (double)((long double)tb.Ds[(size_t)i * Nt + j] + c[0] - c[1]);
+        t[L.Drt + j * Nt + i] = (double)((long double)tb.Dr[(size_t)i * Nt + j] - c[1] + c[2]);
+        t[L.Dst + j * Nt + i] = (double)((long double)tb.Ds[(size_t)i * Nt + j] + c[0] - c[1]);
       }
     for (int e = 0; e < 3; ++e) {
-      for (int i = 0; i < N * Nt; ++i) t[L.E + e * N * Nt + i] = tb.E[e][i];
-      for (int i = 0; i < Nt * N; ++i) t[L.LQ + e * Nt * N + i] = tb.LQ[e][i];
+      for (int a = 0; a < N; ++a)
+        for (int j = 0; j < Nt; ++j) {
+          t[L.E + (e * Nt + j) * N + a] = tb.E[e][(size_t)a * Nt + j];
+          t[L.LQ + (e * N + a) * Nt + j] = tb.LQ[e][(size_t)j * N + a];
+        }
     }
     for (int i = 0; i < N; ++i) {
       for (int a = 0; a < N; ++a) {

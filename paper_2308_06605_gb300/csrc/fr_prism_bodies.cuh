@@ -89,10 +89,10 @@ __device__ __forceinline__ void prism_interp_body(int64_t t, const T *__restrict
     }
   } else {
     const int a = r % N, b = r / N;
-    const T *Ea = tab + L.E + (f - 2) * N * Nt + a * Nt;
+    const T *Ea = tab + L.E + (f - 2) * N * Nt + a;
 #pragma unroll 4
     for (int j = 0; j < Nt; ++j) {
-      const T ej = Ea[j];
+      const T ej = Ea[j * N];
       const T *qj = q + (j + Nt * b) * 5;
 #pragma unroll
       for (int v = 0; v < 5; ++v) acc[v].add(ej, qj[v]);
@@ -108,6 +108,11 @@ __device__ __forceinline__ void prism_interp_body(int64_t t, const T *__restrict
 
 // ------------------------------------------------------------------------------------------
 // 2. Volume kernel.  One block per prism, one thread per solution point.
+// Bound by FP32 issue (double-float) or the FP64 pipe.  Operator entries are read with consecutive
+// threads on consecutive addresses and once for the five variables (row-major tables cost 15 L1
+// wavefronts per load at p = 4, and were read per variable); the gradient sums are bounded ones (Acc).  On
+// the cascade passage (72 case: 25 200 hexahedra, 10 080 prisms, p = 4) the two volume kernels together
+// 1.505 -> 1.236 ms in double-float, 5.06 -> 4.60 ms in FP64.
 // ------------------------------------------------------------------------------------------
 // One prism e handled by `nth` threads of the block (thread index tid in [0, nth)); every thread
 // of the block calls this together (it contains block barriers); inactive sub-blocks
@@ -130,8 +135,9 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
   T *sdQ = sL + 15 * Np;      // [5][5][Nf] Q^I - Q_own at the flux points
   const PhysT<T> &ph = phys_of<T>(dph);
   const bool viscous = dph.viscous != 0;
-  if (active)
-    for (int t = tid; t < 5 * Np; t += nth) sQ[(t % 5) * Np + t / 5] = Q[e * Np * 5 + t];
+  // The gradient acts on the perturbation from the prism's first point (its only reader of sQ).
+  if (active && viscous)
+    for (int t = tid; t < 5 * Np; t += nth) sQ[(t % 5) * Np + t / 5] = Q[e * Np * 5 + t] - Q[e * Np * 5 + t % 5];
   if (viscous && active) {
     for (int t = tid; t < 5 * Nf; t += nth) {
       const int f = t / Nf, r = t % Nf;
@@ -159,62 +165,109 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
     for (int c = 0; c < 9; ++c) S[c] = met[c * Np];
     invJ = met[9 * Np];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) qv[v] = sQ[v * Np + m];
+    for (int v = 0; v < 5; ++v) qv[v] = Q[(e * Np + m) * 5 + v];
     if (viscous) {
-      const T *Dr = tab + L.Dr + q * Nt, *Ds = tab + L.Ds + q * Nt, *D1 = tab + L.D1 + k * N;
-      const T hmk = tab[L.hm + k], hpk = tab[L.hp + k];
-      const T *LQ0 = tab + L.LQ + q * N, *LQ1 = LQ0 + Nt * N, *LQ2 = LQ1 + Nt * N;
       T sj[9];   // S[d][jj] / |J|
 #pragma unroll
       for (int c = 0; c < 9; ++c) sj[c] = S[c] * invJ;
-      // One variable at a time: reference gradient, liftings, correction, physical transform.  The
-      // loop stays rolled (a smaller instruction footprint): the corrected gradient goes through this
-      // thread's own entries of the transformed-flux buffer, which only this thread writes later.
+      // Reference gradient, uncorrected (sG) and corrected (sH), in this thread's own entries, which
+      // only it writes before the next barrier.  Lifted jumps of the quadrilateral faces first (edge
+      // f - 2); sum_f N_f C_f dQ_f with N = (0,0,-1), (0,0,1), (0,-1,0), (1,1,0), (-1,0,0).
+#pragma unroll 1
+      for (int f = 0; f < 3; ++f) {
+        const T *lq = tab + L.LQ + f * N * Nt + q, *dq = sdQ + (2 + f) * 5 * Nf + N * k;
+        T c[N];
+#pragma unroll
+        for (int a = 0; a < N; ++a) c[a] = lq[a * Nt];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          Bound<T> bd;
+#pragma unroll
+          for (int a = 0; a < N; ++a) bd.add(c[a], dq[v * Nf + a]);
+          Acc<T> s(bd);
+#pragma unroll
+          for (int a = 0; a < N; ++a) s.add(c[a], dq[v * Nf + a]);
+          sL[(f * 5 + v) * Np + m] = s.raw();
+        }
+      }
+      {
+        const T *D1 = tab + L.D1 + k * N;
+        const T hmk = -tab[L.hm + k], hpk = tab[L.hp + k];
+        T c[N];
+#pragma unroll
+        for (int a = 0; a < N; ++a) c[a] = D1[a];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          const T jlo = sdQ[v * Nf + q], jhi = sdQ[(5 + v) * Nf + q];
+          Bound<T> bd;
+#pragma unroll
+          for (int a = 0; a < N; ++a) bd.add(c[a], sQ[v * Np + q + Nt * a]);
+          bd.add(hmk, jlo);
+          bd.add(hpk, jhi);
+          Acc<T> s(bd);
+#pragma unroll
+          for (int a = 0; a < N; ++a) s.add(c[a], sQ[v * Np + q + Nt * a]);
+          sG[(10 + v) * Np + m] = s.raw();
+          s.add(hmk, jlo);
+          s.add(hpk, jhi);
+          sH[(10 + v) * Np + m] = s.raw();
+        }
+      }
+      {
+        // Both triangle derivatives of the five variables together: an operator entry is read once.
+        const T *Dr = tab + L.Dr + q, *Ds = tab + L.Ds + q, *sq = sQ + Nt * k;
+        Bound<T> b0[5], b1[5];
+#pragma unroll 3
+        for (int j = 0; j < Nt; ++j) {
+          const T dr = Dr[j * Nt], ds = Ds[j * Nt];
+#pragma unroll
+          for (int v = 0; v < 5; ++v) {
+            const T x = sq[v * Np + j];
+            b0[v].add(dr, x);
+            b1[v].add(ds, x);
+          }
+        }
+        Acc<T> a0[5] = {Acc<T>(b0[0]), Acc<T>(b0[1]), Acc<T>(b0[2]), Acc<T>(b0[3]), Acc<T>(b0[4])};
+        Acc<T> a1[5] = {Acc<T>(b1[0]), Acc<T>(b1[1]), Acc<T>(b1[2]), Acc<T>(b1[3]), Acc<T>(b1[4])};
+#pragma unroll 3
+        for (int j = 0; j < Nt; ++j) {
+          const T dr = Dr[j * Nt], ds = Ds[j * Nt];
+#pragma unroll
+          for (int v = 0; v < 5; ++v) {
+            const T x = sq[v * Np + j];
+            a0[v].add(dr, x);
+            a1[v].add(ds, x);
+          }
+        }
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          const T g0 = a0[v].raw(), g1 = a1[v].raw();
+          sG[v * Np + m] = g0;
+          sG[(5 + v) * Np + m] = g1;
+          const T L2 = sL[v * Np + m], L3 = sL[(5 + v) * Np + m], L4 = sL[(10 + v) * Np + m];
+          Dot<T> c0(g0), c1(g1);
+          c0.plus(L3);
+          c0.plus(-L4);
+          c1.plus(L3);
+          c1.plus(-L2);
+          sH[v * Np + m] = c0.raw();
+          sH[(5 + v) * Np + m] = c1.raw();
+        }
+      }
 #pragma unroll 1
       for (int v = 0; v < 5; ++v) {
-        const T *sq = sQ + v * Np;
-        Dot<T> a0, a1, a2;
-#pragma unroll 4
-        for (int j = 0; j < Nt; ++j) {
-          const T qj = sq[j + Nt * k];
-          a0.add(Dr[j], qj);
-          a1.add(Ds[j], qj);
-        }
+        T gu[3], gc[3];
 #pragma unroll
-        for (int c = 0; c < N; ++c) a2.add(D1[c], sq[q + Nt * c]);
-        const T gu0 = a0.raw(), gu1 = a1.raw(), gu2 = a2.raw();
-        // Lifted jumps: quadrilateral faces (edge e = f - 2) and the two triangles.
-        Dot<T> l2, l3, l4;
-#pragma unroll
-        for (int a = 0; a < N; ++a) {
-          l2.add(LQ0[a], sdQ[(2 * 5 + v) * Nf + a + N * k]);
-          l3.add(LQ1[a], sdQ[(3 * 5 + v) * Nf + a + N * k]);
-          l4.add(LQ2[a], sdQ[(4 * 5 + v) * Nf + a + N * k]);
+        for (int d = 0; d < 3; ++d) {
+          gu[d] = sG[(d * 5 + v) * Np + m];
+          gc[d] = sH[(d * 5 + v) * Np + m];
         }
-        const T L2 = l2.raw(), L3 = l3.raw(), L4 = l4.raw();
-        sL[(0 * 5 + v) * Np + m] = L2;
-        sL[(1 * 5 + v) * Np + m] = L3;
-        sL[(2 * 5 + v) * Np + m] = L4;
-        // sum_f N_f C_f dQ_f with N = (0,0,-1), (0,0,1), (0,-1,0), (1,1,0), (-1,0,0).
-        a0.add(ph.one, L3);
-        a0.add(-ph.one, L4);
-        a1.add(-ph.one, L2);
-        a1.add(ph.one, L3);
-        a2.add(-hmk, sdQ[(0 * 5 + v) * Nf + q]);
-        a2.add(hpk, sdQ[(1 * 5 + v) * Nf + q]);
-        const T gc0 = a0.raw(), gc1 = a1.raw(), gc2 = a2.raw();
 #pragma unroll
         for (int jj = 0; jj < 3; ++jj) {
-          Dot<T> du, dc;
-          du.add(sj[0 * 3 + jj], gu0);
-          du.add(sj[1 * 3 + jj], gu1);
-          du.add(sj[2 * 3 + jj], gu2);
-          dc.add(sj[0 * 3 + jj], gc0);
-          dc.add(sj[1 * 3 + jj], gc1);
-          dc.add(sj[2 * 3 + jj], gc2);
-          const T gc = dc.raw();
-          sH[(jj * 5 + v) * Np + m] = gc;
-          sG[(jj * 5 + v) * Np + m] = dph.ldg ? gc : du.raw();   // LDG: corrected
+          const T du = dot3(sj[jj], gu[0], sj[3 + jj], gu[1], sj[6 + jj], gu[2]);
+          const T dc = dot3(sj[jj], gc[0], sj[3 + jj], gc[1], sj[6 + jj], gc[2]);
+          sH[(jj * 5 + v) * Np + m] = dc;
+          sG[(jj * 5 + v) * Np + m] = dph.ldg ? dc : du;   // LDG: corrected
         }
       }
 #pragma unroll
@@ -247,66 +300,114 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
     }
   }
   __syncthreads();
-  if (viscous && active) {
-    // Gradient traces: interpolated uncorrected gradient + eta * own lifting.  One item per
-    // (gradient component jj, face point) keeps the block busy.
-    for (int t = tid; t < 15 * Nf; t += nth) {
-      const int jj = t / (5 * Nf), fr_ = t - jj * 5 * Nf;
-      const int f = fr_ / Nf, r = fr_ % Nf;
-      if (f < 2 && r >= Nt) continue;
-      const int packed = ef_p[e * 5 + f];
-      const int64_t I = packed >> 4;
-      const int side = (packed >> 3) & 1;
-      T *dst = Gtr + (I * 2 + side) * 15 * Nf + prism_slot<N>(f, r, packed & 7, tri_slot);
-      if (f < 2) {
-        const T *l = tab + (f ? L.lp : L.lm), *hh = tab + (f ? L.hp : L.hm);
+  if (viscous) {
+    // Gradient traces: interpolated uncorrected gradient + eta * own lifting.  Triangular faces: one item
+    // per (gradient component jj, face point).
+    if (active)
+      for (int t = tid; t < 6 * Nt; t += nth) {
+        const int jj = t / (2 * Nt), f = t / Nt % 2, r = t % Nt;
+        const int packed = ef_p[e * 5 + f];
+        const int64_t I = packed >> 4;
+        T *dst = Gtr + (I * 2 + ((packed >> 3) & 1)) * 15 * Nf + prism_slot<N>(f, r, packed & 7, tri_slot) + jj * 5 * Nf;
+        const T *hh = tab + (f ? L.hp : L.hm);
+        T l[N];
+#pragma unroll
+        for (int c = 0; c < N; ++c) l[c] = tab[(f ? L.lp : L.lm) + c];
         Dot<T> lf;
 #pragma unroll
         for (int c = 0; c < N; ++c) lf.add(l[c] * hh[c], sW[(f * 3 + jj) * Np + r + Nt * c]);
         const T lfac = lf.raw();
 #pragma unroll 1
         for (int v = 0; v < 5; ++v) {
-          Dot<T> acc;
+          const T *g = sG + (jj * 5 + v) * Np + r;
+          const T jump = sdQ[(f * 5 + v) * Nf + r];
+          Bound<T> bd;
 #pragma unroll
-          for (int c = 0; c < N; ++c) acc.add(l[c], sG[(jj * 5 + v) * Np + r + Nt * c]);
-          acc.add(lfac, sdQ[(f * 5 + v) * Nf + r]);
-          dst[(jj * 5 + v) * Nf] = acc.raw();
-        }
-      } else {
-        const int a = r % N, b = r / N;
-        const T *Ea = tab + L.E + (f - 2) * N * Nt + a * Nt;
-        const T *lq = sL + ((f - 2) * 5) * Np + Nt * b;
-        const T *w = sW + (f * 3 + jj) * Np + Nt * b;
-#pragma unroll 1
-        for (int v = 0; v < 5; ++v) {
-          const T *g = sG + (jj * 5 + v) * Np + Nt * b;
-          Dot<T> acc;
-          for (int j = 0; j < Nt; ++j) {
-            acc.add(Ea[j], g[j]);
-            acc.add(Ea[j] * w[j], lq[v * Np + j]);
-          }
-          dst[(jj * 5 + v) * Nf] = acc.raw();
+          for (int c = 0; c < N; ++c) bd.add(l[c], g[Nt * c]);
+          bd.add(lfac, jump);
+          Acc<T> acc(bd);
+#pragma unroll
+          for (int c = 0; c < N; ++c) acc.add(l[c], g[Nt * c]);
+          acc.add(lfac, jump);
+          dst[v * Nf] = acc.raw();
         }
       }
+    __syncthreads();
+    // Quadrilateral faces, one after the other: every point adds the face's lifting to its gradient (kept in
+    // registers), the sum replaces the gradient in sG, and the face points interpolate it.  (Interpolating
+    // gradient and lifting by themselves took a product and two sums per term: 2.4 times the
+    // instructions.)
+    T g[15];
+    if (pt) {
+#pragma unroll
+      for (int c = 0; c < 15; ++c) g[c] = sG[c * Np + m];
+    }
+#pragma unroll 1
+    for (int f = 2; f < 5; ++f) {
+      if (pt) {
+#pragma unroll
+        for (int jj = 0; jj < 3; ++jj) {
+          const T w = sW[(f * 3 + jj) * Np + m];
+#pragma unroll
+          for (int v = 0; v < 5; ++v)
+            sG[(jj * 5 + v) * Np + m] = muladd(g[jj * 5 + v], w, sL[((f - 2) * 5 + v) * Np + m]);
+        }
+      }
+      __syncthreads();
+      if (active)
+        for (int t = tid; t < 3 * Nf; t += nth) {
+          const int jj = t / Nf, r = t % Nf, a = r % N, b = r / N;
+          const int packed = ef_p[e * 5 + f];
+          const int64_t I = packed >> 4;
+          T *dst = Gtr + (I * 2 + ((packed >> 3) & 1)) * 15 * Nf + prism_slot<N>(f, r, packed & 7, tri_slot) + jj * 5 * Nf;
+          const T *Ea = tab + L.E + (f - 2) * N * Nt + a, *x = sG + jj * 5 * Np + Nt * b;
+          Bound<T> bd[5];
+#pragma unroll 3
+          for (int j = 0; j < Nt; ++j) {
+            const T ej = Ea[j * N];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) bd[v].add(ej, x[v * Np + j]);
+          }
+          Acc<T> acc[5] = {Acc<T>(bd[0]), Acc<T>(bd[1]), Acc<T>(bd[2]), Acc<T>(bd[3]), Acc<T>(bd[4])};
+#pragma unroll 3
+          for (int j = 0; j < Nt; ++j) {
+            const T ej = Ea[j * N];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) acc[v].add(ej, x[v * Np + j]);
+          }
+#pragma unroll
+          for (int v = 0; v < 5; ++v) dst[v * Nf] = acc[v].raw();
+        }
+      if (f < 4) __syncthreads();
     }
   }
   if (pt) {
-    const T *Drt = tab + L.Drt + q * Nt, *Dst = tab + L.Dst + q * Nt, *D1t = tab + L.D1t + k * N;
+    const T *Drt = tab + L.Drt + q, *Dst = tab + L.Dst + q, *D1t = tab + L.D1t + k * N;
+    const T *h0 = sH + Nt * k, *h1 = h0 + 5 * Np, *h2 = sH + 10 * Np + q;
+    Dot<T> acc[5];
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+      const T dc = D1t[c];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        if (c == 0)
+          acc[v] = Dot<T>(dc, h2[v * Np]);
+        else
+          acc[v].add(dc, h2[v * Np + Nt * c]);
+      }
+    }
+#pragma unroll 3
+    for (int j = 0; j < Nt; ++j) {
+      const T dr = Drt[j * Nt], ds = Dst[j * Nt];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        acc[v].add(dr, h0[v * Np + j]);
+        acc[v].add(ds, h1[v * Np + j]);
+      }
+    }
     T *out = Rpart + (e * Np + m) * 5;
 #pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      const T *h0 = sH + (0 * 5 + v) * Np + Nt * k, *h1 = sH + (1 * 5 + v) * Np + Nt * k;
-      const T *h2 = sH + (2 * 5 + v) * Np + q;
-      Dot<T> acc;
-#pragma unroll 4
-      for (int j = 0; j < Nt; ++j) {
-        acc.add(Drt[j], h0[j]);
-        acc.add(Dst[j], h1[j]);
-      }
-#pragma unroll
-      for (int c = 0; c < N; ++c) acc.add(D1t[c], h2[Nt * c]);
-      out[v] = acc.raw();
-    }
+    for (int v = 0; v < 5; ++v) out[v] = acc[v].raw();
   }
 }
 
@@ -339,11 +440,11 @@ __device__ __forceinline__ void prism_correct_bracket(int64_t e, int m, const T 
     const int packed = ef_p[e * 5 + f];
     const int64_t I = packed >> 4;
     const int side = (packed >> 3) & 1;
-    const T *lq = tab + L.LQ + (f - 2) * Nt * N + q * N;
+    const T *lq = tab + L.LQ + (f - 2) * Nt * N + q;
     const T *src = FI + I * 5 * Nf;
 #pragma unroll
     for (int a = 0; a < N; ++a) {
-      const T w = side ? -lq[a] : lq[a];
+      const T w = side ? -lq[a * Nt] : lq[a * Nt];
       const int slot = orient_slot(packed & 7, a, k, N);
 #pragma unroll
       for (int v = 0; v < 5; ++v) r[v].add(w, src[v * Nf + slot]);
