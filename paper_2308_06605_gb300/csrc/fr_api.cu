@@ -558,7 +558,12 @@ extern "C" fr_status fr_set_closure(fr_mesh *m, const float *params, const float
     if (!(scales[11 + k] > 0.f)) return fail(m, FR_EINVAL, "closure input scales must be positive");
   const int n = FR_CLOSURE_NPARAMS;
   std::vector<uint16_t> w(n);
+  // Device order: the three weight matrices input-major ([input][64]) for coalesced reads, the rest as given.
+  const int in[3] = {11, 64, 64};
   for (int k = 0; k < n; ++k) w[k] = bf16_bits(params[k]);
+  for (int l = 0, o = 0; l < 3; o += 64 * in[l] + 64, ++l)
+    for (int j = 0; j < 64; ++j)
+      for (int c = 0; c < in[l]; ++c) w[o + c * 64 + j] = bf16_bits(params[o + j * in[l] + c]);
   DevMesh &d = m->dev;
   if (!m->d_cw) {
     fr_status s;
