@@ -76,7 +76,7 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
       if (n > 0 && m.tc) {
         if ((err = launch_interp_tc(m, st)) != cudaSuccess) return err;
       } else if (n > 0) {
-        k_interp_faces_smem<N, T><<<(unsigned)((E + epb - 1) / epb), kInterpThreads, 0, st>>>(Qin, m.ef, Qtr, E);
+        k_interp_faces_smem<N, T><<<(unsigned)((E + epb - 1) / epb), interp_threads<N>(), 0, st>>>(Qin, m.ef, Qtr, E);
       }
     } else if (n > 0) {
       k_interp_faces<N, T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(Qin, m.ef, Qtr, E);
