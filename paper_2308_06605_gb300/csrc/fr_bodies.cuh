@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(interp_threads<N>())
 // 2. Volume kernel.  One block per element, one thread per solution point.
 // ------------------------------------------------------------------------------------------
 template <int N>
-constexpr int volume_threads() { return ((N * N * N + 31) / 32) * 32; }
+__host__ __device__ constexpr int volume_threads() { return ((N * N * N + 31) / 32) * 32; }
 // Resident blocks the register budget must allow (smem allows at least this many).
 template <int N>
 constexpr int volume_min_blocks() {
@@ -296,30 +296,42 @@ constexpr int volume_min_blocks() {
 template <int N>
 __host__ __device__ constexpr int volume_smem_values() { return 35 * N * N * N + 30 * N * N; }
 
+// Shared memory of the closure's features and activations, and the block's elements: element e0 + l of
+// l < n has closure_floats<N>() floats at red + l * closure_floats<N>().
+struct ClosureSpace {
+  float *red;
+  int64_t e0;
+  int n, mine;         // elements of the block, and the calling thread's
+};
+template <int N>
+__host__ __device__ constexpr int closure_floats() { return 10 * N * N * N + 1 + 128; }
+
 // One element e handled by `nth` threads of the block (thread index tid in [0, nth)); every
 // thread of the block calls this together (it contains block barriers); inactive sub-blocks
 // (active = false) only take part in the barriers.
-template <int N, typename T, bool VC = false, bool FP32V = false>
+// VISC: 1 viscous, 0 inviscid (only the transformed flux lives in shared memory), 2 decided at run time.
+template <int N, typename T, bool VC, bool FP32V, int VISC>
 __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool active, double *sm_raw,
                                             const T *__restrict__ Q, const T *__restrict__ metrics,
                                             const int32_t *__restrict__ ef, const T *__restrict__ Qtr,
                                             const T *__restrict__ liftfac, T *__restrict__ Gtr,
                                             T *__restrict__ Rpart, const DevPhys &dph,
                                             const double *__restrict__ hel, float *__restrict__ nu_out,
-                                            const int8_t *__restrict__ if_up, int64_t n_interior) {
+                                            const int8_t *__restrict__ if_up, int64_t n_interior,
+                                            const ClosureSpace &cs) {
   constexpr int Np = N * N * N, Nf = N * N;
   using TG = typename GradOf<T, FP32V>::type;   // arithmetic of the viscous branch
   constexpr bool kPert = !std::is_same<TG, T>::value;
   T *sm = reinterpret_cast<T *>(sm_raw);
   T *sQ = sm;                                                // [5][Np]
   TG *sG = reinterpret_cast<TG *>(sQ + 5 * Np);              // [15][Np] uncorrected physical gradient, j*5+v
-  T *sH = sQ + 20 * Np;                                      // [15][Np] transformed flux, index d*5+v
+  T *sH = VISC == 0 ? sm : sQ + 20 * Np;                     // [15][Np] transformed flux, index d*5+v
   TG *sdQ = reinterpret_cast<TG *>(sH + 15 * Np);            // [6][5][Nf] Q^I - Q_own at the flux points
   // FP32 viscous branch: Q minus the element's first point, in FP32, in the upper half of the
   // gradient buffer (the FP32 gradient uses only its lower half).
   TG *sQg = kPert ? reinterpret_cast<TG *>(sQ + 5 * Np) + 15 * Np : nullptr;   // [5][Np]
   // Double-float viscous branch: sQ itself holds the perturbation (only the gradient reads it).
-  constexpr bool kPertDf = std::is_same<TG, df32>::value;
+  constexpr bool kPertDf = std::is_same<TG, df32>::value || VISC == 0;
   const PhysT<T> &ph = phys_of<T>(dph);
   const PhysT<TG> &phg = phys_of<TG>(dph);
   const BasisT<T> &B = basis_ref<N, T, VC>(dph);
@@ -333,7 +345,7 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   // FP32 issue (69 % of the issue slots at 4 warps per scheduler): the bounded sums, the three-term
   // products and paired traces took the double-float kernel from 8860 to 7540 instructions per
   // warp, 4.375 -> 3.80 ms per launch at 48^3 p = 4, 1.34 -> 1.18 ms at 40^3 p = 3, errors unchanged.
-  const bool viscous = dph.viscous != 0;
+  const bool viscous = VISC == 2 ? dph.viscous != 0 : VISC == 1;
   const bool pt = active && tid < Np;
   const int m = tid < Np ? tid : 0, i = m % N, j = (m / N) % N, k = m / (N * N);
   // The point's metric terms are loaded before the staging loops so that their latency overlaps them.
@@ -452,8 +464,8 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   T rho_nu = ph.zero;
   if (viscous && dph.closure) {
     // Eddy-viscosity closure: quadrature-weighted element mean of the corrected velocity
-    // gradient, then one warp evaluates the network (BF16 weights, FP32 accumulation).
-    float *red = reinterpret_cast<float *>(sm + volume_smem_values<N>());   // [10][Np] + 129
+    // gradient, then one warp per element evaluates the network (BF16 weights, FP32 accumulation).
+    float *red = cs.red + cs.mine * closure_floats<N>();
     if (pt) {
       const double ri = 1.0 / to_double(q[0]);
       const double w = (double)B.w[i] * B.w[j] * B.w[k] / to_double(invJ);
@@ -467,12 +479,14 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
       red[9 * Np + m] = (float)w;
     }
     __syncthreads();
-    if (active && tid < 32) {
+    const int lane = threadIdx.x & 31;
+    for (int l = threadIdx.x >> 5; l < cs.n; l += blockDim.x >> 5) {
+      float *rl = cs.red + l * closure_floats<N>();
       float acc[10];
 #pragma unroll
       for (int c = 0; c < 10; ++c) {
         float sacc = 0.f;
-        for (int mm = tid; mm < Np; mm += 32) sacc += red[c * Np + mm];
+        for (int mm = lane; mm < Np; mm += 32) sacc += rl[c * Np + mm];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, o);
         acc[c] = sacc;
@@ -489,11 +503,11 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
           ss += sab * sab;
         }
       x[9] = sqrtf(2.f * ss);
-      x[10] = (float)(hel[e] / N);
-      const float nu = closure_mlp(dph, x, red + 10 * Np + 1, tid);
-      if (tid == 0) {
-        red[10 * Np] = nu;
-        if (nu_out) nu_out[e] = nu;
+      x[10] = (float)(hel[cs.e0 + l] / N);
+      const float nu = closure_mlp(dph, x, rl + 10 * Np + 1, lane);
+      if (lane == 0) {
+        rl[10 * Np] = nu;
+        if (nu_out) nu_out[cs.e0 + l] = nu;
       }
     }
     __syncthreads();
@@ -613,15 +627,47 @@ constexpr int volume_min_blocks_of() {
   return N == 3 ? 20 : (N == 4 ? 10 : (N == 5 ? 5 : (N == 6 ? 3 : (N == 7 ? 2 : volume_min_blocks<N>()))));
 }
 
-template <int N, typename T, bool FP32V = false>
-__global__ void __launch_bounds__(volume_threads<N>(), volume_min_blocks_of<N, T>())
+// Elements per block: one, but 16 (128 threads) at p = 1, whose 8 points would fill a quarter of a warp
+// (double-float 48^3: 0.89 -> 0.295 ms per launch).  At p = 2 (27 of 32 lanes) 7 elements in 192 threads or 9
+// in 256 measured slower than one warp per element (FP64 with the closure 0.470 and 0.459 against 0.448 ms).
+template <int N>
+__host__ __device__ constexpr int volume_epb() { return N == 2 ? 16 : 1; }
+template <int N>
+__host__ __device__ constexpr int volume_block() {
+  return volume_epb<N>() == 1 ? volume_threads<N>() : (volume_epb<N>() * N * N * N + 31) / 32 * 32;
+}
+
+// Euler runs (VISC = 0): 15 N^3 values of shared memory instead of 35 N^3 + 30 N^2 and no gradient
+// registers, so 1024 threads per SM at 64 registers (704 at p = 6).
+template <int N, typename T, int VISC>
+constexpr int volume_blocks() {
+  return VISC == 0 ? (N == 7 ? 2 : (N == 3 ? 32 : 1024 / volume_block<N>()))
+                   : (N == 2 ? 4 : volume_min_blocks_of<N, T>());
+}
+
+// Dynamic shared memory of a block.
+template <int N, typename T>
+size_t volume_smem(bool viscous, bool closure) {
+  return volume_epb<N>() * (viscous ? sizeof(T) * volume_smem_values<N>() + (closure ? sizeof(float) * closure_floats<N>() : 0)
+                                    : sizeof(T) * 15 * N * N * N);
+}
+
+template <int N, typename T, bool FP32V, int VISC>
+__global__ void __launch_bounds__(volume_block<N>(), volume_blocks<N, T, VISC>())
     k_volume(const T *__restrict__ Q, const T *__restrict__ metrics, const int32_t *__restrict__ ef,
              const T *__restrict__ Qtr, const T *__restrict__ liftfac, T *__restrict__ Gtr, T *__restrict__ Rpart,
              DevPhys dph, const double *__restrict__ hel, float *__restrict__ nu_out,
-             const int8_t *__restrict__ if_up, int64_t n_interior) {
+             const int8_t *__restrict__ if_up, int64_t n_interior, int64_t E) {
   extern __shared__ double sm_raw[];
-  volume_body<N, T, false, FP32V>(blockIdx.x, threadIdx.x, blockDim.x, true, sm_raw, Q, metrics, ef, Qtr, liftfac, Gtr,
-                                  Rpart, dph, hel, nu_out, if_up, n_interior);
+  constexpr int EPB = volume_epb<N>(), VALS = VISC == 0 ? 15 * N * N * N : volume_smem_values<N>();
+  constexpr int NTH = EPB == 1 ? volume_threads<N>() : N * N * N;
+  const int64_t e0 = (int64_t)blockIdx.x * EPB;
+  const int le = EPB == 1 ? 0 : (int)threadIdx.x / NTH, tid = EPB == 1 ? (int)threadIdx.x : (int)threadIdx.x % NTH;
+  const int n = EPB == 1 ? 1 : (int)(E - e0 < EPB ? E - e0 : EPB);
+  const int mine = EPB == 1 || le < n ? le : 0;
+  const ClosureSpace cs{reinterpret_cast<float *>(sm_raw + EPB * VALS), e0, n, mine};
+  volume_body<N, T, false, FP32V, VISC>(e0 + mine, tid, NTH, EPB == 1 || le < n, sm_raw + mine * VALS, Q, metrics, ef,
+                                        Qtr, liftfac, Gtr, Rpart, dph, hel, nu_out, if_up, n_interior, cs);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1044,8 +1090,8 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const BatchCase 
       const int tid = (int)threadIdx.x % nth;
       const int64_t e = tk.begin + le;
       const bool active = le < epb && e < tk.end;
-      volume_body<N, T>(e, tid, nth, active, smem + (size_t)(le < epb ? le : 0) * volume_smem_values<N>(), Qin, met,
-                        m.ef, Qtr, lift, Gtr, Rpart, c.ph, m.h, nullptr, m.if_up, m.n_interior);
+      volume_body<N, T, false, false, 2>(e, tid, nth, active, smem + (size_t)(le < epb ? le : 0) * volume_smem_values<N>(), Qin, met,
+                        m.ef, Qtr, lift, Gtr, Rpart, c.ph, m.h, nullptr, m.if_up, m.n_interior, ClosureSpace{nullptr, 0, 0, 0});
       break;
     }
     case TASK_IFACE:

@@ -18,8 +18,9 @@ __global__ void __launch_bounds__(volume_threads<N>(), volume_min_blocks<N>())
                 DevPhys dph, const double *__restrict__ hel, float *__restrict__ nu_out,
                 const int8_t *__restrict__ if_up, int64_t n_interior) {
   extern __shared__ double sm_raw[];
-  volume_body<N, T, true>(blockIdx.x, threadIdx.x, blockDim.x, true, sm_raw, Q, metrics, ef, Qtr, liftfac, Gtr,
-                          Rpart, dph, hel, nu_out, if_up, n_interior);
+  volume_body<N, T, true, false, 2>(blockIdx.x, threadIdx.x, blockDim.x, true, sm_raw, Q, metrics, ef, Qtr, liftfac, Gtr,
+                          Rpart, dph, hel, nu_out, if_up, n_interior,
+                          ClosureSpace{reinterpret_cast<float *>(sm_raw + volume_smem_values<N>()), blockIdx.x, 1, 0});
 }
 
 template <int N, typename T>
@@ -34,7 +35,7 @@ static cudaError_t vcjh_phase_impl(const DevMesh &m, const DevPhys &ph, int phas
   T *Rpart = reinterpret_cast<T *>(m.Rpart);
   const T *met = reinterpret_cast<const T *>(m.metrics);
   if (phase == 1) {
-    const size_t smem = sizeof(T) * (35 * Np + 30 * Nf) + (ph.closure ? sizeof(float) * (10 * Np + 1 + 128) : 0);
+    const size_t smem = sizeof(T) * (35 * Np + 30 * Nf) + (ph.closure ? sizeof(float) * closure_floats<N>() : 0);
     cudaError_t err = cudaFuncSetAttribute(k_volume_vc<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     k_volume_vc<N, T><<<(unsigned)E, volume_threads<N>(), smem, st>>>(
