@@ -919,23 +919,26 @@ __global__ void k_bc_flux(const T *__restrict__ Qtr, const T *__restrict__ Gtr, 
 // ------------------------------------------------------------------------------------------
 // 4. Correction by the common flux, scaling, and output / RK44 stage update (FP64).
 // ------------------------------------------------------------------------------------------
-// Bracket of Eq. 3 at point m of element e: the partial residual rp (5 values) plus the lifted common
-// fluxes of the six faces.
+// Lifted common fluxes of the six faces at point m of element e, on top of the partial residual rp (may be
+// null): the bracket of Eq. 3.
 template <int N, typename T, bool VC>
-__device__ __forceinline__ void correct_bracket(int64_t e, int m, const T *rp, const T *__restrict__ FI,
-                                                const int32_t *__restrict__ ef, const DevPhys &dph, T rv[5]) {
+__device__ __forceinline__ void correct_lift(int64_t e, int m, const T *__restrict__ FI, const int32_t *__restrict__ ef,
+                                             const DevPhys &dph, const T *rp, Dot<T> r[5]) {
+  if (rp)
+#pragma unroll
+    for (int v = 0; v < 5; ++v) r[v] = Dot<T>(rp[v]);
   constexpr int Nf = N * N;
   const int i = m % N, j = (m / N) % N, k = m / (N * N);
   const BasisT<T> &B = basis_ref<N, T, VC>(dph);
-  Dot<T> r[5];
-#pragma unroll
-  for (int v = 0; v < 5; ++v) r[v] = Dot<T>(rp[v]);
   // Faces: (weight, local flux point (a, b)).
   const int fa[6] = {j, j, i, i, i, i};
   const int fb[6] = {k, k, k, k, j, j};
   const T wts[6] = {B.hm[i], B.hp[i], B.hm[j], B.hp[j], B.hm[k], B.hp[k]};
+  // Double-float adds the partial residual after the faces: the xi faces come last, so that in either order
+  // each direction's large pressure parts meet soon after one another.
 #pragma unroll
-  for (int f = 0; f < 6; ++f) {
+  for (int g = 0; g < 6; ++g) {
+    const int f = kGatherFirst<T> ? 5 - g : g;
     const int packed = ef[e * 6 + f];
     const int64_t I = packed >> 4;
     const int side = (packed >> 3) & 1;
@@ -943,10 +946,13 @@ __device__ __forceinline__ void correct_bracket(int64_t e, int m, const T *rp, c
     const T w = side ? -wts[f] : wts[f];
     const T *src = FI + I * 5 * Nf + slot;
 #pragma unroll
-    for (int v = 0; v < 5; ++v) r[v].add(w, src[v * Nf]);
+    for (int v = 0; v < 5; ++v) {
+      if (g == 0 && !rp)
+        r[v] = Dot<T>(w, src[v * Nf]);
+      else
+        r[v].add(w, src[v * Nf]);
+    }
   }
-#pragma unroll
-  for (int v = 0; v < 5; ++v) rv[v] = r[v].get();
 }
 
 // Thread per point (batched stage).
@@ -961,32 +967,41 @@ __device__ __forceinline__ void correct_body(int64_t t, const T *__restrict__ Rp
   if (t >= E * Np) return;
   const int64_t e = t / Np;
   const int m = (int)(t % Np);
+  Dot<T> r[5];
+  correct_lift<N, T, false>(e, m, FI, ef, dph, kGatherFirst<T> ? nullptr : Rpart + t * 5, r);
   T rv[5];
-  correct_bracket<N, T, false>(e, m, Rpart + t * 5, FI, ef, dph, rv);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    if constexpr (kGatherFirst<T>) r[v].plus(Rpart[t * 5 + v]);
+    rv[v] = r[v].get();
+  }
   finish_point<T>(t, rv, -metrics[(e * 10 + 9) * Np + m], sc, Rout, Q, Qc, Un, Unc, acc, flag, dph);
 }
 
 template <int N, typename T, bool VC, bool SRC>
-__global__ void __launch_bounds__(kCorrectThreads, 6) k_correct(const T *__restrict__ Rpart, const T *__restrict__ FI,
+__global__ void __launch_bounds__(kCorrectThreads, std::is_same<T, double>::value ? 6 : 5) k_correct(const T *__restrict__ Rpart, const T *__restrict__ FI,
                           const int32_t *__restrict__ ef, const T *__restrict__ metrics, int64_t E,
                           StageCoef sc, double *__restrict__ Rout, double *__restrict__ Q, T *__restrict__ Qc,
                           double *__restrict__ Un, T *__restrict__ Unc, double *__restrict__ acc,
                           int *__restrict__ flag, DevPhys dph) {
   extern __shared__ double sm_raw[];
   constexpr int Np = N * N * N;
-  T *sr = reinterpret_cast<T *>(sm_raw);
+  const CorrectSmem sm(sm_raw);
   const int64_t first = (int64_t)blockIdx.x * kCorrectThreads;
   const int n = (int)(E * Np - first < kCorrectThreads ? E * Np - first : kCorrectThreads);
-  stage_partial<T>(sr, Rpart, first, n);
-  T rv[5], s{};
+  const StageIn in = stage_inputs<T>(sc, Q, Un, Unc, acc);
+  stage_begin<T>(sm, Rpart + first * 5, first * 5, n, in);
+  Dot<T> r[5];
+  T s{};
+  if constexpr (!kGatherFirst<T>) stage_arrive();
   if ((int)threadIdx.x < n) {
     const int64_t t = first + threadIdx.x, e = t / Np;
     const int m = (int)(t % Np);
-    correct_bracket<N, T, VC>(e, m, sr + threadIdx.x * 5, FI, ef, dph, rv);
+    correct_lift<N, T, VC>(e, m, FI, ef, dph,
+                           kGatherFirst<T> ? nullptr : reinterpret_cast<const T *>(sm.r) + threadIdx.x * 5, r);
     s = -metrics[(e * 10 + 9) * Np + m];
   }
-  finish_block<T, SRC>(first, n, sr, sm_raw + 5 * kCorrectThreads, rv, s, sc, Rout, Q, Qc, Un, Unc, acc, flag,
-                  dph);
+  finish_block<T, SRC>(first, n, sm, r, s, sc, in, Rout, Q, Qc, Un, Unc, acc, flag, dph);
 }
 
 // Meshes with prisms: a triangular interface uses only the first N(N+1)/2 of its N^2 slots;

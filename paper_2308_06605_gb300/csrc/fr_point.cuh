@@ -304,11 +304,32 @@ __host__ __device__ __forceinline__ StageCoef stage_coef(int mode, int stage, do
 // residual without source terms in the element arithmetic, src its source term (FP64; SRC: a template
 // parameter, because as a select its addition and conversion would be paid for by every value).
 // MODE_RESIDUAL writes R; the other modes update the FP64 registers (acc, U_n) and the stage state
-// (FP64 Q, and on the mixed path its double-float copy Qc).  Returns true for a non-finite value at
-// the last stage.
+// (FP64 Q, and on the mixed path its double-float copy Qc).  x1 and x2 are the old register values the
+// stage reads (stage_inputs).  Returns true for a non-finite value at the last stage.
 // ------------------------------------------------------------------------------------------
+// The two arrays a stage reads besides the residual, as 8-byte words (null: not read).  RK44: acc after the
+// first stage, and U_n (its double-float copy for a mixed stage state); SSP(3,3): Q, U_n; SSP(10,4): Q, and
+// U_n or acc where the registers recombine.
+struct StageIn {
+  const double *x1, *x2;
+};
+template <typename T>
+__device__ __forceinline__ StageIn stage_inputs(const StageCoef &c, const double *Q, const double *Un, const T *Unc,
+                                                const double *acc) {
+  if (c.mode == MODE_RESIDUAL) return StageIn{nullptr, nullptr};
+  if (c.mode == MODE_RK) {
+    const double *u = Un;
+    if constexpr (std::is_same<T, df32>::value)
+      if (!c.last) u = reinterpret_cast<const double *>(Unc);
+    return StageIn{c.stage > 0 ? acc : nullptr, u};
+  }
+  if (c.mode == MODE_SSP33) return StageIn{Q, Un};
+  return StageIn{Q, c.last ? acc : (c.stage == 4 ? Un : nullptr)};
+}
+__device__ __forceinline__ df32 as_df32(double x) { return *reinterpret_cast<df32 *>(&x); }
+
 template <typename T, bool SRC>
-__device__ __forceinline__ bool finish_value(int64_t o, T rs, double src, const StageCoef &c,
+__device__ __forceinline__ bool finish_value(int64_t o, T rs, double src, const StageCoef &c, double x1, double x2,
                                              double *__restrict__ Rout, double *__restrict__ Q, T *__restrict__ Qc,
                                              double *__restrict__ Un, T *__restrict__ Unc, double *__restrict__ acc) {
   double rd = to_double(rs);
@@ -323,14 +344,14 @@ __device__ __forceinline__ bool finish_value(int64_t o, T rs, double src, const 
       // formed in double-float from the df32 copy of U_n (with a source term from the FP64 residual,
       // which includes it).
       if (!c.last) {
-        acc[o] = fma(c.b, rd, c.stage == 0 ? 0.0 : acc[o]);
+        acc[o] = fma(c.b, rd, x1);
         if constexpr (SRC)
-          Qc[o] = Unc[o] + df(c.a_hi, c.a_lo) * from_double<T>(rd);
+          Qc[o] = as_df32(x2) + df(c.a_hi, c.a_lo) * from_double<T>(rd);
         else
-          Qc[o] = Unc[o] + df(c.a_hi, c.a_lo) * rs;
+          Qc[o] = as_df32(x2) + df(c.a_hi, c.a_lo) * rs;
         return false;
       }
-      const double nv = fma(c.b, rd, Un[o] + acc[o]);
+      const double nv = fma(c.b, rd, x2 + x1);
       Un[o] = nv;
       Q[o] = nv;
       const T nc = from_double<T>(nv);
@@ -338,13 +359,12 @@ __device__ __forceinline__ bool finish_value(int64_t o, T rs, double src, const 
       Qc[o] = nc;
       return !isfinite(nv);
     } else {
-      const double un = Un[o];
       if (!c.last) {
-        acc[o] = (c.stage == 0 ? 0.0 : acc[o]) + c.b * rd;
-        Q[o] = un + c.a * rd;
+        acc[o] = x1 + c.b * rd;
+        Q[o] = x2 + c.a * rd;
         return false;
       }
-      const double nv = un + acc[o] + c.b * rd;
+      const double nv = x2 + x1 + c.b * rd;
       Un[o] = nv;
       Q[o] = nv;
       return !isfinite(nv);
@@ -355,19 +375,19 @@ __device__ __forceinline__ bool finish_value(int64_t o, T rs, double src, const 
   //   SSP(3,3):  Q <- a_k U_n + b_k (Q + dt R), (a, b) = (0, 1), (3/4, 1/4), (1/3, 2/3).
   //   SSP(10,4): Q <- Q + dt/6 R at stages 0..8; after stage 4 the registers recombine,
   //              q2 = U_n/25 + 9/25 Q, Q <- 15 q2 - 5 Q; stage 9: Q <- q2 + 3/5 Q + dt/10 R.
-  const double q = Q[o];
+  const double q = x1;
   double nq;
   if (c.mode == MODE_SSP33) {
-    nq = c.a * Un[o] + c.b * fma(c.dt, rd, q);
+    nq = c.a * x2 + c.b * fma(c.dt, rd, q);
   } else if (!c.last) {
     nq = fma(c.b, rd, q);
     if (c.stage == 4) {
-      const double q2 = Un[o] / 25.0 + 9.0 / 25.0 * nq;
+      const double q2 = x2 / 25.0 + 9.0 / 25.0 * nq;
       acc[o] = q2;
       nq = 15.0 * q2 - 5.0 * nq;
     }
   } else {
-    nq = acc[o] + 0.6 * q + c.b * rd;
+    nq = x2 + 0.6 * q + c.b * rd;
   }
   Q[o] = nq;
   if constexpr (std::is_same<T, df32>::value) Qc[o] = from_double<T>(nq);
@@ -408,16 +428,23 @@ __device__ __forceinline__ void finish_point(int64_t t, const T rv[5], T s, cons
                                              double *__restrict__ Un, T *__restrict__ Unc, double *__restrict__ acc,
                                              int *__restrict__ flag, const DevPhys &dph) {
   bool bad = false;
+  const StageIn in = stage_inputs<T>(c, Q, Un, Unc, acc);
+  double x1[5], x2[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    x1[v] = in.x1 ? in.x1[t * 5 + v] : 0.0;
+    x2[v] = in.x2 ? in.x2[t * 5 + v] : 0.0;
+  }
   if (dph.src_body || dph.src_sponge) {
     double src[5];
     point_source<T>(t, Q, Qc, dph, src);
 #pragma unroll
     for (int v = 0; v < 5; ++v)
-      bad |= finish_value<T, true>(t * 5 + v, rv[v] * s, src[v], c, Rout, Q, Qc, Un, Unc, acc);
+      bad |= finish_value<T, true>(t * 5 + v, rv[v] * s, src[v], c, x1[v], x2[v], Rout, Q, Qc, Un, Unc, acc);
   } else {
 #pragma unroll
     for (int v = 0; v < 5; ++v)
-      bad |= finish_value<T, false>(t * 5 + v, rv[v] * s, 0.0, c, Rout, Q, Qc, Un, Unc, acc);
+      bad |= finish_value<T, false>(t * 5 + v, rv[v] * s, 0.0, c, x1[v], x2[v], Rout, Q, Qc, Un, Unc, acc);
   }
   if (bad) atomicOr(flag, 1);
 }
@@ -427,49 +454,83 @@ __device__ __forceinline__ void finish_point(int64_t t, const T rv[5], T s, cons
 // partial residual is staged through shared memory (sr, 5 values per thread), the thread of a
 // point replaces its five entries by the residual, and the update runs over the block's values.  With
 // a thread reading its own point's values each 8-byte access of a warp touches ten 128-byte lines.
-// Double-float 48^3 p = 4 1.07 -> 0.93 ms per launch (1.09 ms with the stage coefficients from the host
-// but not the staging), FP64 32^3 p = 4 0.447 -> 0.399 ms; bound by the FP64 pipe (two conversions, an
-// addition and an FMA per value) beside 3.5 GB of traffic (0.51 ms).  6 blocks per SM (40 registers); 5
-// measured 0.97 ms.
+// The copies into shared memory (cp.async: partial residual and the stage's two old register values) are in
+// flight while the double-float kernel gathers the fluxes.  Double-float 48^3 p = 4 1.07 -> 0.80 ms per launch
+// (0.93 with the partial residual alone staged by plain loads), FP64 32^3 p = 4 0.447 -> 0.398 ms; bound by the
+// FP64 pipe (two conversions, an addition and an FMA per value) beside 3.5 GB of traffic (0.51 ms at
+// 48^3).  FP64 6 blocks per SM (40 registers), double-float 5 (48; 6 measured the same).
 constexpr int kCorrectThreads = 256;
 
+// Shared memory of a block: the partial residual (replaced by the residual), the stage's two old register
+// values, and with source terms their five FP64 values per point.
+struct CorrectSmem {
+  double *r, *x1, *x2, *src;
+  __device__ __forceinline__ explicit CorrectSmem(double *p)
+      : r(p), x1(p + 5 * kCorrectThreads), x2(p + 10 * kCorrectThreads), src(p + 15 * kCorrectThreads) {}
+};
+
+__device__ __forceinline__ void copy_async8(double *dst, const double *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+
+// Start the copies of everything the block reads by value; the lifted fluxes are gathered meanwhile.  base:
+// first value of the block in the registers, part: of its partial residual, n: points.
 template <typename T>
-__device__ __forceinline__ void stage_partial(T *sr, const T *__restrict__ Rpart, int64_t first, int n) {
-  for (int i = threadIdx.x; i < n * 5; i += kCorrectThreads) sr[i] = Rpart[first * 5 + i];
+__device__ __forceinline__ void stage_begin(const CorrectSmem &sm, const T *part, int64_t base, int n, const StageIn &in) {
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const int i = threadIdx.x + k * kCorrectThreads;
+    if (i < n * 5) {
+      copy_async8(sm.r + i, reinterpret_cast<const double *>(part) + i);
+      if (in.x1) copy_async8(sm.x1 + i, in.x1 + base + i);
+      if (in.x2) copy_async8(sm.x2 + i, in.x2 + base + i);
+    }
+  }
+}
+__device__ __forceinline__ void stage_arrive() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
 }
 
-// first: flat index of the block's first point in the registers, n: points of the block; this thread's
-// bracket rv and s = -1/|J| (used if threadIdx.x < n).  ss: shared memory for the source terms.
+// Double-float gathers and lifts the fluxes while the copies arrive and adds the partial residual last; in
+// FP64 that addition is one more operation per value on the pipe that bounds the kernel (0.399 -> 0.447 ms
+// at 32^3 p = 4), so there the sum starts from the staged residual.
+template <typename T> constexpr bool kGatherFirst = std::is_same<T, df32>::value;
+
+// first: flat index of the block's first point in the registers, n: points of the block; this thread's lifted
+// fluxes rv (FP64: with the partial residual) and s = -1/|J| (used if threadIdx.x < n).
 template <typename T, bool SRC>
-__device__ __forceinline__ void finish_block(int64_t first, int n, T *sr, double *ss, const T rv[5], T s,
-                                             const StageCoef &c, double *__restrict__ Rout, double *__restrict__ Q,
-                                             T *__restrict__ Qc, double *__restrict__ Un, T *__restrict__ Unc,
-                                             double *__restrict__ acc, int *__restrict__ flag, const DevPhys &dph) {
+__device__ __forceinline__ void finish_block(int64_t first, int n, const CorrectSmem &sm, Dot<T> rv[5], T s,
+                                             const StageCoef &c, const StageIn &in, double *__restrict__ Rout,
+                                             double *__restrict__ Q, T *__restrict__ Qc, double *__restrict__ Un,
+                                             T *__restrict__ Unc, double *__restrict__ acc, int *__restrict__ flag,
+                                             const DevPhys &dph) {
   const int me = threadIdx.x;
+  T *sr = reinterpret_cast<T *>(sm.r);
+  if constexpr (kGatherFirst<T>) stage_arrive();
   if (me < n) {
 #pragma unroll
-    for (int v = 0; v < 5; ++v) sr[me * 5 + v] = rv[v] * s;
+    for (int v = 0; v < 5; ++v) {
+      if constexpr (kGatherFirst<T>) rv[v].plus(sr[me * 5 + v]);
+      sr[me * 5 + v] = rv[v].get() * s;
+    }
     if constexpr (SRC) {
       double src[5];
       point_source<T>(first + me, Q, Qc, dph, src);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) ss[me * 5 + v] = src[v];
+      for (int v = 0; v < 5; ++v) sm.src[me * 5 + v] = src[v];
     }
   }
   __syncthreads();
   bool bad = false;
 #pragma unroll 5
   for (int i = me; i < n * 5; i += kCorrectThreads)
-    bad |= finish_value<T, SRC>(first * 5 + i, sr[i], SRC ? ss[i] : 0.0, c, Rout, Q, Qc, Un, Unc, acc);
+    bad |= finish_value<T, SRC>(first * 5 + i, sr[i], SRC ? sm.src[i] : 0.0, c, in.x1 ? sm.x1[i] : 0.0,
+                                in.x2 ? sm.x2[i] : 0.0, Rout, Q, Qc, Un, Unc, acc);
   if (bad) atomicOr(flag, 1);
 }
 
 inline bool has_source(const DevPhys &ph) { return ph.src_body || ph.src_sponge; }
-// Shared memory of a correction block: the staged residual and, with a source term, its five FP64
-// values per point.
-inline size_t correct_smem(const DevPhys &ph) {
-  return sizeof(double) * 5 * kCorrectThreads * (has_source(ph) ? 2 : 1);
-}
+inline size_t correct_smem(const DevPhys &ph) { return sizeof(double) * 5 * kCorrectThreads * (has_source(ph) ? 4 : 3); }
 
 }  // namespace frx

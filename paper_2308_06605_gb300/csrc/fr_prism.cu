@@ -58,19 +58,22 @@ __global__ void __launch_bounds__(kCorrectThreads)
                     double *__restrict__ acc, int *__restrict__ flag, DevPhys dph) {
   extern __shared__ double sm_raw[];
   constexpr int Np = N * (N + 1) / 2 * N;
-  T *sr = reinterpret_cast<T *>(sm_raw);
+  const CorrectSmem sm(sm_raw);
   const int64_t first = (int64_t)blockIdx.x * kCorrectThreads;
   const int n = (int)(Ep * Np - first < kCorrectThreads ? Ep * Np - first : kCorrectThreads);
-  stage_partial<T>(sr, Rpart, first, n);
-  T rv[5], s{};
+  const StageIn in = stage_inputs<T>(sc, Q, Un, Unc, acc);
+  stage_begin<T>(sm, Rpart + first * 5, (first_point + first) * 5, n, in);
+  Dot<T> r[5];
+  T s{};
+  if constexpr (!kGatherFirst<T>) stage_arrive();
   if ((int)threadIdx.x < n) {
     const int64_t t = first + threadIdx.x, e = t / Np;
     const int m = (int)(t % Np);
-    prism_correct_bracket<N, T>(e, m, sr + threadIdx.x * 5, FI, ef_p, tab, tri_slot, rv);
+    prism_correct_lift<N, T>(e, m, FI, ef_p, tab, tri_slot,
+                             kGatherFirst<T> ? nullptr : reinterpret_cast<const T *>(sm.r) + threadIdx.x * 5, r);
     s = -metrics[(e * 10 + 9) * Np + m];
   }
-  finish_block<T, SRC>(first_point + first, n, sr, sm_raw + 5 * kCorrectThreads, rv, s, sc, Rout, Q, Qc, Un,
-                  Unc, acc, flag, dph);
+  finish_block<T, SRC>(first_point + first, n, sm, r, s, sc, in, Rout, Q, Qc, Un, Unc, acc, flag, dph);
 }
 
 // dt bound per prism: cfl h / ((2p + 1) max(|u| + c)) over its points (FP64 state).

@@ -415,15 +415,15 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
 // 4. Correction by the common flux, scaling and output / RK44 update.  Thread per prism point.
 // ------------------------------------------------------------------------------------------
 template <int N, typename T>
-__device__ __forceinline__ void prism_correct_bracket(int64_t e, int m, const T *rp, const T *__restrict__ FI,
-                                                      const int32_t *__restrict__ ef_p, const T *__restrict__ tab,
-                                                      const int32_t *__restrict__ tri_slot, T rv[5]) {
+__device__ __forceinline__ void prism_correct_lift(int64_t e, int m, const T *__restrict__ FI,
+                                                   const int32_t *__restrict__ ef_p, const T *__restrict__ tab,
+                                                   const int32_t *__restrict__ tri_slot, const T *rp, Dot<T> r[5]) {
+  if (rp)
+#pragma unroll
+    for (int v = 0; v < 5; ++v) r[v] = Dot<T>(rp[v]);
   constexpr int Nt = N * (N + 1) / 2, Nf = N * N;
   constexpr PrismTab L = prism_tab(N);
   const int q = m % Nt, k = m / Nt;
-  Dot<T> r[5];
-#pragma unroll
-  for (int v = 0; v < 5; ++v) r[v] = Dot<T>(rp[v]);
 #pragma unroll
   for (int f = 0; f < 2; ++f) {
     const int packed = ef_p[e * 5 + f];
@@ -433,7 +433,12 @@ __device__ __forceinline__ void prism_correct_bracket(int64_t e, int m, const T 
     const T w = side ? -h : h;
     const T *src = FI + I * 5 * Nf + tri_slot[(packed & 7) * Nt + q];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) r[v].add(w, src[v * Nf]);
+    for (int v = 0; v < 5; ++v) {
+      if (f == 0 && !rp)
+        r[v] = Dot<T>(w, src[v * Nf]);
+      else
+        r[v].add(w, src[v * Nf]);
+    }
   }
 #pragma unroll
   for (int f = 2; f < 5; ++f) {
@@ -450,8 +455,6 @@ __device__ __forceinline__ void prism_correct_bracket(int64_t e, int m, const T 
       for (int v = 0; v < 5; ++v) r[v].add(w, src[v * Nf + slot]);
     }
   }
-#pragma unroll
-  for (int v = 0; v < 5; ++v) rv[v] = r[v].get();
 }
 
 // Thread per point (batched stage).
@@ -468,8 +471,14 @@ __device__ __forceinline__ void prism_correct_body(int64_t t, const T *__restric
   if (t >= Ep * Np) return;
   const int64_t e = t / Np;
   const int m = (int)(t % Np);
+  Dot<T> r[5];
+  prism_correct_lift<N, T>(e, m, FI, ef_p, tab, tri_slot, kGatherFirst<T> ? nullptr : Rpart + t * 5, r);
   T rv[5];
-  prism_correct_bracket<N, T>(e, m, Rpart + t * 5, FI, ef_p, tab, tri_slot, rv);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    if constexpr (kGatherFirst<T>) r[v].plus(Rpart[t * 5 + v]);
+    rv[v] = r[v].get();
+  }
   finish_point<T>(first_point + t, rv, -metrics[(e * 10 + 9) * Np + m], sc, Rout, Q, Qc, Un, Unc, acc,
                   flag, dph);
 }
