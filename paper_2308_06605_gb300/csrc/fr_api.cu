@@ -455,10 +455,28 @@ static cudaMemcpyKind kind_of(int where, bool to_device) {
   return to_device ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost;
 }
 
+// True if a kernel of this mesh may read p directly: an aligned pointer to plain memory of the mesh's
+// device, which is the current one.  Anything else a copy accepts (another device's memory, an odd
+// address, a thread on another device) keeps the copies.
+static bool readable_here(const fr_mesh *m, const void *p) {
+  if (reinterpret_cast<uintptr_t>(p) % sizeof(double)) return false;
+  int cur = -1;
+  cudaPointerAttributes at;
+  if (cudaGetDevice(&cur) != cudaSuccess || cur != m->device || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == m->device;
+}
+
 extern "C" fr_status fr_set_state(fr_mesh *m, const double *Q, int32_t where) {
   fr_status st = check_mesh(m);
   if (st) return st;
   if (!Q || (where != FR_HOST && where != FR_DEVICE)) return fail(m, FR_EINVAL, "bad state pointer or where");
+  if (where == FR_DEVICE && readable_here(m, Q)) {
+    FR_CUDA(m, launch_start_state(m->dev, Q, m->stream));
+    return FR_OK;
+  }
   const size_t bytes = state_bytes(m->dev);
   FR_CUDA(m, cudaMemcpyAsync(m->dev.Q, Q, bytes, kind_of(where, true), m->stream));
   FR_CUDA(m, cudaMemcpyAsync(m->dev.Un, m->dev.Q, bytes, cudaMemcpyDeviceToDevice, m->stream));

@@ -188,6 +188,8 @@ cudaError_t upload_tc_tables();
 
 // Mixed path: refresh the df32 copy of the state after it was set from outside.
 cudaError_t launch_state_copy(const DevMesh &m, cudaStream_t st);
+// Q, U_n and their double-float copies from a state on the mesh's device (8-byte aligned).
+cudaError_t launch_start_state(const DevMesh &m, const double *src, cudaStream_t st);
 cudaError_t launch_max_dt(const DevMesh &m, const DevPhys &ph, double cfl, double *d_out, cudaStream_t st);
 
 }  // namespace frx
