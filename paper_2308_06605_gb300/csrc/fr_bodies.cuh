@@ -30,6 +30,7 @@
 
 #include "df32.cuh"
 #include "fr_device.hpp"
+#include "fr_f32x2.cuh"
 #include "fr_point.cuh"
 #include "fr_prism_bodies.cuh"
 
@@ -341,8 +342,10 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   // element's first point, which makes up for Acc's larger error where a variable has a large mean
   // (density, energy).  The divergence keeps Dot: it acts on the flux itself, whose pressure part is
   // nearly constant at low Mach number, and with Acc the momentum residual's error against 64 bits grew
-  // from 3.8e-10 to 1.2e-9 (TGV 40^3, p = 3, Ma 0.1) for 3 % of the kernel's time.  The kernel is bound by
-  // FP32 issue (69 % of the issue slots at 4 warps per scheduler): the bounded sums, the three-term
+  // from 3.8e-10 to 1.2e-9 (TGV 40^3, p = 3, Ma 0.1) for 3 % of the kernel's time.  Transform and traces use
+  // packed instructions in double-float (48^3 p = 4 3.09 -> 3.00 ms, 28^3 p = 5 1.174 -> 1.154, but 24^3 p = 6 1.30 ->
+  // 1.315 with its spills; packing the gradient's and the flux's
+  // variables in pairs as well measured 3.03).  The kernel is bound by FP32 issue (69 % of the issue slots at 4 warps per scheduler): the bounded sums, the three-term
   // products and paired traces took the double-float kernel from 8860 to 7540 instructions per
   // warp, 4.375 -> 3.80 ms per launch at 48^3 p = 4, 1.34 -> 1.18 ms at 40^3 p = 3, errors unchanged.
   const bool viscous = VISC == 2 ? dph.viscous != 0 : VISC == 1;
@@ -389,9 +392,17 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
 #pragma unroll
     for (int v = 0; v < 5; ++v) q[v] = kPertDf ? Q[(e * Np + m) * 5 + v] : sQ[v * Np + m];
     if (viscous) {
-      TG sj[9];   // S[d][jj] / |J|
+      // S[d][jj] / |J|.  Double-float transforms the uncorrected and the corrected gradient as the two lanes
+      // of packed instructions (their parts wait in shared memory lane by lane: (hi, hi) in sG, (lo, lo) in sGc).
+      constexpr bool kPack = std::is_same<TG, df32>::value;
+      typename std::conditional<kPack, d2, TG>::type sj[9];
 #pragma unroll
-      for (int c = 0; c < 9; ++c) sj[c] = to_g<TG>(S[c] * invJ);
+      for (int c = 0; c < 9; ++c) {
+        if constexpr (kPack)
+          sj[c] = dup(S[c] * invJ);
+        else
+          sj[c] = to_g<TG>(S[c] * invJ);
+      }
       // The reference gradient, uncorrected and corrected, goes through shared memory, in this thread's
       // own entries of the gradient and transformed-flux buffers, which only this thread writes before
       // the next barrier (R gradient values of type TG per entry of type T).
@@ -434,27 +445,53 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
           Acc<TG> s(bd);
 #pragma unroll
           for (int a = 0; a < N; ++a) s.add(c[a], x[a]);
-          sG[(d * 5 + v) * Np + m] = s.raw();
+          const TG gu = s.raw();
           s.add(hlo, jlo);
           s.add(hhi, jhi);
-          sGc[gslot(d * 5 + v)] = s.raw();
+          const TG gc = s.raw();
+          if constexpr (kPack) {
+            sG[(d * 5 + v) * Np + m] = df(gu.hi, gc.hi);
+            sGc[gslot(d * 5 + v)] = df(gu.lo, gc.lo);
+          } else {
+            sG[(d * 5 + v) * Np + m] = gu;
+            sGc[gslot(d * 5 + v)] = gc;
+          }
         }
       }
 #pragma unroll 1
       for (int v = 0; v < 5; ++v) {
-        TG gu[3], gc[3];
+        TG du[3], dc[3];
+        if constexpr (kPack) {
+          d2 g[3];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          gu[d] = sG[(d * 5 + v) * Np + m];
-          gc[d] = sGc[gslot(d * 5 + v)];
+          for (int d = 0; d < 3; ++d) {
+            const df32 h = sG[(d * 5 + v) * Np + m], l = sGc[gslot(d * 5 + v)];
+            g[d] = d2{mkf2(h.hi, h.lo), mkf2(l.hi, l.lo)};
+          }
+#pragma unroll
+          for (int jj = 0; jj < 3; ++jj) {
+            const d2 r = dot3(sj[jj], g[0], sj[3 + jj], g[1], sj[6 + jj], g[2]);
+            du[jj] = lane0(r);
+            dc[jj] = lane1(r);
+          }
+        } else {
+          TG gu[3], gc[3];
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            gu[d] = sG[(d * 5 + v) * Np + m];
+            gc[d] = sGc[gslot(d * 5 + v)];
+          }
+#pragma unroll
+          for (int jj = 0; jj < 3; ++jj) {
+            du[jj] = dot3(sj[jj], gu[0], sj[3 + jj], gu[1], sj[6 + jj], gu[2]);
+            dc[jj] = dot3(sj[jj], gc[0], sj[3 + jj], gc[1], sj[6 + jj], gc[2]);
+          }
         }
 #pragma unroll
         for (int jj = 0; jj < 3; ++jj) {
-          const TG du = dot3(sj[jj], gu[0], sj[3 + jj], gu[1], sj[6 + jj], gu[2]);
-          const TG dc = dot3(sj[jj], gc[0], sj[3 + jj], gc[1], sj[6 + jj], gc[2]);
-          sGc[gslot(jj * 5 + v)] = dc;
+          sGc[gslot(jj * 5 + v)] = dc[jj];
           // Face-gradient source: BR2 the uncorrected gradient (+ eta r_f), LDG the corrected one.
-          sG[(jj * 5 + v) * Np + m] = dph.ldg ? dc : du;
+          sG[(jj * 5 + v) * Np + m] = dph.ldg ? dc[jj] : du[jj];
         }
       }
 #pragma unroll
@@ -571,26 +608,54 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
       TG lg[N];
 #pragma unroll
       for (int c = 0; c < N; ++c) lg[c] = to_g<TG>(l0[c]);
+      if constexpr (std::is_same<TG, df32>::value) {
+        // Double-float: the two ends are the lanes of packed instructions.
+        d2 lc[N];
+#pragma unroll
+        for (int c = 0; c < N; ++c) lc[c] = pack(lg[c], lg[N - 1 - c]);
+        const d2 lw = pack(lj[0], lj[S - 1]);
 #pragma unroll 1
-      for (int v = 0; v < 5; ++v) {
-        const TG *sg = sG + (jj * 5 + v) * Np + base;
-        TG x[N];
+        for (int v = 0; v < 5; ++v) {
+          const TG *sg = sG + (jj * 5 + v) * Np + base;
+          const d2 jump = pack(sdQ[(f0 * 5 + v) * Nf + r], sdQ[((f0 + 1) * 5 + v) * Nf + r]);
+          d2 x[N];
+          Bound<d2> bd;
 #pragma unroll
-        for (int c = 0; c < N; ++c) x[c] = sg[c * sd];
+          for (int c = 0; c < N; ++c) {
+            x[c] = dup(sg[c * sd]);
+            bd.add(lc[c], x[c]);
+          }
+          bd.add(lw, jump);
+          Acc<d2> acc(bd);
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-          // l(+1) is l(-1) mirrored.
-          auto l = [&](int c) { return s ? lg[N - 1 - c] : lg[c]; };
-          const TG jump = sdQ[((f0 + s) * 5 + v) * Nf + r];
-          Bound<TG> bd;
+          for (int c = 0; c < N; ++c) acc.add(lc[c], x[c]);
+          acc.add(lw, jump);
+          const d2 g = acc.raw();
+          dst[0][v * Nf] = lane0(g);
+          dst[S - 1][v * Nf] = lane1(g);
+        }
+      } else {
+#pragma unroll 1
+        for (int v = 0; v < 5; ++v) {
+          const TG *sg = sG + (jj * 5 + v) * Np + base;
+          TG x[N];
 #pragma unroll
-          for (int c = 0; c < N; ++c) bd.add(l(c), x[c]);
-          bd.add(lj[s], jump);
-          Acc<TG> acc(bd);
+          for (int c = 0; c < N; ++c) x[c] = sg[c * sd];
 #pragma unroll
-          for (int c = 0; c < N; ++c) acc.add(l(c), x[c]);
-          acc.add(lj[s], jump);
-          dst[s][v * Nf] = from_g<T>(acc.raw());
+          for (int s = 0; s < S; ++s) {
+            // l(+1) is l(-1) mirrored.
+            auto l = [&](int c) { return s ? lg[N - 1 - c] : lg[c]; };
+            const TG jump = sdQ[((f0 + s) * 5 + v) * Nf + r];
+            Bound<TG> bd;
+#pragma unroll
+            for (int c = 0; c < N; ++c) bd.add(l(c), x[c]);
+            bd.add(lj[s], jump);
+            Acc<TG> acc(bd);
+#pragma unroll
+            for (int c = 0; c < N; ++c) acc.add(l(c), x[c]);
+            acc.add(lj[s], jump);
+            dst[s][v * Nf] = from_g<T>(acc.raw());
+          }
         }
       }
     }

@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include "fr_bodies.cuh"
+#include "fr_pair.cuh"
 
 namespace frx {
 
@@ -65,6 +66,23 @@ __global__ void k_min_reduce(const double *__restrict__ x, int64_t n, double *__
 #define FR_EV_END(k) \
   if (ev) cudaEventRecord(ev->stop[k], st)
 
+// The packed volume kernel on this mesh's hexahedra, if it is the faster one (pair_pays); `done` says so.
+template <int N, bool FP32V, int VISC>
+static cudaError_t launch_pair(const DevMesh &m, const DevPhys &ph, cudaStream_t st, bool &done) {
+  if constexpr (pair_pays<N, FP32V, VISC>()) {
+    auto df = [](double *p) { return reinterpret_cast<df32 *>(p); };
+    auto pk = k_volume_pair<N, FP32V, VISC>;
+    constexpr int smem = pair_smem<N, FP32V, VISC>();
+    cudaError_t err = cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (err != cudaSuccess) return err;
+    pk<<<(unsigned)((m.E + 1) / 2), volume_threads<N>(), smem, st>>>(df(m.Qc), df(m.metrics), m.ef, df(m.Qtr),
+                                                                    df(m.liftfac), df(m.Gtr), df(m.Rpart), ph, m.if_up,
+                                                                    m.n_interior, m.E);
+    done = true;
+  }
+  return cudaSuccess;
+}
+
 template <int N, typename T>
 static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, int stage, double dt,
                                  double *Rout, cudaStream_t st, const PhaseEvents *ev, int phases) {
@@ -116,8 +134,17 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
     if (E > 0 && ph.vc_basis) {
       if ((err = launch_vcjh_phase(m, ph, 1, mode, stage, dt, Rout, st)) != cudaSuccess) return err;
     } else if (E > 0) {
-      kern<<<(unsigned)((E + volume_epb<N>() - 1) / volume_epb<N>()), volume_block<N>(), smem, st>>>(
-          Qin, met, m.ef, Qtr, lift, Gtr, Rpart, ph, m.h, m.nu, m.if_up, m.n_interior, E);
+      // The closure's features need the whole element in one block's warps: scalar kernel.
+      bool done = false;
+      if constexpr (std::is_same<T, df32>::value)
+        if (!ph.closure) {
+          err = !ph.viscous ? launch_pair<N, false, 0>(m, ph, st, done)
+                            : (m.vf32 ? launch_pair<N, true, 1>(m, ph, st, done) : launch_pair<N, false, 1>(m, ph, st, done));
+          if (err != cudaSuccess) return err;
+        }
+      if (!done)
+        kern<<<(unsigned)((E + volume_epb<N>() - 1) / volume_epb<N>()), volume_block<N>(), smem, st>>>(
+            Qin, met, m.ef, Qtr, lift, Gtr, Rpart, ph, m.h, m.nu, m.if_up, m.n_interior, E);
     }
     if ((err = launch_prism_phase(m, ph, 1, mode, stage, dt, Rout, st)) != cudaSuccess) return err;
     FR_EV_END(1);

@@ -1,0 +1,269 @@
+// Hexahedral volume kernel with two elements per thread, in packed double-float (or FP32) arithmetic.
+//
+// With two elements per thread the loads, addresses and loop overhead, a quarter of the scalar kernel's
+// instructions, fill the issue slots that the packed arithmetic (fr_f32x2.cuh) leaves.
+#pragma once
+
+#include "fr_bodies.cuh"
+
+namespace frx {
+namespace {
+
+// Arithmetic of the viscous branch: pairs of double-float values, or of FP32 (FR_PREC_MIXED_VF32).
+template <typename TG> __device__ __forceinline__ TG to_pg(d2 x);
+template <> __device__ __forceinline__ d2 to_pg<d2>(d2 x) { return x; }
+template <> __device__ __forceinline__ f2 to_pg<f2>(d2 x) { return padd(x.hi, x.lo); }
+__device__ __forceinline__ d2 from_pg(d2 x) { return x; }
+__device__ __forceinline__ d2 from_pg(f2 x) { return d2{x, dupf(0.f)}; }
+template <typename TG> __device__ __forceinline__ TG dup_g(df32 x) { return to_pg<TG>(dup(x)); }
+
+template <typename TG>
+__device__ __forceinline__ PhysT<TG> pair_phys(const PhysT<df32> &p) {
+  PhysT<TG> r;
+  r.cT = dup_g<TG>(p.cT);
+  r.mu = dup_g<TG>(p.mu);
+  r.m2mu3 = dup_g<TG>(p.m2mu3);
+  r.kappa = dup_g<TG>(p.kappa);
+  return r;
+}
+
+// Bytes of shared memory per pair of elements: state perturbation 5, gradient 15 and flux 15 per point, jumps 30
+// per N^2; an inviscid run keeps the flux only.
+template <int N, bool FP32V, int VISC>
+constexpr int pair_smem() {
+  constexpr int Np = N * N * N, Nf = N * N, G = FP32V ? 8 : 16;
+  return VISC ? 20 * Np * G + 15 * Np * 16 + 30 * Nf * G : 15 * Np * 16;
+}
+template <int N, bool FP32V, int VISC>
+constexpr int pair_blocks() {
+  // By shared memory (227 KB per SM), and not below 128 registers per thread.
+  constexpr int by_smem = 227 * 1024 / (pair_smem<N, FP32V, VISC>() + 1024);
+  constexpr int by_regs = 512 / volume_threads<N>();
+  return by_smem < by_regs ? by_smem : (by_regs > 0 ? by_regs : 1);
+}
+
+// Where it runs, and what the volume kernel takes per launch against the scalar one (GB300).  It halves the
+// warps of an SM for the same shared memory, so it gains where enough of them remain: FP32 viscous branch
+// 40^3 p = 3 0.623 -> 0.572 ms, 32^3 p = 4 0.643 -> 0.600, 28^3 p = 5 0.844 -> 0.740, 20^3 p = 7 0.937 -> 0.842
+// (not p = 2: 0.324 -> 0.331, p = 6: 0.912 -> 0.946); double-float 40^3 p = 2 0.463 -> 0.449, p = 3 0.985 -> 0.946
+// (not 48^3 p = 4: 3.09 -> 3.51 with 8 warps per SM, 3.21 with 12 at less shared memory); inviscid 40^3 p = 2
+// 0.097 -> 0.087, p = 3 0.210 -> 0.191, 32^3 p = 4 0.244 -> 0.231.
+template <int N, bool FP32V, int VISC>
+constexpr bool pair_pays() {
+  return VISC == 0 ? (!FP32V && N >= 3 && N <= 5) : (FP32V ? (N == 4 || N == 5 || N == 6 || N == 8) : (N == 3 || N == 4));
+}
+
+// One thread per solution point of the elements e0 and e1; the operations of volume_body in its order.  An odd
+// mesh's last block holds one element twice: both lanes then store the same values.
+template <int N, bool FP32V, int VISC>
+__global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VISC>())
+    k_volume_pair(const df32 *__restrict__ Q, const df32 *__restrict__ metrics, const int32_t *__restrict__ ef,
+                  const df32 *__restrict__ Qtr, const df32 *__restrict__ liftfac, df32 *__restrict__ Gtr,
+                  df32 *__restrict__ Rpart, DevPhys dph, const int8_t *__restrict__ if_up, int64_t n_interior, int64_t E) {
+  extern __shared__ float4 sm_pair[];
+  constexpr int Np = N * N * N, Nf = N * N, nth = volume_threads<N>();
+  using TG = typename std::conditional<FP32V, f2, d2>::type;
+  d2 *sH = reinterpret_cast<d2 *>(sm_pair);                    // [15][Np] transformed flux, index d*5+v
+  TG *sQ = reinterpret_cast<TG *>(sH + 15 * Np);               // [5][Np] perturbation from the first point
+  TG *sG = sQ + 5 * Np;                                        // [15][Np] uncorrected gradient, j*5+v
+  TG *sdQ = sG + 15 * Np;                                      // [6][5][Nf] Q^I - Q_own at the flux points
+  const int64_t e0 = (int64_t)blockIdx.x * 2, e1 = e0 + 1 < E ? e0 + 1 : e0;
+  const int tid = threadIdx.x;
+  const BasisT<df32> &B = cbasis<df32>(N);
+  const bool pt = tid < Np;
+  const int m = pt ? tid : 0, i = m % N, j = (m / N) % N, k = m / (N * N);
+  const df32 *Q0 = Q + e0 * Np * 5, *Q1 = Q + e1 * Np * 5;
+  d2 S[9], invJ, q[5];
+  if (pt) {
+    const df32 *m0 = metrics + e0 * 10 * Np + m, *m1 = metrics + e1 * 10 * Np + m;
+#pragma unroll
+    for (int c = 0; c < 9; ++c) S[c] = pack(m0[c * Np], m1[c * Np]);
+    invJ = pack(m0[9 * Np], m1[9 * Np]);
+  }
+  if constexpr (VISC != 0) {
+    for (int t = tid; t < 5 * Np; t += nth)
+      sQ[(t % 5) * Np + t / 5] = to_pg<TG>(pack(Q0[t], Q1[t]) - pack(Q0[t % 5], Q1[t % 5]));
+    for (int t = tid; t < 6 * Nf; t += nth) {
+      const int f = t / Nf, r = t % Nf;
+      const df32 *own[2], *oth[2];
+      float w[2];
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        const int packed = ef[(l ? e1 : e0) * 6 + f];
+        const int64_t I = packed >> 4;
+        const int side = (packed >> 3) & 1, slot = slot_of(packed & 7, r % N, r / N, N);
+        own[l] = Qtr + (I * 2 + side) * 5 * Nf + slot;
+        oth[l] = Qtr + (I * 2 + (1 - side)) * 5 * Nf + slot;
+        w[l] = 0.5f;
+        if (dph.ldg && I < n_interior) w[l] = side == (if_up[I] ? 0 : 1) ? 0.f : 1.f;
+      }
+#pragma unroll
+      for (int v = 0; v < 5; ++v)
+        sdQ[(f * 5 + v) * Nf + r] = to_pg<TG>(scale2(
+            pack(oth[0][v * Nf], oth[1][v * Nf]) - pack(own[0][v * Nf], own[1][v * Nf]), mkf2(w[0], w[1])));
+    }
+  }
+  __syncthreads();
+  TG G[15];
+  if (pt) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) q[v] = pack(Q0[m * 5 + v], Q1[m * 5 + v]);
+    if constexpr (VISC != 0) {
+      TG sj[9];   // S[d][jj] / |J|
+#pragma unroll
+      for (int c = 0; c < 9; ++c) sj[c] = to_pg<TG>(S[c] * invJ);
+      constexpr int R = sizeof(d2) / sizeof(TG);
+      TG *sGc = reinterpret_cast<TG *>(sH);
+      auto gslot = [&](int c) { return ((c / R) * Np + m) * R + c % R; };
+#pragma unroll 1
+      for (int d = 0; d < 3; ++d) {
+        const int row = d == 0 ? i : (d == 1 ? j : k), st = axis_stride<N>(d), at = m - row * st;
+        const int r = d == 0 ? j + N * k : (d == 1 ? i + N * k : i + N * j);
+        TG c[N];
+#pragma unroll
+        for (int a = 0; a < N; ++a) c[a] = dup_g<TG>(B.D[row * N + a]);
+        const TG hlo = -dup_g<TG>(B.hm[row]), hhi = dup_g<TG>(B.hp[row]);
+        const TG *dq = sdQ + d * 10 * Nf + r;
+#pragma unroll 1
+        for (int v = 0; v < 5; ++v) {
+          const TG jlo = dq[v * Nf], jhi = dq[(5 + v) * Nf];
+          TG x[N];
+          Bound<TG> bd;
+#pragma unroll
+          for (int a = 0; a < N; ++a) {
+            x[a] = sQ[v * Np + at + a * st];
+            bd.add(c[a], x[a]);
+          }
+          bd.add(hlo, jlo);
+          bd.add(hhi, jhi);
+          Acc<TG> s(bd);
+#pragma unroll
+          for (int a = 0; a < N; ++a) s.add(c[a], x[a]);
+          sG[(d * 5 + v) * Np + m] = s.raw();
+          s.add(hlo, jlo);
+          s.add(hhi, jhi);
+          sGc[gslot(d * 5 + v)] = s.raw();
+        }
+      }
+#pragma unroll 1
+      for (int v = 0; v < 5; ++v) {
+        TG gu[3], gc[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          gu[d] = sG[(d * 5 + v) * Np + m];
+          gc[d] = sGc[gslot(d * 5 + v)];
+        }
+#pragma unroll
+        for (int jj = 0; jj < 3; ++jj) {
+          const TG du = dot3(sj[jj], gu[0], sj[3 + jj], gu[1], sj[6 + jj], gu[2]);
+          const TG dc = dot3(sj[jj], gc[0], sj[3 + jj], gc[1], sj[6 + jj], gc[2]);
+          sGc[gslot(jj * 5 + v)] = dc;
+          // Face-gradient source: BR2 the uncorrected gradient (+ eta r_f), LDG the corrected one.
+          sG[(jj * 5 + v) * Np + m] = dph.ldg ? dc : du;
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 15; ++c) G[c] = sGc[gslot(c)];
+    }
+    const d2 ri = reciprocal(q[0]);
+    const d2 u[3] = {q[1] * ri, q[2] * ri, q[3] * ri};
+    const d2 p = dup(dph.f.gm1) * (q[4] - scale2(dot3(q[1], u[0], q[2], u[1], q[3], u[2]), 0.5f));
+    d2 tau[6], hq[3], mom[6], en[3];
+    if constexpr (VISC != 0) {
+      const PhysT<TG> pg = pair_phys<TG>(dph.f);
+      TG qg[5], ug[3], taug[6], hqg[3], rig;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) qg[v] = to_pg<TG>(q[v]);
+      if constexpr (FP32V) {
+        rig = reciprocal(qg[0]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) ug[c] = qg[1 + c] * rig;
+      } else {
+        rig = ri;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) ug[c] = u[c];
+      }
+      viscous_stress<TG>(qg, ug, rig, G, pg, visc_of(pg), taug, hqg);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) hq[a] = from_pg(hqg[a]);
+#pragma unroll
+      for (int a = 0; a < 6; ++a) tau[a] = from_pg(taug[a]);
+    }
+    physical_flux<d2>(q, u, p, VISC != 0, tau, hq, mom, en);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      d2 f[5];
+      transformed_flux<d2>(q, mom, en, S + 3 * d, f);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
+    }
+  }
+  __syncthreads();
+  if constexpr (VISC != 0) {
+    for (int t = tid; t < 9 * Nf; t += nth) {
+      const int jj = t / (3 * Nf), dr = t - jj * 3 * Nf;
+      const int d = dr / Nf, r = dr % Nf;
+      int base, sd;
+      face_line<N>(2 * d, r, base, sd);
+      df32 *dst[2][2];
+      TG lj[2];
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        const int f = 2 * d + s;
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+          const int packed = ef[(l ? e1 : e0) * 6 + f];
+          const int64_t I = packed >> 4;
+          dst[s][l] = Gtr + (I * 2 + ((packed >> 3) & 1)) * 15 * Nf + slot_of(packed & 7, r % N, r / N, N) + jj * 5 * Nf;
+        }
+        lj[s] = to_pg<TG>(dup(dph.f.eta) *
+                          pack(liftfac[((e0 * 6 + f) * 3 + jj) * Nf + r], liftfac[((e1 * 6 + f) * 3 + jj) * Nf + r]));
+      }
+#pragma unroll 1
+      for (int v = 0; v < 5; ++v) {
+        const TG *sg = sG + (jj * 5 + v) * Np + base;
+        TG x[N];
+#pragma unroll
+        for (int c = 0; c < N; ++c) x[c] = sg[c * sd];
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          auto l = [&](int c) { return dup_g<TG>(s ? B.lp[c] : B.lm[c]); };
+          const TG jump = sdQ[((2 * d + s) * 5 + v) * Nf + r];
+          Bound<TG> bd;
+#pragma unroll
+          for (int c = 0; c < N; ++c) bd.add(l(c), x[c]);
+          bd.add(lj[s], jump);
+          Acc<TG> acc(bd);
+#pragma unroll
+          for (int c = 0; c < N; ++c) acc.add(l(c), x[c]);
+          acc.add(lj[s], jump);
+          const d2 g = from_pg(acc.raw());
+          dst[s][0][v * Nf] = lane0(g);
+          dst[s][1][v * Nf] = lane1(g);
+        }
+      }
+    }
+  }
+  if (pt) {
+    df32 *out0 = Rpart + (e0 * Np + m) * 5, *out1 = Rpart + (e1 * Np + m) * 5;
+#pragma unroll 1
+    for (int v = 0; v < 5; ++v) {
+      const d2 *h0 = sH + (0 * 5 + v) * Np, *h1 = sH + (1 * 5 + v) * Np, *h2 = sH + (2 * 5 + v) * Np;
+      Dot<d2> acc(dup(B.Dt[i * N]), h0[N * j + N * N * k]);
+      acc.add(dup(B.Dt[j * N]), h1[i + N * N * k]);
+      acc.add(dup(B.Dt[k * N]), h2[i + N * j]);
+#pragma unroll
+      for (int a = 1; a < N; ++a) {
+        acc.add(dup(B.Dt[i * N + a]), h0[a + N * j + N * N * k]);
+        acc.add(dup(B.Dt[j * N + a]), h1[i + N * a + N * N * k]);
+        acc.add(dup(B.Dt[k * N + a]), h2[i + N * j + N * N * a]);
+      }
+      const d2 o = acc.raw();
+      out0[v] = lane0(o);
+      out1[v] = lane1(o);
+    }
+  }
+}
+
+}  // namespace
+}  // namespace frx
