@@ -311,7 +311,8 @@ __host__ __device__ constexpr int closure_floats() { return 10 * N * N * N + 1 +
 // thread of the block calls this together (it contains block barriers); inactive sub-blocks
 // (active = false) only take part in the barriers.
 // VISC: 1 viscous, 0 inviscid (only the transformed flux lives in shared memory), 2 decided at run time.
-template <int N, typename T, bool VC, bool FP32V, int VISC>
+// SPLIT: five groups of volume_threads<N>() threads, one per variable in the gradient and the divergence.
+template <int N, typename T, bool VC, bool FP32V, int VISC, bool SPLIT = false>
 __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool active, double *sm_raw,
                                             const T *__restrict__ Q, const T *__restrict__ metrics,
                                             const int32_t *__restrict__ ef, const T *__restrict__ Qtr,
@@ -349,11 +350,13 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   // products and paired traces took the double-float kernel from 8860 to 7540 instructions per
   // warp, 4.375 -> 3.80 ms per launch at 48^3 p = 4, 1.34 -> 1.18 ms at 40^3 p = 3, errors unchanged.
   const bool viscous = VISC == 2 ? dph.viscous != 0 : VISC == 1;
-  const bool pt = active && tid < Np;
-  const int m = tid < Np ? tid : 0, i = m % N, j = (m / N) % N, k = m / (N * N);
+  const int grp = SPLIT ? tid / volume_threads<N>() : 0, tp = SPLIT ? tid % volume_threads<N>() : tid;
+  const int v0 = SPLIT ? grp : 0, v1 = SPLIT ? grp + 1 : 5;     // this thread's variables
+  const bool mine = active && tp < Np, pt = mine && grp == 0;
+  const int m = tp < Np ? tp : 0, i = m % N, j = (m / N) % N, k = m / (N * N);
   // The point's metric terms are loaded before the staging loops so that their latency overlaps them.
   T S[9], invJ, q[5];
-  if (pt) {
+  if (mine) {
     const T *met = metrics + e * 10 * Np + m;
 #pragma unroll
     for (int c = 0; c < 9; ++c) S[c] = met[c * Np];
@@ -388,9 +391,16 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   }
   __syncthreads();
   TG G[15];
-  if (pt) {
+  // The reference gradient, uncorrected and corrected, goes through shared memory, in this thread's own
+  // entries of the gradient and transformed-flux buffers, which only this thread writes before the next
+  // barrier (R gradient values of type TG per entry of type T).
+  constexpr int R = sizeof(T) / sizeof(TG);
+  TG *sGc = reinterpret_cast<TG *>(sH);
+  auto gslot = [&](int c) { return ((c / R) * Np + m) * R + c % R; };
+  if (mine) {
+    if (pt)
 #pragma unroll
-    for (int v = 0; v < 5; ++v) q[v] = kPertDf ? Q[(e * Np + m) * 5 + v] : sQ[v * Np + m];
+      for (int v = 0; v < 5; ++v) q[v] = kPertDf ? Q[(e * Np + m) * 5 + v] : sQ[v * Np + m];
     if (viscous) {
       // S[d][jj] / |J|.  Double-float transforms the uncorrected and the corrected gradient as the two lanes
       // of packed instructions (their parts wait in shared memory lane by lane: (hi, hi) in sG, (lo, lo) in sGc).
@@ -403,12 +413,6 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
         else
           sj[c] = to_g<TG>(S[c] * invJ);
       }
-      // The reference gradient, uncorrected and corrected, goes through shared memory, in this thread's
-      // own entries of the gradient and transformed-flux buffers, which only this thread writes before
-      // the next barrier (R gradient values of type TG per entry of type T).
-      constexpr int R = sizeof(T) / sizeof(TG);
-      TG *sGc = reinterpret_cast<TG *>(sH);
-      auto gslot = [&](int c) { return ((c / R) * Np + m) * R + c % R; };
       const TG *sq;
       if constexpr (kPert)
         sq = sQg;
@@ -430,7 +434,7 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
         const TG hlo = -to_g<TG>(B.hm[row]), hhi = to_g<TG>(B.hp[row]);
         const TG *dq = sdQ + d * 10 * Nf + r;
 #pragma unroll(N == 8 ? 5 : 1)
-        for (int v = 0; v < 5; ++v) {
+        for (int v = v0; v < v1; ++v) {
           // Derivative along the point's line, then the two faces' correction added to the same sum.
           const TG jlo = dq[v * Nf], jhi = dq[(5 + v) * Nf];
           TG x[N];
@@ -459,7 +463,7 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
         }
       }
 #pragma unroll 1
-      for (int v = 0; v < 5; ++v) {
+      for (int v = v0; v < v1; ++v) {
         TG du[3], dc[3];
         if constexpr (kPack) {
           d2 g[3];
@@ -494,9 +498,16 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
           sG[(jj * 5 + v) * Np + m] = dph.ldg ? dc[jj] : du[jj];
         }
       }
+      if constexpr (!SPLIT)
+#pragma unroll
+        for (int c = 0; c < 15; ++c) G[c] = sGc[gslot(c)];
+    }
+  }
+  if constexpr (SPLIT) {
+    __syncthreads();
+    if (pt)
 #pragma unroll
       for (int c = 0; c < 15; ++c) G[c] = sGc[gslot(c)];
-    }
   }
   T rho_nu = ph.zero;
   if (viscous && dph.closure) {
@@ -660,11 +671,10 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
       }
     }
   }
-  if (active && tid < Np) {
-    const int m = tid, i = m % N, j = (m / N) % N, k = m / (N * N);
+  if (mine) {
     T *out = Rpart + (e * Np + m) * 5;
 #pragma unroll 1
-    for (int v = 0; v < 5; ++v) {
+    for (int v = v0; v < v1; ++v) {
       const T *h0 = sH + (0 * 5 + v) * Np, *h1 = sH + (1 * 5 + v) * Np, *h2 = sH + (2 * 5 + v) * Np;
       Dot<T> acc(B.Dt[i * N], h0[N * j + N * N * k]);
       acc.add(B.Dt[j * N], h1[i + N * N * k]);
@@ -715,6 +725,30 @@ template <int N, typename T>
 size_t volume_smem(bool viscous, bool closure) {
   return volume_epb<N>() * (viscous ? sizeof(T) * volume_smem_values<N>() + (closure ? sizeof(float) * closure_floats<N>() : 0)
                                     : sizeof(T) * 15 * N * N * N);
+}
+
+// Few elements: five groups of threads per element, one per variable in the gradient and the divergence (one of
+// them also forms the fluxes).  With one or two elements per SM the kernel above is a chain of one warp's
+// instructions (an FP64 one issues every 64 cycles per scheduler, and the other schedulers idle): FP64
+// 64 elements at p = 2 28.8 -> 16.4 us per launch, 125 at p = 3 29.3 -> 18.6, 125 at p = 4 30.7 -> 26.6;
+// double-float 64 at p = 2 18.5 -> 10.4, 216 at p = 3 18.5 -> 12.3, 64 at p = 4 14.8 -> 14.5.  Limits: where the SMs
+// fill up it costs an extra barrier and the four groups' idle time at the fluxes (FP64 p = 2 18.7 against
+// 28.7 us at 216 elements but 34.3 against 29.2 at 512, p = 3 25.0 against 30.0 and 44.6 against 41.5, p = 4
+// 47.5 against 43.6 at 216), so two elements per SM at p = 2 and 3 and one at p = 4.  p = 1 puts 16 elements in
+// a block, p >= 5 has seven and more warps per element anyway.
+template <int N>
+constexpr int64_t volume_split_max() { return N == 3 || N == 4 ? 2 * 152 : (N == 5 ? 152 : 0); }
+
+template <int N, typename T, bool FP32V>
+__global__ void __launch_bounds__(5 * volume_threads<N>())
+    k_volume_split(const T *__restrict__ Q, const T *__restrict__ metrics, const int32_t *__restrict__ ef,
+                   const T *__restrict__ Qtr, const T *__restrict__ liftfac, T *__restrict__ Gtr, T *__restrict__ Rpart,
+                   DevPhys dph, const double *__restrict__ hel, float *__restrict__ nu_out,
+                   const int8_t *__restrict__ if_up, int64_t n_interior) {
+  extern __shared__ double sm_raw[];
+  const ClosureSpace cs{reinterpret_cast<float *>(sm_raw + volume_smem_values<N>()), blockIdx.x, 1, 0};
+  volume_body<N, T, false, FP32V, 1, true>(blockIdx.x, threadIdx.x, 5 * volume_threads<N>(), true, sm_raw, Q, metrics, ef,
+                                           Qtr, liftfac, Gtr, Rpart, dph, hel, nu_out, if_up, n_interior, cs);
 }
 
 template <int N, typename T, bool FP32V, int VISC>
@@ -1020,8 +1054,8 @@ __device__ __forceinline__ void correct_lift(int64_t e, int m, const T *__restri
   }
 }
 
-// Thread per point (batched stage).
-template <int N, typename T>
+// Thread per point (small meshes and the batched stage).
+template <int N, typename T, bool VC = false>
 __device__ __forceinline__ void correct_body(int64_t t, const T *__restrict__ Rpart, const T *__restrict__ FI,
                                              const int32_t *__restrict__ ef, const T *__restrict__ metrics,
                                              int64_t E, const StageCoef &sc, double *__restrict__ Rout,
@@ -1033,7 +1067,7 @@ __device__ __forceinline__ void correct_body(int64_t t, const T *__restrict__ Rp
   const int64_t e = t / Np;
   const int m = (int)(t % Np);
   Dot<T> r[5];
-  correct_lift<N, T, false>(e, m, FI, ef, dph, kGatherFirst<T> ? nullptr : Rpart + t * 5, r);
+  correct_lift<N, T, VC>(e, m, FI, ef, dph, kGatherFirst<T> ? nullptr : Rpart + t * 5, r);
   T rv[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
@@ -1041,6 +1075,22 @@ __device__ __forceinline__ void correct_body(int64_t t, const T *__restrict__ Rp
     rv[v] = r[v].get();
   }
   finish_point<T>(t, rv, -metrics[(e * 10 + 9) * Np + m], sc, Rout, Q, Qc, Un, Unc, acc, flag, dph);
+}
+
+// Up to 256 points per SM (one block of the kernel below on each): one thread per point in blocks of one
+// warp, which spreads the chain of loads and FP64 instructions over more schedulers and has no
+// staging barriers.  FP64 8^3 p = 3 12.6 -> 10.6 us per launch, 4^3 p = 2 10.4 -> 8.6, double-float 8^3 p = 3 10.9 -> 9.3;
+// at 64000 points 14.4 against 14.7 us, and at 32^3 p = 4 0.398 ms staged against 0.431.
+constexpr int64_t kCorrectPointMax = 152 * 256;
+
+template <int N, typename T>
+__global__ void __launch_bounds__(32)
+    k_correct_point(const T *__restrict__ Rpart, const T *__restrict__ FI, const int32_t *__restrict__ ef,
+                    const T *__restrict__ metrics, int64_t E, StageCoef sc, double *__restrict__ Rout,
+                    double *__restrict__ Q, T *__restrict__ Qc, double *__restrict__ Un, T *__restrict__ Unc,
+                    double *__restrict__ acc, int *__restrict__ flag, DevPhys dph) {
+  correct_body<N, T>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, Rpart, FI, ef, metrics, E, sc, Rout, Q, Qc, Un, Unc,
+                     acc, flag, dph);
 }
 
 template <int N, typename T, bool VC, bool SRC>

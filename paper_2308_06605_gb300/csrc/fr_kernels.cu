@@ -136,8 +136,19 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
     } else if (E > 0) {
       // The closure's features need the whole element in one block's warps: scalar kernel.
       bool done = false;
+      if constexpr (volume_split_max<N>() > 0)
+        if (ph.viscous && E <= volume_split_max<N>()) {
+          auto sk = k_volume_split<N, T, false>;
+          if constexpr (std::is_same<T, df32>::value)
+            if (m.vf32) sk = k_volume_split<N, T, true>;
+          err = cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+          if (err != cudaSuccess) return err;
+          sk<<<(unsigned)E, 5 * volume_threads<N>(), smem, st>>>(Qin, met, m.ef, Qtr, lift, Gtr, Rpart, ph, m.h, m.nu,
+                                                                 m.if_up, m.n_interior);
+          done = true;
+        }
       if constexpr (std::is_same<T, df32>::value)
-        if (!ph.closure) {
+        if (!done && !ph.closure) {
           err = !ph.viscous ? launch_pair<N, false, 0>(m, ph, st, done)
                             : (m.vf32 ? launch_pair<N, true, 1>(m, ph, st, done) : launch_pair<N, false, 1>(m, ph, st, done));
           if (err != cudaSuccess) return err;
@@ -179,6 +190,10 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
     FR_EV_BEGIN(3);
     if (n > 0 && ph.vc_basis) {
       if ((err = launch_vcjh_phase(m, ph, 3, mode, stage, dt, Rout, st)) != cudaSuccess) return err;
+    } else if (n > 0 && n <= kCorrectPointMax) {
+      k_correct_point<N, T><<<(unsigned)((n + 31) / 32), 32, 0, st>>>(
+          Rpart, FI, m.ef, met, E, stage_coef(mode, stage, dt), Rout, m.Q, Qc, m.Un, reinterpret_cast<T *>(m.Unc), m.acc,
+          m.flag, ph);
     } else if (n > 0) {
       auto ck = has_source(ph) ? k_correct<N, T, false, true> : k_correct<N, T, false, false>;
       ck<<<(unsigned)((n + kCorrectThreads - 1) / kCorrectThreads), kCorrectThreads, correct_smem(ph), st>>>(

@@ -7,7 +7,8 @@ element fewer and more than a full block, viscous and inviscid, at the suite's b
 double-float 1e-9, FP32 viscous branch 2e-8 of the magnitude scale at Re 400).  Odd element counts leave the
 packed volume kernel's last block with one element.  Closure training (32 samples per block, at most 304 blocks,
 partial rows limited by the workspace): loss and gradient at the suite's FP32 bars.  Order projection
-with the most elements per block, 1e-13."""
+with the most elements per block, 1e-13.  Meshes just below and above the sizes where the kernels for few
+elements or points give way to the full ones."""
 import numpy as np
 import pytest
 
@@ -15,7 +16,9 @@ from paper_2308_06605_gb300 import fr
 from paper_2308_06605_gb300 import inputs as I
 from oracle import mlp
 from oracle import project as PJ
+from oracle import timeint as TI
 from oracle.hexfr import HexFR
+from oracle.mixedfr import MixedFR
 
 from helpers import assert_residual_parity, assert_state_parity, ensure_lib
 
@@ -105,3 +108,39 @@ def test_one_mesh_twice_in_a_batch_keeps_its_order():
             m.rk_stage(s, 0.0, 1e-3)
         want = m.get_state()
     assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], want)
+
+
+def _flat(arrs):
+    return np.concatenate([np.asarray(a).reshape(-1, 5) for a in arrs])
+
+
+# Element counts at the limits of the volume kernel that splits an element's variables over thread groups (304 at
+# p = 2 and 3, 152 at p = 4) and of the correction kernel with one thread per point (38912 points).
+@pytest.mark.parametrize("p,box", [(1, (17, 17, 17)), (2, (19, 4, 4)), (2, (61, 5, 1)), (2, (12, 12, 11)),
+                                   (3, (19, 4, 4)), (3, (61, 5, 1)), (3, (19, 8, 4)), (3, (29, 7, 3)), (4, (19, 4, 2)),
+                                   (4, (17, 3, 3)), (4, (13, 6, 4)), (5, (8, 6, 4)), (6, (5, 5, 5)), (7, (5, 4, 4))])
+def test_small_mesh_limits(p, box):
+    d = I.hex_box_mesh(box, seed=6, rotate=True, affine=((1.0, 0.2, 0.0), (0.0, 1.0, 0.1), (0.1, 0.0, 1.0)))
+    ph = I.tgv_physics(Ma=0.2, Re=400.0)
+    ora = MixedFR(d, ph, p)
+    Qs = [np.ascontiguousarray(I.tgv_state(x, Ma=0.2, perturb=1e-2, seed=1)) for x in ora.x]
+    R, S, dt = _flat(ora.residual(Qs)), _flat(ora.residual(Qs, magnitude=True)), 2e-5
+    ora.set_source(accel=(0.3, -0.2, 0.1))
+    S1 = _flat(ora.residual(Qs, magnitude=True))
+    want = [_flat(TI.rk44(ora.residual, Qs, dt))]
+    if p == 3:
+        want.append(_flat(TI.SCHEMES["ssprk33"](ora.residual, Qs, dt)))
+    for precision, bar in [(fr.FR_PREC_FP64, 1e-12), (fr.FR_PREC_MIXED, 1e-9), (fr.FR_PREC_MIXED_VF32, 2e-8)]:
+        ph.precision = precision
+        with fr.Mesh(d, ph, p) as g:
+            g.set_state(_flat(Qs))
+            got = g.residual().reshape(-1, 5)
+            if precision == fr.FR_PREC_MIXED_VF32:      # thin cells are mostly viscous: the suite's normwise bar
+                assert (np.abs(got - R).max(axis=0) <= 1e-6 * np.abs(R).max(axis=0)).all()
+            else:
+                assert_residual_parity(got, R, S, bar)
+            g.set_source(accel=(0.3, -0.2, 0.1))
+            for scheme, w in zip((fr.FR_RK44, fr.FR_SSPRK33), want):
+                g.set_state(_flat(Qs))
+                g.rk_step(0.0, dt, scheme)
+                assert_state_parity(g.get_state().reshape(-1, 5), w, S1, dt, bar)
