@@ -457,7 +457,7 @@ __device__ __forceinline__ void finish_point(int64_t t, const T rv[5], T s, cons
 // The copies into shared memory (cp.async: partial residual and the stage's two old register values) are in
 // flight while the double-float kernel gathers the fluxes.  Double-float 48^3 p = 4 1.07 -> 0.80 ms per launch
 // (0.93 with the partial residual alone staged by plain loads), FP64 32^3 p = 4 0.447 -> 0.398 ms; bound by the
-// FP64 pipe (two conversions, an addition and an FMA per value) beside 3.5 GB of traffic (0.51 ms at
+// FP64 pipe (an addition and an FMA per value, the last stage a split into double-float) beside 3.5 GB of traffic (0.51 ms at
 // 48^3).  FP64 6 blocks per SM (40 registers), double-float 5 (48; 6 measured the same).
 constexpr int kCorrectThreads = 256;
 

@@ -144,3 +144,24 @@ def test_small_mesh_limits(p, box):
                 g.set_state(_flat(Qs))
                 g.rk_step(0.0, dt, scheme)
                 assert_state_parity(g.get_state().reshape(-1, 5), w, S1, dt, bar)
+
+
+@pytest.mark.parametrize("flux", [0, 1])
+def test_zero_and_subnormal_values(flux):
+    """Double-float values that the integer conversion to FP64 leaves to the instruction: zeros and FP32 subnormals."""
+    d = I.hex_box_mesh((4, 3, 3), seed=2, rotate=True, perturb=0.1)
+    ph = I.tgv_physics(Ma=0.2, Re=400.0)
+    ph.inviscid_flux = flux
+    ora = HexFR(d, ph, 3)
+    Q = np.ascontiguousarray(I.tgv_state(ora.x, Ma=0.2, perturb=1e-2, seed=1))
+    Q[:, ::3, 1:4] = (0.0, 1e-39, -3e-42)
+    Q[:, 1::3, 0] = np.float32(1.25)
+    S, dt = ora.residual(Q, magnitude=True), 1e-4
+    ph.precision = fr.FR_PREC_MIXED
+    with fr.Mesh(d, ph, 3) as g:
+        g.set_state(Q)
+        assert_residual_parity(g.residual(), ora.residual(Q), S, 1e-9)
+        for scheme, f in ((fr.FR_RK44, TI.rk44), (fr.FR_SSPRK33, TI.SCHEMES["ssprk33"])):
+            g.set_state(Q)
+            g.rk_step(0.0, dt, scheme)
+            assert_state_parity(g.get_state(), f(lambda q: [ora.residual(q[0])], [Q], dt)[0], S, dt, 1e-9)
