@@ -189,7 +189,7 @@ static cudaError_t enqueue_stage(fr_batch *b, int stage) {
 // (points).  One case's four kernels depend on one another and leave the GPU partly idle at every launch's
 // start and end; cases do not depend on each other.  A mesh that is listed twice keeps the serial order.
 // 16 vortex cases (9.2 M points, double-float, states set and read): 8.84 ms per step with one branch,
-// 7.61 with four, 7.63 with eight.
+// 7.61 with four, 7.63 with eight; 6.72 with four since to_double runs on the integer pipe.
 static cudaError_t make_branches(fr_batch *b) {
   std::vector<int> order(b->cases.size());
   for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;

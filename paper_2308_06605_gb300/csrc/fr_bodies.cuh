@@ -346,7 +346,7 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   // from 3.8e-10 to 1.2e-9 (TGV 40^3, p = 3, Ma 0.1) for 3 % of the kernel's time.  Transform and traces use
   // packed instructions in double-float (48^3 p = 4 3.09 -> 3.00 ms, 28^3 p = 5 1.174 -> 1.154, but 24^3 p = 6 1.30 ->
   // 1.315 with its spills; packing the gradient's and the flux's
-  // variables in pairs as well measured 3.03).  The kernel is bound by FP32 issue (69 % of the issue slots at 4 warps per scheduler): the bounded sums, the three-term
+  // variables in pairs as well measured 3.03).  The kernel is bound by FP32 issue (76 % of the issue slots at 5 warps per scheduler): the bounded sums, the three-term
   // products and paired traces took the double-float kernel from 8860 to 7540 instructions per
   // warp, 4.375 -> 3.80 ms per launch at 48^3 p = 4, 1.34 -> 1.18 ms at 40^3 p = 3, errors unchanged.
   const bool viscous = VISC == 2 ? dph.viscous != 0 : VISC == 1;
@@ -853,7 +853,7 @@ __device__ __forceinline__ void iface_body(int64_t t, const T *__restrict__ Qtr,
 
 // 5 resident blocks of 128 threads (96 registers, no spills with the Rusanov flux; the Roe flux is an
 // instantiation of its own, which would otherwise set the registers of both), 6 with the FP32 viscous
-// part.  Measured at 5 / 6 blocks: double-float 48^3 p = 4 0.682 / 0.747 ms, FP64 32^3 p = 4 0.843 / 0.857
+// part.  Measured at 5 / 6 blocks: double-float 48^3 p = 4 0.682 / 0.747 ms (0.691 since the FP32 to FP64 conversions moved to the integer pipe), FP64 32^3 p = 4 0.843 / 0.857
 // ms, FP32 viscous 40^3 p = 3 0.231 / 0.220 ms.  Before the viscous flux was formed along the normal and
 // the Roe branch split off: 0.869, 1.072 and 0.232 ms (memory floor 0.48 ms at 48^3; FP64 is bound by its
 // pipe: 185 operations per point instead of 240, Roe 330 instead of 500).

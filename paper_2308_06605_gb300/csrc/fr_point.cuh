@@ -455,7 +455,7 @@ __device__ __forceinline__ void finish_point(int64_t t, const T rv[5], T s, cons
 // point replaces its five entries by the residual, and the update runs over the block's values.  With
 // a thread reading its own point's values each 8-byte access of a warp touches ten 128-byte lines.
 // The copies into shared memory (cp.async: partial residual and the stage's two old register values) are in
-// flight while the double-float kernel gathers the fluxes.  Double-float 48^3 p = 4 1.07 -> 0.80 ms per launch
+// flight while the double-float kernel gathers the fluxes.  Double-float 48^3 p = 4 1.07 -> 0.80 ms per launch (0.757 with to_double on the integer pipe)
 // (0.93 with the partial residual alone staged by plain loads), FP64 32^3 p = 4 0.447 -> 0.398 ms; bound by the
 // FP64 pipe (an addition and an FMA per value, the last stage a split into double-float) beside 3.5 GB of traffic (0.51 ms at
 // 48^3).  FP64 6 blocks per SM (40 registers), double-float 5 (48; 6 measured the same).
