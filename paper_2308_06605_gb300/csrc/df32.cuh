@@ -189,45 +189,6 @@ template <> struct Dot<df32> {
   __device__ __forceinline__ df32 raw() const { return fast_two_sum(s, e); }
 };
 
-// Sum of products with a bound known beforehand: Bound collects b >= sum_i |c_i x_i|, Acc then adds
-// the terms.  double and float: the bound is empty and the sum is the FMA chain of Dot.  df32: the
-// leading parts are summed on top of an offset m = 2.125 b, so the running value a stays within
-// [1.1 b, 3.2 b]; there both a' - a (a' = fl(a + c x), one FMA) and the final a - m are exact (their
-// operands lie on the grid of the smaller one and differ by less than 2^24 of its steps), so the
-// rounding error of every step is one more FMA, c x - (a' - a) -- a two_sum whose three-operation
-// error term is free of the operands' order (Rump, Ogita & Oishi 2008, "Accurate floating-point
-// summation": extraction against a large constant).  7 FP32 instructions per term (the bound
-// included) and 4 at the end, where Dot takes 12 and 3; the offset costs at most two bits of the
-// error term, which is kept to 2^-24 of one grid step (about 2^-48 of b).
-template <typename T> struct Bound {
-  __device__ __forceinline__ void add(T, T) {}
-};
-template <> struct Bound<df32> {
-  float b;
-  __device__ __forceinline__ Bound() : b(0.f) {}
-  __device__ __forceinline__ void add(df32 c, df32 x) { b = __fmaf_rn(::fabsf(c.hi), ::fabsf(x.hi), b); }
-};
-
-template <typename T> struct Acc {
-  T s;
-  __device__ __forceinline__ explicit Acc(const Bound<T> &) : s(0) {}
-  __device__ __forceinline__ void add(T c, T x) { s = fma(c, x, s); }
-  __device__ __forceinline__ T raw() const { return s; }
-};
-template <> struct Acc<df32> {
-  float a, m, e;
-  __device__ __forceinline__ explicit Acc(const Bound<df32> &b) : e(0.f) { a = m = __fmul_rn(2.125f, b.b); }
-  __device__ __forceinline__ void add(df32 c, df32 x) {
-    const float t = __fmaf_rn(c.hi, x.hi, a);
-    float r = __fmaf_rn(c.hi, x.hi, -__fsub_rn(t, a));
-    r = __fmaf_rn(c.hi, x.lo, r);
-    r = __fmaf_rn(c.lo, x.hi, r);
-    a = t;
-    e = __fadd_rn(e, r);
-  }
-  __device__ __forceinline__ df32 raw() const { return fast_two_sum(__fsub_rn(a, m), e); }
-};
-
 // a0 b0 + a1 b1 + a2 b2.  df32: the leading products by two two_sums, every error in one term
 // (31 FP32 instructions; three Dot terms started from zero take 39).
 __device__ __forceinline__ double dot3(double a0, double b0, double a1, double b1, double a2, double b2) {

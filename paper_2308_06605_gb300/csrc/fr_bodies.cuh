@@ -332,23 +332,17 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   // FP32 viscous branch: Q minus the element's first point, in FP32, in the upper half of the
   // gradient buffer (the FP32 gradient uses only its lower half).
   TG *sQg = kPert ? reinterpret_cast<TG *>(sQ + 5 * Np) + 15 * Np : nullptr;   // [5][Np]
-  // Double-float viscous branch: sQ itself holds the perturbation (only the gradient reads it).
-  constexpr bool kPertDf = std::is_same<TG, df32>::value || VISC == 0;
   const PhysT<T> &ph = phys_of<T>(dph);
   const PhysT<TG> &phg = phys_of<TG>(dph);
   const BasisT<T> &B = basis_ref<N, T, VC>(dph);
   // Sums of products end with raw(): the compensated sum renormalised by one fast_two_sum only (an
-  // error of the order of 2^-48 of the sum of the terms' magnitudes).  The gradient and the gradient
-  // traces use the cheaper bounded sums (Acc); in double-float they act on the perturbation from the
-  // element's first point, which makes up for Acc's larger error where a variable has a large mean
-  // (density, energy).  The divergence keeps Dot: it acts on the flux itself, whose pressure part is
-  // nearly constant at low Mach number, and with Acc the momentum residual's error against 64 bits grew
-  // from 3.8e-10 to 1.2e-9 (TGV 40^3, p = 3, Ma 0.1) for 3 % of the kernel's time.  Transform and traces use
-  // packed instructions in double-float (48^3 p = 4 3.09 -> 3.00 ms, 28^3 p = 5 1.174 -> 1.154, but 24^3 p = 6 1.30 ->
-  // 1.315 with its spills; packing the gradient's and the flux's
-  // variables in pairs as well measured 3.03).  The kernel is bound by FP32 issue (76 % of the issue slots at 5 warps per scheduler): the bounded sums, the three-term
-  // products and paired traces took the double-float kernel from 8860 to 7540 instructions per
-  // warp, 4.375 -> 3.80 ms per launch at 48^3 p = 4, 1.34 -> 1.18 ms at 40^3 p = 3, errors unchanged.
+  // error of the order of 2^-48 of the sum of the terms' magnitudes).  All of them are compensated sums
+  // (Dot).  Summing the gradient and its traces on top of a large offset instead (7 FP32 instructions per term for
+  // 12) took 3 % off this kernel at 48^3 p = 4 (3.13 -> 3.05 ms), but a variable of zero mean lost up to three
+  // bits: at p = 7 and Re 0.1 the momentum residual's error grew from 1.4e-11 to 5.0e-11 on hexahedra and from 2.0e-11 to
+  // 1.8e-10 on prisms.  Transform and traces use packed instructions in double-float (48^3 p = 4 3.09 -> 3.00 ms,
+  // 28^3 p = 5 1.174 -> 1.154, but 24^3 p = 6 1.30 -> 1.315 with its spills; packing the gradient's and the flux's
+  // variables in pairs as well measured 3.03).  The kernel is bound by FP32 issue.
   const bool viscous = VISC == 2 ? dph.viscous != 0 : VISC == 1;
   const int grp = SPLIT ? tid / volume_threads<N>() : 0, tp = SPLIT ? tid % volume_threads<N>() : tid;
   const int v0 = SPLIT ? grp : 0, v1 = SPLIT ? grp + 1 : 5;     // this thread's variables
@@ -362,13 +356,10 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
     for (int c = 0; c < 9; ++c) S[c] = met[c * Np];
     invJ = met[9 * Np];
   }
-  if (active && (viscous || !kPertDf))
+  if (active && VISC != 0)
     for (int t = tid; t < 5 * Np; t += nth) {
       const T x = Q[e * Np * 5 + t];
-      if constexpr (kPertDf)
-        sQ[(t % 5) * Np + t / 5] = x - Q[e * Np * 5 + t % 5];
-      else
-        sQ[(t % 5) * Np + t / 5] = x;
+      sQ[(t % 5) * Np + t / 5] = x;
       if constexpr (kPert)
         if (viscous) sQg[(t % 5) * Np + t / 5] = to_g<TG>(x - Q[e * Np * 5 + t % 5]);
     }
@@ -400,7 +391,7 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   if (mine) {
     if (pt)
 #pragma unroll
-      for (int v = 0; v < 5; ++v) q[v] = kPertDf ? Q[(e * Np + m) * 5 + v] : sQ[v * Np + m];
+      for (int v = 0; v < 5; ++v) q[v] = VISC == 0 ? Q[(e * Np + m) * 5 + v] : sQ[v * Np + m];
     if (viscous) {
       // S[d][jj] / |J|.  Double-float transforms the uncorrected and the corrected gradient as the two lanes
       // of packed instructions (their parts wait in shared memory lane by lane: (hi, hi) in sG, (lo, lo) in sGc).
@@ -437,18 +428,9 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
         for (int v = v0; v < v1; ++v) {
           // Derivative along the point's line, then the two faces' correction added to the same sum.
           const TG jlo = dq[v * Nf], jhi = dq[(5 + v) * Nf];
-          TG x[N];
-          Bound<TG> bd;
+          Dot<TG> s(c[0], sq[v * Np + at]);
 #pragma unroll
-          for (int a = 0; a < N; ++a) {
-            x[a] = sq[v * Np + at + a * st];
-            bd.add(c[a], x[a]);
-          }
-          bd.add(hlo, jlo);
-          bd.add(hhi, jhi);
-          Acc<TG> s(bd);
-#pragma unroll
-          for (int a = 0; a < N; ++a) s.add(c[a], x[a]);
+          for (int a = 1; a < N; ++a) s.add(c[a], sq[v * Np + at + a * st]);
           const TG gu = s.raw();
           s.add(hlo, jlo);
           s.add(hhi, jhi);
@@ -629,17 +611,9 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
         for (int v = 0; v < 5; ++v) {
           const TG *sg = sG + (jj * 5 + v) * Np + base;
           const d2 jump = pack(sdQ[(f0 * 5 + v) * Nf + r], sdQ[((f0 + 1) * 5 + v) * Nf + r]);
-          d2 x[N];
-          Bound<d2> bd;
+          Dot<d2> acc(lc[0], dup(sg[0]));
 #pragma unroll
-          for (int c = 0; c < N; ++c) {
-            x[c] = dup(sg[c * sd]);
-            bd.add(lc[c], x[c]);
-          }
-          bd.add(lw, jump);
-          Acc<d2> acc(bd);
-#pragma unroll
-          for (int c = 0; c < N; ++c) acc.add(lc[c], x[c]);
+          for (int c = 1; c < N; ++c) acc.add(lc[c], dup(sg[c * sd]));
           acc.add(lw, jump);
           const d2 g = acc.raw();
           dst[0][v * Nf] = lane0(g);
@@ -657,13 +631,9 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
             // l(+1) is l(-1) mirrored.
             auto l = [&](int c) { return s ? lg[N - 1 - c] : lg[c]; };
             const TG jump = sdQ[((f0 + s) * 5 + v) * Nf + r];
-            Bound<TG> bd;
+            Dot<TG> acc(l(0), x[0]);
 #pragma unroll
-            for (int c = 0; c < N; ++c) bd.add(l(c), x[c]);
-            bd.add(lj[s], jump);
-            Acc<TG> acc(bd);
-#pragma unroll
-            for (int c = 0; c < N; ++c) acc.add(l(c), x[c]);
+            for (int c = 1; c < N; ++c) acc.add(l(c), x[c]);
             acc.add(lj[s], jump);
             dst[s][v * Nf] = from_g<T>(acc.raw());
           }

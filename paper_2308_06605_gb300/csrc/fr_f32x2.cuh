@@ -114,32 +114,5 @@ template <> struct Dot<d2> {
   }
   __device__ __forceinline__ d2 raw() const { return fast_two_sum(s, e); }
 };
-template <> struct Bound<d2> {
-  f2 b;
-  __device__ __forceinline__ Bound() : b(dupf(0.f)) {}
-  __device__ __forceinline__ void add(d2 c, d2 x) { b = pfma(pabs(c.hi), pabs(x.hi), b); }
-};
-template <> struct Bound<f2> {
-  __device__ __forceinline__ void add(f2, f2) {}
-};
-template <> struct Acc<f2> {
-  f2 s;
-  __device__ __forceinline__ explicit Acc(const Bound<f2> &) : s(dupf(0.f)) {}
-  __device__ __forceinline__ void add(f2 c, f2 x) { s = pfma(c, x, s); }
-  __device__ __forceinline__ f2 raw() const { return s; }
-};
-template <> struct Acc<d2> {
-  f2 a, m, e;
-  __device__ __forceinline__ explicit Acc(const Bound<d2> &b) : e(dupf(0.f)) { a = m = pmul(dupf(2.125f), b.b); }
-  __device__ __forceinline__ void add(d2 c, d2 x) {
-    const f2 t = pfma(c.hi, x.hi, a);
-    f2 r = pfma(c.hi, x.hi, psub(a, t));
-    r = pfma(c.hi, x.lo, r);
-    r = pfma(c.lo, x.hi, r);
-    a = t;
-    e = padd(e, r);
-  }
-  __device__ __forceinline__ d2 raw() const { return fast_two_sum(psub(a, m), e); }
-};
 
 }  // namespace frx

@@ -27,7 +27,7 @@ __device__ __forceinline__ PhysT<TG> pair_phys(const PhysT<df32> &p) {
   return r;
 }
 
-// Bytes of shared memory per pair of elements: state perturbation 5, gradient 15 and flux 15 per point, jumps 30
+// Bytes of shared memory per pair of elements: state (FP32 branch: its perturbation) 5, gradient 15 and flux 15 per point, jumps 30
 // per N^2; an inviscid run keeps the flux only.
 template <int N, bool FP32V, int VISC>
 constexpr int pair_smem() {
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
   constexpr int Np = N * N * N, Nf = N * N, nth = volume_threads<N>();
   using TG = typename std::conditional<FP32V, f2, d2>::type;
   d2 *sH = reinterpret_cast<d2 *>(sm_pair);                    // [15][Np] transformed flux, index d*5+v
-  TG *sQ = reinterpret_cast<TG *>(sH + 15 * Np);               // [5][Np] perturbation from the first point
+  TG *sQ = reinterpret_cast<TG *>(sH + 15 * Np);               // [5][Np] state; FP32: less the first point's
   TG *sG = sQ + 5 * Np;                                        // [15][Np] uncorrected gradient, j*5+v
   TG *sdQ = sG + 15 * Np;                                      // [6][5][Nf] Q^I - Q_own at the flux points
   const int64_t e0 = (int64_t)blockIdx.x * 2, e1 = e0 + 1 < E ? e0 + 1 : e0;
@@ -82,7 +82,8 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
   }
   if constexpr (VISC != 0) {
     for (int t = tid; t < 5 * Np; t += nth)
-      sQ[(t % 5) * Np + t / 5] = to_pg<TG>(pack(Q0[t], Q1[t]) - pack(Q0[t % 5], Q1[t % 5]));
+      sQ[(t % 5) * Np + t / 5] = FP32V ? to_pg<TG>(pack(Q0[t], Q1[t]) - pack(Q0[t % 5], Q1[t % 5]))
+                                       : to_pg<TG>(pack(Q0[t], Q1[t]));
     for (int t = tid; t < 6 * Nf; t += nth) {
       const int f = t / Nf, r = t % Nf;
       const df32 *own[2], *oth[2];
@@ -127,18 +128,9 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
 #pragma unroll 1
         for (int v = 0; v < 5; ++v) {
           const TG jlo = dq[v * Nf], jhi = dq[(5 + v) * Nf];
-          TG x[N];
-          Bound<TG> bd;
+          Dot<TG> s(c[0], sQ[v * Np + at]);
 #pragma unroll
-          for (int a = 0; a < N; ++a) {
-            x[a] = sQ[v * Np + at + a * st];
-            bd.add(c[a], x[a]);
-          }
-          bd.add(hlo, jlo);
-          bd.add(hhi, jhi);
-          Acc<TG> s(bd);
-#pragma unroll
-          for (int a = 0; a < N; ++a) s.add(c[a], x[a]);
+          for (int a = 1; a < N; ++a) s.add(c[a], sQ[v * Np + at + a * st]);
           sG[(d * 5 + v) * Np + m] = s.raw();
           s.add(hlo, jlo);
           s.add(hhi, jhi);
@@ -229,13 +221,9 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
         for (int s = 0; s < 2; ++s) {
           auto l = [&](int c) { return dup_g<TG>(s ? B.lp[c] : B.lm[c]); };
           const TG jump = sdQ[((2 * d + s) * 5 + v) * Nf + r];
-          Bound<TG> bd;
+          Dot<TG> acc(l(0), x[0]);
 #pragma unroll
-          for (int c = 0; c < N; ++c) bd.add(l(c), x[c]);
-          bd.add(lj[s], jump);
-          Acc<TG> acc(bd);
-#pragma unroll
-          for (int c = 0; c < N; ++c) acc.add(l(c), x[c]);
+          for (int c = 1; c < N; ++c) acc.add(l(c), x[c]);
           acc.add(lj[s], jump);
           const d2 g = from_pg(acc.raw());
           dst[s][0][v * Nf] = lane0(g);

@@ -110,9 +110,9 @@ __device__ __forceinline__ void prism_interp_body(int64_t t, const T *__restrict
 // 2. Volume kernel.  One block per prism, one thread per solution point.
 // Bound by FP32 issue (double-float) or the FP64 pipe.  Operator entries are read with consecutive
 // threads on consecutive addresses and once for the five variables (row-major tables cost 15 L1
-// wavefronts per load at p = 4, and were read per variable); the gradient sums are bounded ones (Acc).  On
-// the cascade passage (72 case: 25 200 hexahedra, 10 080 prisms, p = 4) the two volume kernels together
-// 1.505 -> 1.236 ms in double-float, 5.06 -> 4.60 ms in FP64.
+// wavefronts per load at p = 4, and were read per variable).  On the cascade passage (72 case: 25 200
+// hexahedra, 10 080 prisms, p = 4) the two volume kernels together 1.505 -> 1.260 ms in double-float, 5.06 ->
+// 4.60 ms in FP64.
 // ------------------------------------------------------------------------------------------
 // One prism e handled by `nth` threads of the block (thread index tid in [0, nth)); every thread
 // of the block calls this together (it contains block barriers); inactive sub-blocks
@@ -135,9 +135,8 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
   T *sdQ = sL + 15 * Np;      // [5][5][Nf] Q^I - Q_own at the flux points
   const PhysT<T> &ph = phys_of<T>(dph);
   const bool viscous = dph.viscous != 0;
-  // The gradient acts on the perturbation from the prism's first point (its only reader of sQ).
   if (active && viscous)
-    for (int t = tid; t < 5 * Np; t += nth) sQ[(t % 5) * Np + t / 5] = Q[e * Np * 5 + t] - Q[e * Np * 5 + t % 5];
+    for (int t = tid; t < 5 * Np; t += nth) sQ[(t % 5) * Np + t / 5] = Q[e * Np * 5 + t];
   if (viscous && active) {
     for (int t = tid; t < 5 * Nf; t += nth) {
       const int f = t / Nf, r = t % Nf;
@@ -181,12 +180,9 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
         for (int a = 0; a < N; ++a) c[a] = lq[a * Nt];
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
-          Bound<T> bd;
+          Dot<T> s(c[0], dq[v * Nf]);
 #pragma unroll
-          for (int a = 0; a < N; ++a) bd.add(c[a], dq[v * Nf + a]);
-          Acc<T> s(bd);
-#pragma unroll
-          for (int a = 0; a < N; ++a) s.add(c[a], dq[v * Nf + a]);
+          for (int a = 1; a < N; ++a) s.add(c[a], dq[v * Nf + a]);
           sL[(f * 5 + v) * Np + m] = s.raw();
         }
       }
@@ -199,14 +195,9 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
           const T jlo = sdQ[v * Nf + q], jhi = sdQ[(5 + v) * Nf + q];
-          Bound<T> bd;
+          Dot<T> s(c[0], sQ[v * Np + q]);
 #pragma unroll
-          for (int a = 0; a < N; ++a) bd.add(c[a], sQ[v * Np + q + Nt * a]);
-          bd.add(hmk, jlo);
-          bd.add(hpk, jhi);
-          Acc<T> s(bd);
-#pragma unroll
-          for (int a = 0; a < N; ++a) s.add(c[a], sQ[v * Np + q + Nt * a]);
+          for (int a = 1; a < N; ++a) s.add(c[a], sQ[v * Np + q + Nt * a]);
           sG[(10 + v) * Np + m] = s.raw();
           s.add(hmk, jlo);
           s.add(hpk, jhi);
@@ -216,19 +207,7 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
       {
         // Both triangle derivatives of the five variables together: an operator entry is read once.
         const T *Dr = tab + L.Dr + q, *Ds = tab + L.Ds + q, *sq = sQ + Nt * k;
-        Bound<T> b0[5], b1[5];
-#pragma unroll 3
-        for (int j = 0; j < Nt; ++j) {
-          const T dr = Dr[j * Nt], ds = Ds[j * Nt];
-#pragma unroll
-          for (int v = 0; v < 5; ++v) {
-            const T x = sq[v * Np + j];
-            b0[v].add(dr, x);
-            b1[v].add(ds, x);
-          }
-        }
-        Acc<T> a0[5] = {Acc<T>(b0[0]), Acc<T>(b0[1]), Acc<T>(b0[2]), Acc<T>(b0[3]), Acc<T>(b0[4])};
-        Acc<T> a1[5] = {Acc<T>(b1[0]), Acc<T>(b1[1]), Acc<T>(b1[2]), Acc<T>(b1[3]), Acc<T>(b1[4])};
+        Dot<T> a0[5], a1[5];
 #pragma unroll 3
         for (int j = 0; j < Nt; ++j) {
           const T dr = Dr[j * Nt], ds = Ds[j * Nt];
@@ -321,13 +300,9 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
         for (int v = 0; v < 5; ++v) {
           const T *g = sG + (jj * 5 + v) * Np + r;
           const T jump = sdQ[(f * 5 + v) * Nf + r];
-          Bound<T> bd;
+          Dot<T> acc(l[0], g[0]);
 #pragma unroll
-          for (int c = 0; c < N; ++c) bd.add(l[c], g[Nt * c]);
-          bd.add(lfac, jump);
-          Acc<T> acc(bd);
-#pragma unroll
-          for (int c = 0; c < N; ++c) acc.add(l[c], g[Nt * c]);
+          for (int c = 1; c < N; ++c) acc.add(l[c], g[Nt * c]);
           acc.add(lfac, jump);
           dst[v * Nf] = acc.raw();
         }
@@ -361,14 +336,7 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
           const int64_t I = packed >> 4;
           T *dst = Gtr + (I * 2 + ((packed >> 3) & 1)) * 15 * Nf + prism_slot<N>(f, r, packed & 7, tri_slot) + jj * 5 * Nf;
           const T *Ea = tab + L.E + (f - 2) * N * Nt + a, *x = sG + jj * 5 * Np + Nt * b;
-          Bound<T> bd[5];
-#pragma unroll 3
-          for (int j = 0; j < Nt; ++j) {
-            const T ej = Ea[j * N];
-#pragma unroll
-            for (int v = 0; v < 5; ++v) bd[v].add(ej, x[v * Np + j]);
-          }
-          Acc<T> acc[5] = {Acc<T>(bd[0]), Acc<T>(bd[1]), Acc<T>(bd[2]), Acc<T>(bd[3]), Acc<T>(bd[4])};
+          Dot<T> acc[5];
 #pragma unroll 3
           for (int j = 0; j < Nt; ++j) {
             const T ej = Ea[j * N];

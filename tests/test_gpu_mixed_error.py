@@ -1,0 +1,34 @@
+"""Error of the double-float residual against the FP64 one (marked gpu), L2 per momentum component.
+
+The suite's bar of 1e-9 of the magnitude scale leaves three bits of room; here the bars are 1.4 to 2 times
+what compensated sums give (gradient, gradient traces, divergence, lifting: an error of 2^-48 of each sum's
+terms).  Re 0.1: the residual is the divergence of the viscous stress, so the gradient's own error shows."""
+import numpy as np
+import pytest
+
+from paper_2308_06605_gb300 import fr
+from paper_2308_06605_gb300 import inputs as I
+
+from helpers import ensure_lib
+
+pytestmark = pytest.mark.gpu
+
+
+def _momentum_error(p, n, prisms, Re):
+    ensure_lib()
+    d = I.hex_box_mesh((n, n, n), seed=4, rotate=prisms is None, perturb=0.1, prisms=prisms)
+    R = []
+    for precision in (fr.FR_PREC_FP64, fr.FR_PREC_MIXED):
+        ph = I.tgv_physics(Ma=0.1, Re=Re)
+        ph.precision = precision
+        with fr.Mesh(d, ph, p) as m:
+            m.set_state(np.ascontiguousarray(I.tgv_state(m.solution_points(), Ma=0.1, perturb=1e-2, seed=1)))
+            R.append(m.residual().reshape(-1, 5)[:, 1:4])
+    return np.linalg.norm(R[1] - R[0], axis=0) / np.linalg.norm(R[0], axis=0)
+
+
+@pytest.mark.parametrize("p,n,bar", [(5, 8, 2e-11), (7, 6, 4e-11)])
+@pytest.mark.parametrize("prisms", [None, "all"])
+def test_viscous_residual(prisms, p, n, bar):
+    err = _momentum_error(p, n, prisms, 0.1)
+    assert (err <= bar).all(), err
