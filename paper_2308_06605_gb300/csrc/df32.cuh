@@ -140,6 +140,7 @@ template <> struct Dot<double> {
   __device__ __forceinline__ explicit Dot(double x) : s(x) {}
   __device__ __forceinline__ void add(double c, double x) { s = fma(c, x, s); }
   __device__ __forceinline__ void plus(double x) { s += x; }
+  __device__ __forceinline__ void join(const Dot &o) { s += o.s; }
   __device__ __forceinline__ double get() const { return s; }
   __device__ __forceinline__ double raw() const { return s; }
 };
@@ -179,6 +180,12 @@ template <> struct Dot<df32> {
     const df32 t = two_sum(s, x.hi);
     s = t.hi;
     e = __fadd_rn(e, __fadd_rn(t.lo, x.lo));
+  }
+  // Another sum on top of this one (8 instructions).
+  __device__ __forceinline__ void join(const Dot &o) {
+    const df32 t = two_sum(s, o.s);
+    s = t.hi;
+    e = __fadd_rn(e, __fadd_rn(t.lo, o.e));
   }
   __device__ __forceinline__ df32 get() const {
     const df32 r = two_sum(s, e);

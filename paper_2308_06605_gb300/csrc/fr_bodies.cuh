@@ -1086,7 +1086,7 @@ __global__ void __launch_bounds__(kCorrectThreads, std::is_same<T, double>::valu
                            kGatherFirst<T> ? nullptr : reinterpret_cast<const T *>(sm.r) + threadIdx.x * 5, r);
     s = -metrics[(e * 10 + 9) * Np + m];
   }
-  finish_block<T, SRC>(first, n, sm, r, s, sc, in, Rout, Q, Qc, Un, Unc, acc, flag, dph);
+  finish_block<T, SRC>(first, n, sm, r, nullptr, s, sc, in, Rout, Q, Qc, Un, Unc, acc, flag, dph);
 }
 
 // Meshes with prisms: a triangular interface uses only the first N(N+1)/2 of its N^2 slots;

@@ -498,10 +498,11 @@ __device__ __forceinline__ void stage_arrive() {
 template <typename T> constexpr bool kGatherFirst = std::is_same<T, df32>::value;
 
 // first: flat index of the block's first point in the registers, n: points of the block; this thread's lifted
-// fluxes rv (FP64: with the partial residual) and s = -1/|J| (used if threadIdx.x < n).
+// fluxes rv (FP64: with the partial residual), a second part of them that is added after the residual (may be
+// null) and s = -1/|J| (used if threadIdx.x < n).
 template <typename T, bool SRC>
-__device__ __forceinline__ void finish_block(int64_t first, int n, const CorrectSmem &sm, Dot<T> rv[5], T s,
-                                             const StageCoef &c, const StageIn &in, double *__restrict__ Rout,
+__device__ __forceinline__ void finish_block(int64_t first, int n, const CorrectSmem &sm, Dot<T> rv[5],
+                                             const Dot<T> *last, T s, const StageCoef &c, const StageIn &in, double *__restrict__ Rout,
                                              double *__restrict__ Q, T *__restrict__ Qc, double *__restrict__ Un,
                                              T *__restrict__ Unc, double *__restrict__ acc, int *__restrict__ flag,
                                              const DevPhys &dph) {
@@ -512,6 +513,7 @@ __device__ __forceinline__ void finish_block(int64_t first, int n, const Correct
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       if constexpr (kGatherFirst<T>) rv[v].plus(sr[me * 5 + v]);
+      if (last) rv[v].join(last[v]);
       sr[me * 5 + v] = rv[v].get() * s;
     }
     if constexpr (SRC) {

@@ -63,17 +63,17 @@ __global__ void __launch_bounds__(kCorrectThreads)
   const int n = (int)(Ep * Np - first < kCorrectThreads ? Ep * Np - first : kCorrectThreads);
   const StageIn in = stage_inputs<T>(sc, Q, Un, Unc, acc);
   stage_begin<T>(sm, Rpart + first * 5, (first_point + first) * 5, n, in);
-  Dot<T> r[5];
+  Dot<T> r[5], line[5];
   T s{};
   if constexpr (!kGatherFirst<T>) stage_arrive();
   if ((int)threadIdx.x < n) {
     const int64_t t = first + threadIdx.x, e = t / Np;
     const int m = (int)(t % Np);
     prism_correct_lift<N, T>(e, m, FI, ef_p, tab, tri_slot,
-                             kGatherFirst<T> ? nullptr : reinterpret_cast<const T *>(sm.r) + threadIdx.x * 5, r);
+                             kGatherFirst<T> ? nullptr : reinterpret_cast<const T *>(sm.r) + threadIdx.x * 5, r, line);
     s = -metrics[(e * 10 + 9) * Np + m];
   }
-  finish_block<T, SRC>(first_point + first, n, sm, r, s, sc, in, Rout, Q, Qc, Un, Unc, acc, flag, dph);
+  finish_block<T, SRC>(first_point + first, n, sm, r, kGatherFirst<T> ? line : nullptr, s, sc, in, Rout, Q, Qc, Un, Unc, acc, flag, dph);
 }
 
 // dt bound per prism: cfl h / ((2p + 1) max(|u| + c)) over its points (FP64 state).

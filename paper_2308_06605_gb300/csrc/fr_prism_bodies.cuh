@@ -352,16 +352,20 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
   if (pt) {
     const T *Drt = tab + L.Drt + q, *Dst = tab + L.Dst + q, *D1t = tab + L.D1t + k * N;
     const T *h0 = sH + Nt * k, *h1 = h0 + 5 * Np, *h2 = sH + 10 * Np + q;
-    Dot<T> acc[5];
+    // The line's sum and the triangle's are kept apart until the end: each holds the large pressure part of some
+    // momentum component, on top of which the other's terms would lose their last bits.  With the line's terms
+    // first in one sum the error of the momentum component along the prisms' axis was 3.4 times as large (p = 7,
+    // Ma 0.1), with the triangle's first that of the other two 1.2 times.
+    Dot<T> acc[5], line[5];
 #pragma unroll
     for (int c = 0; c < N; ++c) {
       const T dc = D1t[c];
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         if (c == 0)
-          acc[v] = Dot<T>(dc, h2[v * Np]);
+          line[v] = Dot<T>(dc, h2[v * Np]);
         else
-          acc[v].add(dc, h2[v * Np + Nt * c]);
+          line[v].add(dc, h2[v * Np + Nt * c]);
       }
     }
 #pragma unroll 3
@@ -375,17 +379,24 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
     }
     T *out = Rpart + (e * Np + m) * 5;
 #pragma unroll
-    for (int v = 0; v < 5; ++v) out[v] = acc[v].raw();
+    for (int v = 0; v < 5; ++v) {
+      acc[v].join(line[v]);
+      out[v] = acc[v].raw();
+    }
   }
 }
 
 // ------------------------------------------------------------------------------------------
 // 4. Correction by the common flux, scaling and output / RK44 update.  Thread per prism point.
 // ------------------------------------------------------------------------------------------
+// Lifted common fluxes of the five faces at point m of prism e.  FP64: on top of the partial residual rp, in r,
+// and `line` stays empty.  Double-float (rp null, the residual is added later): the quadrilaterals' in r and the
+// triangles' in `line`, which joins r after the residual, for the reason given at the divergence.
 template <int N, typename T>
 __device__ __forceinline__ void prism_correct_lift(int64_t e, int m, const T *__restrict__ FI,
                                                    const int32_t *__restrict__ ef_p, const T *__restrict__ tab,
-                                                   const int32_t *__restrict__ tri_slot, const T *rp, Dot<T> r[5]) {
+                                                   const int32_t *__restrict__ tri_slot, const T *rp, Dot<T> r[5],
+                                                   Dot<T> line[5]) {
   if (rp)
 #pragma unroll
     for (int v = 0; v < 5; ++v) r[v] = Dot<T>(rp[v]);
@@ -402,10 +413,12 @@ __device__ __forceinline__ void prism_correct_lift(int64_t e, int m, const T *__
     const T *src = FI + I * 5 * Nf + tri_slot[(packed & 7) * Nt + q];
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
-      if (f == 0 && !rp)
-        r[v] = Dot<T>(w, src[v * Nf]);
-      else
+      if (rp)
         r[v].add(w, src[v * Nf]);
+      else if (f == 0)
+        line[v] = Dot<T>(w, src[v * Nf]);
+      else
+        line[v].add(w, src[v * Nf]);
     }
   }
 #pragma unroll
@@ -420,7 +433,12 @@ __device__ __forceinline__ void prism_correct_lift(int64_t e, int m, const T *__
       const T w = side ? -lq[a * Nt] : lq[a * Nt];
       const int slot = orient_slot(packed & 7, a, k, N);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) r[v].add(w, src[v * Nf + slot]);
+      for (int v = 0; v < 5; ++v) {
+        if (f == 2 && a == 0 && !rp)
+          r[v] = Dot<T>(w, src[v * Nf + slot]);
+        else
+          r[v].add(w, src[v * Nf + slot]);
+      }
     }
   }
 }
@@ -439,12 +457,15 @@ __device__ __forceinline__ void prism_correct_body(int64_t t, const T *__restric
   if (t >= Ep * Np) return;
   const int64_t e = t / Np;
   const int m = (int)(t % Np);
-  Dot<T> r[5];
-  prism_correct_lift<N, T>(e, m, FI, ef_p, tab, tri_slot, kGatherFirst<T> ? nullptr : Rpart + t * 5, r);
+  Dot<T> r[5], line[5];
+  prism_correct_lift<N, T>(e, m, FI, ef_p, tab, tri_slot, kGatherFirst<T> ? nullptr : Rpart + t * 5, r, line);
   T rv[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
-    if constexpr (kGatherFirst<T>) r[v].plus(Rpart[t * 5 + v]);
+    if constexpr (kGatherFirst<T>) {
+      r[v].plus(Rpart[t * 5 + v]);
+      r[v].join(line[v]);
+    }
     rv[v] = r[v].get();
   }
   finish_point<T>(first_point + t, rv, -metrics[(e * 10 + 9) * Np + m], sc, Rout, Q, Qc, Un, Unc, acc,
