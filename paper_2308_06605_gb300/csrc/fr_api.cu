@@ -1,4 +1,5 @@
 // C ABI (include/fr.h): mesh lifetime, state transfer, residual and RK44 stages.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -455,10 +456,32 @@ static cudaMemcpyKind kind_of(int where, bool to_device) {
   return to_device ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost;
 }
 
-// True if a kernel of this mesh may read p directly: an aligned pointer to plain memory of the mesh's
-// device, which is the current one.  Anything else a copy accepts (another device's memory, an odd
-// address, a thread on another device) keeps the copies.
-static bool readable_here(const fr_mesh *m, const void *p) {
+// True if [p, p + bytes) lies inside one allocation.  The driver's query is found through the runtime, so the
+// library still loads where there is no driver.
+static bool within_allocation(const void *p, size_t bytes) {
+  using Query = CUresult(CUDAAPI *)(CUdeviceptr *, size_t *, CUdeviceptr);
+  static const Query query = [] {
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      fn = nullptr;
+    }
+    return reinterpret_cast<Query>(fn);
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+  if (!query || query(&base, &size, at) != CUDA_SUCCESS) return false;
+  return at >= base && bytes <= size && at - base <= size - bytes;
+}
+
+// True if a kernel of this mesh may read bytes at p directly: an aligned range inside one allocation of
+// plain memory of the mesh's device, which is the current one.  Anything else keeps the copies, which accept it
+// (another device's memory, an odd address, a thread on another device) or refuse it (a buffer shorter than the
+// state).
+static bool readable_here(const fr_mesh *m, const void *p, size_t bytes) {
   if (reinterpret_cast<uintptr_t>(p) % sizeof(double)) return false;
   int cur = -1;
   cudaPointerAttributes at;
@@ -466,18 +489,18 @@ static bool readable_here(const fr_mesh *m, const void *p) {
     cudaGetLastError();
     return false;
   }
-  return at.type == cudaMemoryTypeDevice && at.device == m->device;
+  return at.type == cudaMemoryTypeDevice && at.device == m->device && within_allocation(p, bytes);
 }
 
 extern "C" fr_status fr_set_state(fr_mesh *m, const double *Q, int32_t where) {
   fr_status st = check_mesh(m);
   if (st) return st;
   if (!Q || (where != FR_HOST && where != FR_DEVICE)) return fail(m, FR_EINVAL, "bad state pointer or where");
-  if (where == FR_DEVICE && readable_here(m, Q)) {
+  const size_t bytes = state_bytes(m->dev);
+  if (where == FR_DEVICE && readable_here(m, Q, bytes)) {
     FR_CUDA(m, launch_start_state(m->dev, Q, m->stream));
     return FR_OK;
   }
-  const size_t bytes = state_bytes(m->dev);
   FR_CUDA(m, cudaMemcpyAsync(m->dev.Q, Q, bytes, kind_of(where, true), m->stream));
   FR_CUDA(m, cudaMemcpyAsync(m->dev.Un, m->dev.Q, bytes, cudaMemcpyDeviceToDevice, m->stream));
   FR_CUDA(m, launch_state_copy(m->dev, m->stream));
