@@ -128,7 +128,10 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
     auto kern = ph.viscous ? k_volume<N, T, false, 1> : k_volume<N, T, false, 0>;
     if constexpr (std::is_same<T, df32>::value)
       if (m.vf32 && ph.viscous) kern = k_volume<N, T, true, 1>;
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // The kernel's limit is set to its largest block, with the closure, whether this mesh has one or not: it is a
+    // property of the kernel, and another thread's launch of it may come between this call and the launch below.
+    const int cap = (int)volume_smem<N, T>(ph.viscous, true);
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
     if (err != cudaSuccess) return err;
     FR_EV_BEGIN(1);
     if (E > 0 && ph.vc_basis) {
@@ -141,7 +144,7 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
           auto sk = k_volume_split<N, T, false>;
           if constexpr (std::is_same<T, df32>::value)
             if (m.vf32) sk = k_volume_split<N, T, true>;
-          err = cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+          err = cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
           if (err != cudaSuccess) return err;
           sk<<<(unsigned)E, 5 * volume_threads<N>(), smem, st>>>(Qin, met, m.ef, Qtr, lift, Gtr, Rpart, ph, m.h, m.nu,
                                                                  m.if_up, m.n_interior);

@@ -120,9 +120,24 @@ __global__ void __launch_bounds__(kProjectThreads)
     out.put(e0 * n2 + i, along<Nd, 5 * Ntd>(L, b, i, Ns));
 }
 
-// Elements per block: about four items per thread at the larger of the two orders, which also keeps the
-// block's shared memory below 48 KB.
-int project_epb(int values) { return std::min(16, std::max(1, 4 * kProjectThreads / values)); }
+// Elements per block: about four items per thread at the larger of the two orders.
+constexpr int project_epb(int values) { return std::min(16, std::max(1, 4 * kProjectThreads / values)); }
+
+// Shared memory of a block of k_project_prism from Ns to Nd points per line.
+constexpr size_t project_prism_smem(int Ns, int Nd) {
+  const int Nts = Ns * (Ns + 1) / 2, Ntd = Nd * (Nd + 1) / 2;
+  const int epb = project_epb(std::max(Nts * Ns, Ntd * Nd) * 5);
+  return sizeof(double) * ((size_t)Nts * Ntd + Ns * Nd + 5 * (size_t)epb * Ns * (Nts + Ntd));
+}
+// No pair of orders needs more than the 48 KB that a launch may ask for without raising the kernel's limit, which
+// two threads' calls would set to different sizes.
+constexpr size_t project_prism_smem_max() {
+  size_t most = 0;
+  for (int s = 2; s <= kMaxN; ++s)
+    for (int d = 2; d <= kMaxN; ++d) most = std::max(most, project_prism_smem(s, d));
+  return most;
+}
+static_assert(project_prism_smem_max() <= 48 * 1024, "k_project_prism launches without a raised limit");
 
 template <int Nd>
 cudaError_t launch_project(const DevMesh &a, const DevMesh &b, const std::vector<double> &L,
@@ -142,10 +157,8 @@ cudaError_t launch_project(const DevMesh &a, const DevMesh &b, const std::vector
     std::memcpy(op.L, L.data(), L.size() * sizeof(double));
     std::memcpy(op.T, Tt.data(), Tt.size() * sizeof(double));
     const int epb = project_epb(std::max(a.Npp, b.Npp) * 5);
-    const size_t smem = sizeof(double) * ((size_t)a.Nt * b.Nt + a.N * b.N + 5 * (size_t)epb * a.N * (a.Nt + b.Nt));
+    const size_t smem = project_prism_smem(a.N, b.N);
     const int64_t os = a.E * a.Np * 5, od = b.E * b.Np * 5;
-    cudaError_t e = cudaFuncSetAttribute(k_project_prism<Nd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     k_project_prism<Nd><<<(unsigned)((a.Ep + epb - 1) / epb), kProjectThreads, smem, st>>>(
         a.Q + os, StateOut{b.Q + od, b.Un + od, Qc ? Qc + od : nullptr, Unc ? Unc + od : nullptr}, op, a.Ep, a.N, epb);
   }

@@ -35,8 +35,9 @@ static cudaError_t vcjh_phase_impl(const DevMesh &m, const DevPhys &ph, int phas
   T *Rpart = reinterpret_cast<T *>(m.Rpart);
   const T *met = reinterpret_cast<const T *>(m.metrics);
   if (phase == 1) {
-    const size_t smem = sizeof(T) * (35 * Np + 30 * Nf) + (ph.closure ? sizeof(float) * closure_floats<N>() : 0);
-    cudaError_t err = cudaFuncSetAttribute(k_volume_vc<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t plain = sizeof(T) * (35 * Np + 30 * Nf), cap = plain + sizeof(float) * closure_floats<N>();
+    const size_t smem = ph.closure ? cap : plain;
+    cudaError_t err = cudaFuncSetAttribute(k_volume_vc<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap);
     if (err != cudaSuccess) return err;
     k_volume_vc<N, T><<<(unsigned)E, volume_threads<N>(), smem, st>>>(
         Qin, met, m.ef, reinterpret_cast<const T *>(m.Qtr), reinterpret_cast<const T *>(m.liftfac), Gtr, Rpart, ph,
