@@ -332,8 +332,10 @@ template <typename T, bool SRC>
 __device__ __forceinline__ bool finish_value(int64_t o, T rs, double src, const StageCoef &c, double x1, double x2,
                                              double *__restrict__ Rout, double *__restrict__ Q, T *__restrict__ Qc,
                                              double *__restrict__ Un, T *__restrict__ Unc, double *__restrict__ acc) {
+  // Products and sums that the compiler could contract in more than one way are written as the operations they
+  // are: the staged kernel and the one with a thread per point have to give the same bits.
   double rd = to_double(rs);
-  if constexpr (SRC) rd += src;
+  if constexpr (SRC) rd = __dadd_rn(rd, src);
   if (c.mode == MODE_RESIDUAL) {
     Rout[o] = rd;
     return false;
@@ -360,11 +362,11 @@ __device__ __forceinline__ bool finish_value(int64_t o, T rs, double src, const 
       return !isfinite(nv);
     } else {
       if (!c.last) {
-        acc[o] = x1 + c.b * rd;
-        Q[o] = x2 + c.a * rd;
+        acc[o] = fma(c.b, rd, x1);
+        Q[o] = fma(c.a, rd, x2);
         return false;
       }
-      const double nv = x2 + x1 + c.b * rd;
+      const double nv = fma(c.b, rd, x2 + x1);
       Un[o] = nv;
       Q[o] = nv;
       return !isfinite(nv);
@@ -378,16 +380,16 @@ __device__ __forceinline__ bool finish_value(int64_t o, T rs, double src, const 
   const double q = x1;
   double nq;
   if (c.mode == MODE_SSP33) {
-    nq = c.a * x2 + c.b * fma(c.dt, rd, q);
+    nq = fma(c.b, fma(c.dt, rd, q), __dmul_rn(c.a, x2));
   } else if (!c.last) {
     nq = fma(c.b, rd, q);
     if (c.stage == 4) {
-      const double q2 = x2 / 25.0 + 9.0 / 25.0 * nq;
+      const double q2 = fma(9.0 / 25.0, nq, x2 / 25.0);
       acc[o] = q2;
-      nq = 15.0 * q2 - 5.0 * nq;
+      nq = fma(15.0, q2, -5.0 * nq);
     }
   } else {
-    nq = x2 + 0.6 * q + c.b * rd;
+    nq = fma(c.b, rd, fma(0.6, q, x2));
   }
   Q[o] = nq;
   if constexpr (std::is_same<T, df32>::value) Qc[o] = from_double<T>(nq);
@@ -412,12 +414,12 @@ __device__ __forceinline__ void point_source(int64_t t, const double *__restrict
     src[1] = q[0] * dph.accel[0];
     src[2] = q[0] * dph.accel[1];
     src[3] = q[0] * dph.accel[2];
-    src[4] = q[1] * dph.accel[0] + q[2] * dph.accel[1] + q[3] * dph.accel[2];
+    src[4] = fma(q[3], dph.accel[2], fma(q[2], dph.accel[1], q[1] * dph.accel[0]));
   }
   if (dph.src_sponge) {
     const double sg = dph.sigma[t];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) src[v] -= sg * (q[v] - dph.Q_ref[t * 5 + v]);
+    for (int v = 0; v < 5; ++v) src[v] = fma(-sg, q[v] - dph.Q_ref[t * 5 + v], src[v]);
   }
 }
 
