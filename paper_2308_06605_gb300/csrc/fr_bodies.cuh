@@ -549,6 +549,18 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
     const T u[3] = {q[1] * ri, q[2] * ri, q[3] * ri};
     const T p = ph.gm1 * (q[4] - scale2(dot3(q[1], u[0], q[2], u[1], q[3], u[2]), 0.5f));
     T tau[6], hq[3], mom[6], en[3];
+    bool formed = false;
+    if constexpr (std::is_same<T, double>::value && VISC != 1)
+      if (!viscous) {
+        formed = true;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          double f[5];
+          inviscid_transformed(q, u, p, S + 3 * d, f);
+#pragma unroll
+          for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
+        }
+      }
     if (viscous) {
       if constexpr (kPert) {
         TG qg[5], ug[3], taug[6], hqg[3];
@@ -566,13 +578,15 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
         viscous_stress<T>(q, u, ri, G, ph, visc_with(ph, rho_nu, dph), tau, hq);
       }
     }
-    physical_flux<T>(q, u, p, viscous, tau, hq, mom, en);
+    if (!formed) {
+      physical_flux<T>(q, u, p, viscous, tau, hq, mom, en);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      T f[5];
-      transformed_flux<T>(q, mom, en, S + 3 * d, f);
+      for (int d = 0; d < 3; ++d) {
+        T f[5];
+        transformed_flux<T>(q, mom, en, S + 3 * d, f);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
+        for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
+      }
     }
   }
   __syncthreads();

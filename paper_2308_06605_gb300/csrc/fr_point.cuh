@@ -258,6 +258,18 @@ __device__ __forceinline__ void physical_flux(const T q[5], const T u[3], T p, b
   }
 }
 
+// Inviscid transformed flux of reference direction d in FP64, from the contravariant velocity: 12 operations per
+// direction where the tensor above and its transform take 18 (the viscous part is what the tensor saves on).  Every
+// FP64 element kernel without a viscous branch uses it, each with the same operations.
+__device__ __forceinline__ void inviscid_transformed(const double q[5], const double u[3], double p, const double Sd[3],
+                                                     double f[5]) {
+  const double Ud = fma(Sd[2], u[2], fma(Sd[1], u[1], Sd[0] * u[0]));
+  f[0] = q[0] * Ud;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) f[1 + i] = fma(q[1 + i], Ud, Sd[i] * p);
+  f[4] = __dadd_rn(q[4], p) * Ud;
+}
+
 // Transformed flux of reference direction d, F^_d = sum_j S[d][j] (F - Fv)_j (Eq. 1); Sd = S[d][0..2].
 template <typename T>
 __device__ __forceinline__ void transformed_flux(const T q[5], const T m[6], const T en[3], const T Sd[3], T f[5]) {

@@ -267,14 +267,28 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
       const T u[3] = {qv[1] * ri, qv[2] * ri, qv[3] * ri};
       const T p = ph.gm1 * (qv[4] - scale2(dot3(qv[1], u[0], qv[2], u[1], qv[3], u[2]), 0.5f));
       T tau[6], hq[3], mom[6], en[3];
-      if (viscous) viscous_stress<T>(qv, u, ri, G, ph, visc_of(ph), tau, hq);
-      physical_flux<T>(qv, u, p, viscous, tau, hq, mom, en);
+      bool formed = false;
+      if constexpr (std::is_same<T, double>::value)
+        if (!viscous) {
+          formed = true;
 #pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        T f[5];
-        transformed_flux<T>(qv, mom, en, S + 3 * d, f);
+          for (int d = 0; d < 3; ++d) {
+            double f[5];
+            inviscid_transformed(qv, u, p, S + 3 * d, f);
 #pragma unroll
-        for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
+            for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
+          }
+        }
+      if (!formed) {
+        if (viscous) viscous_stress<T>(qv, u, ri, G, ph, visc_of(ph), tau, hq);
+        physical_flux<T>(qv, u, p, viscous, tau, hq, mom, en);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          T f[5];
+          transformed_flux<T>(qv, mom, en, S + 3 * d, f);
+#pragma unroll
+          for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
+        }
       }
     }
   }
