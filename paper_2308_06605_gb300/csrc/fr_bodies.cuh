@@ -1067,14 +1067,14 @@ __device__ __forceinline__ void correct_body(int64_t t, const T *__restrict__ Rp
 // at 64000 points 14.4 against 14.7 us, and at 32^3 p = 4 0.398 ms staged against 0.431.
 constexpr int64_t kCorrectPointMax = 152 * 256;
 
-template <int N, typename T>
+template <int N, typename T, bool VC>
 __global__ void __launch_bounds__(32)
     k_correct_point(const T *__restrict__ Rpart, const T *__restrict__ FI, const int32_t *__restrict__ ef,
                     const T *__restrict__ metrics, int64_t E, StageCoef sc, double *__restrict__ Rout,
                     double *__restrict__ Q, T *__restrict__ Qc, double *__restrict__ Un, T *__restrict__ Unc,
                     double *__restrict__ acc, int *__restrict__ flag, DevPhys dph) {
-  correct_body<N, T>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, Rpart, FI, ef, metrics, E, sc, Rout, Q, Qc, Un, Unc,
-                     acc, flag, dph);
+  correct_body<N, T, VC>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, Rpart, FI, ef, metrics, E, sc, Rout, Q, Qc, Un,
+                         Unc, acc, flag, dph);
 }
 
 template <int N, typename T, bool VC, bool SRC>

@@ -194,7 +194,7 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
     if (n > 0 && ph.vc_basis) {
       if ((err = launch_vcjh_phase(m, ph, 3, mode, stage, dt, Rout, st)) != cudaSuccess) return err;
     } else if (n > 0 && n <= kCorrectPointMax) {
-      k_correct_point<N, T><<<(unsigned)((n + 31) / 32), 32, 0, st>>>(
+      k_correct_point<N, T, false><<<(unsigned)((n + 31) / 32), 32, 0, st>>>(
           Rpart, FI, m.ef, met, E, stage_coef(mode, stage, dt), Rout, m.Q, Qc, m.Un, reinterpret_cast<T *>(m.Unc), m.acc,
           m.flag, ph);
     } else if (n > 0) {

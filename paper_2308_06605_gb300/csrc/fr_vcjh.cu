@@ -44,10 +44,15 @@ static cudaError_t vcjh_phase_impl(const DevMesh &m, const DevPhys &ph, int phas
         m.h, m.nu, m.if_up, m.n_interior);
   } else if (phase == 3) {
     const int64_t n = E * Np;
+    T *Qc = m.mixed ? reinterpret_cast<T *>(m.Qc) : nullptr, *Unc = reinterpret_cast<T *>(m.Unc);
+    if (n <= kCorrectPointMax) {
+      k_correct_point<N, T, true><<<(unsigned)((n + 31) / 32), 32, 0, st>>>(
+          Rpart, FI, m.ef, met, E, stage_coef(mode, stage, dt), Rout, m.Q, Qc, m.Un, Unc, m.acc, m.flag, ph);
+      return cudaGetLastError();
+    }
     auto ck = has_source(ph) ? k_correct<N, T, true, true> : k_correct<N, T, true, false>;
     ck<<<(unsigned)((n + kCorrectThreads - 1) / kCorrectThreads), kCorrectThreads, correct_smem(ph), st>>>(
-        Rpart, FI, m.ef, met, E, stage_coef(mode, stage, dt), Rout, m.Q,
-        m.mixed ? reinterpret_cast<T *>(m.Qc) : nullptr, m.Un, reinterpret_cast<T *>(m.Unc), m.acc, m.flag, ph);
+        Rpart, FI, m.ef, met, E, stage_coef(mode, stage, dt), Rout, m.Q, Qc, m.Un, Unc, m.acc, m.flag, ph);
   } else {
     return cudaErrorInvalidValue;
   }
