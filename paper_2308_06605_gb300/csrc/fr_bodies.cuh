@@ -691,24 +691,31 @@ constexpr int volume_min_blocks_of() {
 // in 256 measured slower than one warp per element (FP64 with the closure 0.470 and 0.459 against 0.448 ms).
 template <int N>
 __host__ __device__ constexpr int volume_epb() { return N == 2 ? 16 : 1; }
-template <int N>
+// The same at p = 1 on viscous meshes up to this many elements: one element per warp, as long as such blocks (8 per
+// SM) are resident at once.  A thread of the 16-element block does four times as much of the staging and the traces,
+// which the idle lanes do not pay back before the SMs fill.  Volume launch, one element / 16 elements per block:
+// FP64 200 elements 21.4 / 30.7 us, 800 26.5 / 30.6, 1200 31.5 / 31.0, 1600 41.2 / 30.9; with the closure 28.8 /
+// 45.3, 32.9 / 45.3, 41.2 / 46.8, 48.6 / 47.4; double-float 12.5 / 16.9, 13.7 / 16.6, 14.2 / 17.1, 16.6 / 17.0; FP32
+// viscous branch 10.3 / 14.8, 10.9 / 15.1, 11.5 / 15.2, 12.4 / 15.3.
+constexpr int64_t kSingleMax = 8 * 152;
+template <int N, int EPB = volume_epb<N>()>
 __host__ __device__ constexpr int volume_block() {
-  return volume_epb<N>() == 1 ? volume_threads<N>() : (volume_epb<N>() * N * N * N + 31) / 32 * 32;
+  return EPB == 1 ? volume_threads<N>() : (EPB * N * N * N + 31) / 32 * 32;
 }
 
 // Euler runs (VISC = 0): 15 N^3 values of shared memory instead of 35 N^3 + 30 N^2 and no gradient
 // registers, so 1024 threads per SM at 64 registers (704 at p = 6).
-template <int N, typename T, int VISC>
+template <int N, typename T, int VISC, int EPB>
 constexpr int volume_blocks() {
   return VISC == 0 ? (N == 7 ? 2 : (N == 3 ? 32 : 1024 / volume_block<N>()))
-                   : (N == 2 ? 4 : volume_min_blocks_of<N, T>());
+                   : (EPB == 16 ? 4 : volume_min_blocks_of<N, T>());
 }
 
 // Dynamic shared memory of a block.
-template <int N, typename T>
+template <int N, typename T, int EPB = volume_epb<N>()>
 size_t volume_smem(bool viscous, bool closure) {
-  return volume_epb<N>() * (viscous ? sizeof(T) * volume_smem_values<N>() + (closure ? sizeof(float) * closure_floats<N>() : 0)
-                                    : sizeof(T) * 15 * N * N * N);
+  return EPB * (viscous ? sizeof(T) * volume_smem_values<N>() + (closure ? sizeof(float) * closure_floats<N>() : 0)
+                        : sizeof(T) * 15 * N * N * N);
 }
 
 // Few elements: five groups of threads per element, one per variable in the gradient and the divergence (one of
@@ -735,14 +742,14 @@ __global__ void __launch_bounds__(5 * volume_threads<N>())
                                            Qtr, liftfac, Gtr, Rpart, dph, hel, nu_out, if_up, n_interior, cs);
 }
 
-template <int N, typename T, bool FP32V, int VISC>
-__global__ void __launch_bounds__(volume_block<N>(), volume_blocks<N, T, VISC>())
+template <int N, typename T, bool FP32V, int VISC, int EPB = volume_epb<N>()>
+__global__ void __launch_bounds__(volume_block<N, EPB>(), volume_blocks<N, T, VISC, EPB>())
     k_volume(const T *__restrict__ Q, const T *__restrict__ metrics, const int32_t *__restrict__ ef,
              const T *__restrict__ Qtr, const T *__restrict__ liftfac, T *__restrict__ Gtr, T *__restrict__ Rpart,
              DevPhys dph, const double *__restrict__ hel, float *__restrict__ nu_out,
              const int8_t *__restrict__ if_up, int64_t n_interior, int64_t E) {
   extern __shared__ double sm_raw[];
-  constexpr int EPB = volume_epb<N>(), VALS = VISC == 0 ? 15 * N * N * N : volume_smem_values<N>();
+  constexpr int VALS = VISC == 0 ? 15 * N * N * N : volume_smem_values<N>();
   constexpr int NTH = EPB == 1 ? volume_threads<N>() : N * N * N;
   const int64_t e0 = (int64_t)blockIdx.x * EPB;
   const int le = EPB == 1 ? 0 : (int)threadIdx.x / NTH, tid = EPB == 1 ? (int)threadIdx.x : (int)threadIdx.x % NTH;

@@ -137,8 +137,19 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
     if (E > 0 && ph.vc_basis) {
       if ((err = launch_vcjh_phase(m, ph, 1, mode, stage, dt, Rout, st)) != cudaSuccess) return err;
     } else if (E > 0) {
-      // The closure's features need the whole element in one block's warps: scalar kernel.
       bool done = false;
+      if constexpr (N == 2)
+        if (ph.viscous && E <= kSingleMax) {
+          auto k1 = k_volume<N, T, false, 1, 1>;
+          if constexpr (std::is_same<T, df32>::value)
+            if (m.vf32) k1 = k_volume<N, T, true, 1, 1>;
+          err = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)volume_smem<N, T, 1>(true, true));
+          if (err != cudaSuccess) return err;
+          k1<<<(unsigned)E, volume_block<N, 1>(), volume_smem<N, T, 1>(true, ph.closure), st>>>(
+              Qin, met, m.ef, Qtr, lift, Gtr, Rpart, ph, m.h, m.nu, m.if_up, m.n_interior, E);
+          done = true;
+        }
       if constexpr (volume_split_max<N>() > 0)
         if (ph.viscous && E <= volume_split_max<N>()) {
           auto sk = k_volume_split<N, T, false>;
@@ -150,6 +161,7 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
                                                                  m.if_up, m.n_interior);
           done = true;
         }
+      // The packed kernel has no closure.
       if constexpr (std::is_same<T, df32>::value)
         if (!done && !ph.closure) {
           err = !ph.viscous ? launch_pair<N, false, 0>(m, ph, st, done)
