@@ -66,13 +66,14 @@ __global__ void k_min_reduce(const double *__restrict__ x, int64_t n, double *__
 #define FR_EV_END(k) \
   if (ev) cudaEventRecord(ev->stop[k], st)
 
-// The packed volume kernel on this mesh's hexahedra, if it is the faster one (pair_pays); `done` says so.
-template <int N, bool FP32V, int VISC>
+// The packed volume kernel on this mesh's hexahedra, if it is the faster one (pair_built, pair_pays); `done` says so.
+template <int N, bool VISC>
 static cudaError_t launch_pair(const DevMesh &m, const DevPhys &ph, cudaStream_t st, bool &done) {
-  if constexpr (pair_pays<N, FP32V, VISC>()) {
+  if constexpr (pair_built<N, VISC>()) {
+    if (!pair_pays<N, VISC>(m.E)) return cudaSuccess;
     auto df = [](double *p) { return reinterpret_cast<df32 *>(p); };
-    auto pk = k_volume_pair<N, FP32V, VISC>;
-    constexpr int smem = pair_smem<N, FP32V, VISC>();
+    auto pk = k_volume_pair<N, VISC>;
+    constexpr int smem = pair_smem<N, VISC>();
     cudaError_t err = cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (err != cudaSuccess) return err;
     pk<<<(unsigned)((m.E + 1) / 2), volume_threads<N>(), smem, st>>>(df(m.Qc), df(m.metrics), m.ef, df(m.Qtr),
@@ -163,9 +164,8 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
         }
       // The packed kernel has no closure.
       if constexpr (std::is_same<T, df32>::value)
-        if (!done && !ph.closure) {
-          err = !ph.viscous ? launch_pair<N, false, 0>(m, ph, st, done)
-                            : (m.vf32 ? launch_pair<N, true, 1>(m, ph, st, done) : launch_pair<N, false, 1>(m, ph, st, done));
+        if (!done && !ph.closure && (m.vf32 || !ph.viscous)) {
+          err = ph.viscous ? launch_pair<N, true>(m, ph, st, done) : launch_pair<N, false>(m, ph, st, done);
           if (err != cudaSuccess) return err;
         }
       if (!done)

@@ -1,4 +1,5 @@
-// Hexahedral volume kernel with two elements per thread, in packed double-float (or FP32) arithmetic.
+// Hexahedral volume kernel with two elements per thread, in packed arithmetic: the inviscid flux and its
+// divergence in double-float, the viscous branch in FP32 (FR_PREC_MIXED_VF32).
 //
 // With two elements per thread the loads, addresses and loop overhead, a quarter of the scalar kernel's
 // instructions, fill the issue slots that the packed arithmetic (fr_f32x2.cuh) leaves.
@@ -9,64 +10,76 @@
 namespace frx {
 namespace {
 
-// Arithmetic of the viscous branch: pairs of double-float values, or of FP32 (FR_PREC_MIXED_VF32).
-template <typename TG> __device__ __forceinline__ TG to_pg(d2 x);
-template <> __device__ __forceinline__ d2 to_pg<d2>(d2 x) { return x; }
-template <> __device__ __forceinline__ f2 to_pg<f2>(d2 x) { return padd(x.hi, x.lo); }
-__device__ __forceinline__ d2 from_pg(d2 x) { return x; }
-__device__ __forceinline__ d2 from_pg(f2 x) { return d2{x, dupf(0.f)}; }
-template <typename TG> __device__ __forceinline__ TG dup_g(df32 x) { return to_pg<TG>(dup(x)); }
+__device__ __forceinline__ f2 to_f2(d2 x) { return padd(x.hi, x.lo); }
+__device__ __forceinline__ d2 from_f2(f2 x) { return d2{x, dupf(0.f)}; }
+__device__ __forceinline__ f2 dup_f2(df32 x) { return to_f2(dup(x)); }
 
-template <typename TG>
-__device__ __forceinline__ PhysT<TG> pair_phys(const PhysT<df32> &p) {
-  PhysT<TG> r;
-  r.cT = dup_g<TG>(p.cT);
-  r.mu = dup_g<TG>(p.mu);
-  r.m2mu3 = dup_g<TG>(p.m2mu3);
-  r.kappa = dup_g<TG>(p.kappa);
+__device__ __forceinline__ PhysT<f2> pair_phys(const PhysT<df32> &p) {
+  PhysT<f2> r;
+  r.cT = dup_f2(p.cT);
+  r.mu = dup_f2(p.mu);
+  r.m2mu3 = dup_f2(p.m2mu3);
+  r.kappa = dup_f2(p.kappa);
   return r;
 }
 
-// Bytes of shared memory per pair of elements: state (FP32 branch: its perturbation) 5, gradient 15 and flux 15 per point, jumps 30
-// per N^2; an inviscid run keeps the flux only.
-template <int N, bool FP32V, int VISC>
+// Bytes of shared memory per pair of elements: state perturbation 5, gradient 15 (FP32) and flux 15 (double-float) per
+// point, jumps 30 per N^2; an inviscid run keeps the flux only.
+template <int N, bool VISC>
 constexpr int pair_smem() {
-  constexpr int Np = N * N * N, Nf = N * N, G = FP32V ? 8 : 16;
-  return VISC ? 20 * Np * G + 15 * Np * 16 + 30 * Nf * G : 15 * Np * 16;
+  constexpr int Np = N * N * N, Nf = N * N;
+  return VISC ? 20 * Np * 8 + 15 * Np * 16 + 30 * Nf * 8 : 15 * Np * 16;
 }
-template <int N, bool FP32V, int VISC>
+template <int N, bool VISC>
 constexpr int pair_blocks() {
   // By shared memory (227 KB per SM), and not below 128 registers per thread.
-  constexpr int by_smem = 227 * 1024 / (pair_smem<N, FP32V, VISC>() + 1024);
+  constexpr int by_smem = 227 * 1024 / (pair_smem<N, VISC>() + 1024);
   constexpr int by_regs = 512 / volume_threads<N>();
   return by_smem < by_regs ? by_smem : (by_regs > 0 ? by_regs : 1);
 }
 
-// Where it runs, and what the volume kernel takes per launch against the scalar one (GB300).  It halves the
+// Orders it is built for, and what the volume kernel takes per launch against the scalar one (GB300).  It halves the
 // warps of an SM for the same shared memory, so it gains where enough of them remain: FP32 viscous branch
-// 40^3 p = 3 0.623 -> 0.572 ms, 32^3 p = 4 0.643 -> 0.600, 28^3 p = 5 0.844 -> 0.740, 20^3 p = 7 0.937 -> 0.842
-// (not p = 2: 0.324 -> 0.331, p = 6: 0.912 -> 0.946); double-float 40^3 p = 2 0.463 -> 0.449, p = 3 0.985 -> 0.946
-// (not 48^3 p = 4: 3.09 -> 3.51 with 8 warps per SM, 3.21 with 12 at less shared memory); inviscid 40^3 p = 2
-// 0.097 -> 0.087, p = 3 0.210 -> 0.191, 32^3 p = 4 0.244 -> 0.231.
-template <int N, bool FP32V, int VISC>
-constexpr bool pair_pays() {
-  return VISC == 0 ? (!FP32V && N >= 3 && N <= 5) : (FP32V ? (N == 4 || N == 5 || N == 6 || N == 8) : (N == 3 || N == 4));
+// 40^3 p = 3 0.638 -> 0.571 ms, 4800 elements p = 4 0.106 -> 0.097, p = 5 0.193 -> 0.170, p = 7 0.562 -> 0.493 (not
+// p = 2: 0.324 -> 0.331 at 40^3, p = 6: 0.912 -> 0.946 at 24^3); inviscid 40^3 p = 2 0.098 -> 0.086, p = 3 0.209 -> 0.191,
+// 4800 elements p = 4 0.042 -> 0.041.  With the viscous branch in double-float it was slower at every size (40^3
+// p = 2 0.445 -> 0.460, p = 3 0.938 -> 0.960, 48^3 p = 4 3.09 -> 3.51).
+template <int N, bool VISC>
+constexpr bool pair_built() {
+  return VISC ? N == 4 || N == 5 || N == 6 || N == 8 : N >= 3 && N <= 5;
+}
+
+// Element counts it pays at.  A block of it lasts longer than one of the scalar kernel, and there are half as many, so
+// on meshes of a few elements per SM (152) the scalar kernel is through first; where exactly depends on how
+// the blocks of either fill the SMs.  Volume launch, pair / scalar, us:
+//   FP32 viscous p = 3:  308 elements 14.5 / 13.6, 800 17.8 / 16.4, 1200 18.5 / 18.5, 1600 22.4 / 24.8
+//     (2400: 33.4 / 33.0), 4800 53.8 / 57.6;
+//   p = 4:  153 14.6 / 14.0, 308 18.4 / 16.3, 400 18.6 / 16.4, 500 18.6 / 18.4, 600 18.6 / 18.7, 800 22.7 / 26.1;
+//   p = 5:  100 16.5 / 14.5, 153 16.7 / 18.4, 250 16.7 / 18.8, 308 24.6 / 23.0, 400 25.0 / 24.4, 500 25.4 / 29.8;
+//   p = 7:  100 31.4 / 20.9, 153 31.6 / 35.1, 250 32.2 / 37.0, 308 56.2 / 51.2, 400 58.5 / 52.1, 500 60.6 / 69.0;
+//   inviscid p = 2:  100 7.9 / 6.8, 600 8.1 / 7.9, 1200 8.3 / 8.3, 1600 8.8 / 8.3, 2400 9.0 / 10.1;
+//   p = 3:  100 8.0 / 7.5, 308 8.3 / 8.1, 800 9.7 / 8.5, 1200 10.0 / 10.2, 1600 11.3 / 12.2;
+//   p = 4:  100 8.3 / 7.9, 308 10.2 / 9.2, 400 10.4 / 9.8, 500 10.4 / 10.4, 600 10.3 / 10.8, 1200 14.5 / 14.9.
+// At p = 5 and 7 one pair block per SM beats the second scalar block, two do not beat the third.
+template <int N, bool VISC>
+bool pair_pays(int64_t E) {
+  if (VISC && N >= 6) return E > 152 && (E <= 2 * 152 || E > 3 * 152);
+  return E > 152 * (VISC ? (N == 4 ? 8 : 4) : (N == 3 ? 12 : (N == 4 ? 8 : 3)));
 }
 
 // One thread per solution point of the elements e0 and e1; the operations of volume_body in its order.  An odd
 // mesh's last block holds one element twice: both lanes then store the same values.
-template <int N, bool FP32V, int VISC>
-__global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VISC>())
+template <int N, bool VISC>
+__global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, VISC>())
     k_volume_pair(const df32 *__restrict__ Q, const df32 *__restrict__ metrics, const int32_t *__restrict__ ef,
                   const df32 *__restrict__ Qtr, const df32 *__restrict__ liftfac, df32 *__restrict__ Gtr,
                   df32 *__restrict__ Rpart, DevPhys dph, const int8_t *__restrict__ if_up, int64_t n_interior, int64_t E) {
   extern __shared__ float4 sm_pair[];
   constexpr int Np = N * N * N, Nf = N * N, nth = volume_threads<N>();
-  using TG = typename std::conditional<FP32V, f2, d2>::type;
   d2 *sH = reinterpret_cast<d2 *>(sm_pair);                    // [15][Np] transformed flux, index d*5+v
-  TG *sQ = reinterpret_cast<TG *>(sH + 15 * Np);               // [5][Np] state; FP32: less the first point's
-  TG *sG = sQ + 5 * Np;                                        // [15][Np] uncorrected gradient, j*5+v
-  TG *sdQ = sG + 15 * Np;                                      // [6][5][Nf] Q^I - Q_own at the flux points
+  f2 *sQ = reinterpret_cast<f2 *>(sH + 15 * Np);               // [5][Np] perturbation from the first point
+  f2 *sG = sQ + 5 * Np;                                        // [15][Np] uncorrected gradient, j*5+v
+  f2 *sdQ = sG + 15 * Np;                                      // [6][5][Nf] Q^I - Q_own at the flux points
   const int64_t e0 = (int64_t)blockIdx.x * 2, e1 = e0 + 1 < E ? e0 + 1 : e0;
   const int tid = threadIdx.x;
   const BasisT<df32> &B = cbasis<df32>(N);
@@ -80,10 +93,9 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
     for (int c = 0; c < 9; ++c) S[c] = pack(m0[c * Np], m1[c * Np]);
     invJ = pack(m0[9 * Np], m1[9 * Np]);
   }
-  if constexpr (VISC != 0) {
+  if constexpr (VISC) {
     for (int t = tid; t < 5 * Np; t += nth)
-      sQ[(t % 5) * Np + t / 5] = FP32V ? to_pg<TG>(pack(Q0[t], Q1[t]) - pack(Q0[t % 5], Q1[t % 5]))
-                                       : to_pg<TG>(pack(Q0[t], Q1[t]));
+      sQ[(t % 5) * Np + t / 5] = to_f2(pack(Q0[t], Q1[t]) - pack(Q0[t % 5], Q1[t % 5]));
     for (int t = tid; t < 6 * Nf; t += nth) {
       const int f = t / Nf, r = t % Nf;
       const df32 *own[2], *oth[2];
@@ -100,35 +112,35 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
       }
 #pragma unroll
       for (int v = 0; v < 5; ++v)
-        sdQ[(f * 5 + v) * Nf + r] = to_pg<TG>(scale2(
+        sdQ[(f * 5 + v) * Nf + r] = to_f2(scale2(
             pack(oth[0][v * Nf], oth[1][v * Nf]) - pack(own[0][v * Nf], own[1][v * Nf]), mkf2(w[0], w[1])));
     }
   }
   __syncthreads();
-  TG G[15];
+  f2 G[15];
   if (pt) {
 #pragma unroll
     for (int v = 0; v < 5; ++v) q[v] = pack(Q0[m * 5 + v], Q1[m * 5 + v]);
-    if constexpr (VISC != 0) {
-      TG sj[9];   // S[d][jj] / |J|
+    if constexpr (VISC) {
+      f2 sj[9];   // S[d][jj] / |J|
 #pragma unroll
-      for (int c = 0; c < 9; ++c) sj[c] = to_pg<TG>(S[c] * invJ);
-      constexpr int R = sizeof(d2) / sizeof(TG);
-      TG *sGc = reinterpret_cast<TG *>(sH);
+      for (int c = 0; c < 9; ++c) sj[c] = to_f2(S[c] * invJ);
+      constexpr int R = sizeof(d2) / sizeof(f2);
+      f2 *sGc = reinterpret_cast<f2 *>(sH);
       auto gslot = [&](int c) { return ((c / R) * Np + m) * R + c % R; };
 #pragma unroll 1
       for (int d = 0; d < 3; ++d) {
         const int row = d == 0 ? i : (d == 1 ? j : k), st = axis_stride<N>(d), at = m - row * st;
         const int r = d == 0 ? j + N * k : (d == 1 ? i + N * k : i + N * j);
-        TG c[N];
+        f2 c[N];
 #pragma unroll
-        for (int a = 0; a < N; ++a) c[a] = dup_g<TG>(B.D[row * N + a]);
-        const TG hlo = -dup_g<TG>(B.hm[row]), hhi = dup_g<TG>(B.hp[row]);
-        const TG *dq = sdQ + d * 10 * Nf + r;
+        for (int a = 0; a < N; ++a) c[a] = dup_f2(B.D[row * N + a]);
+        const f2 hlo = -dup_f2(B.hm[row]), hhi = dup_f2(B.hp[row]);
+        const f2 *dq = sdQ + d * 10 * Nf + r;
 #pragma unroll 1
         for (int v = 0; v < 5; ++v) {
-          const TG jlo = dq[v * Nf], jhi = dq[(5 + v) * Nf];
-          Dot<TG> s(c[0], sQ[v * Np + at]);
+          const f2 jlo = dq[v * Nf], jhi = dq[(5 + v) * Nf];
+          Dot<f2> s(c[0], sQ[v * Np + at]);
 #pragma unroll
           for (int a = 1; a < N; ++a) s.add(c[a], sQ[v * Np + at + a * st]);
           sG[(d * 5 + v) * Np + m] = s.raw();
@@ -139,7 +151,7 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
       }
 #pragma unroll 1
       for (int v = 0; v < 5; ++v) {
-        TG gu[3], gc[3];
+        f2 gu[3], gc[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
           gu[d] = sG[(d * 5 + v) * Np + m];
@@ -147,8 +159,8 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
         }
 #pragma unroll
         for (int jj = 0; jj < 3; ++jj) {
-          const TG du = dot3(sj[jj], gu[0], sj[3 + jj], gu[1], sj[6 + jj], gu[2]);
-          const TG dc = dot3(sj[jj], gc[0], sj[3 + jj], gc[1], sj[6 + jj], gc[2]);
+          const f2 du = dot3(sj[jj], gu[0], sj[3 + jj], gu[1], sj[6 + jj], gu[2]);
+          const f2 dc = dot3(sj[jj], gc[0], sj[3 + jj], gc[1], sj[6 + jj], gc[2]);
           sGc[gslot(jj * 5 + v)] = dc;
           // Face-gradient source: BR2 the uncorrected gradient (+ eta r_f), LDG the corrected one.
           sG[(jj * 5 + v) * Np + m] = dph.ldg ? dc : du;
@@ -161,27 +173,21 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
     const d2 u[3] = {q[1] * ri, q[2] * ri, q[3] * ri};
     const d2 p = dup(dph.f.gm1) * (q[4] - scale2(dot3(q[1], u[0], q[2], u[1], q[3], u[2]), 0.5f));
     d2 tau[6], hq[3], mom[6], en[3];
-    if constexpr (VISC != 0) {
-      const PhysT<TG> pg = pair_phys<TG>(dph.f);
-      TG qg[5], ug[3], taug[6], hqg[3], rig;
+    if constexpr (VISC) {
+      const PhysT<f2> pg = pair_phys(dph.f);
+      f2 qg[5], ug[3], taug[6], hqg[3], rig;
 #pragma unroll
-      for (int v = 0; v < 5; ++v) qg[v] = to_pg<TG>(q[v]);
-      if constexpr (FP32V) {
-        rig = reciprocal(qg[0]);
+      for (int v = 0; v < 5; ++v) qg[v] = to_f2(q[v]);
+      rig = reciprocal(qg[0]);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) ug[c] = qg[1 + c] * rig;
-      } else {
-        rig = ri;
+      for (int c = 0; c < 3; ++c) ug[c] = qg[1 + c] * rig;
+      viscous_stress<f2>(qg, ug, rig, G, pg, visc_of(pg), taug, hqg);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) ug[c] = u[c];
-      }
-      viscous_stress<TG>(qg, ug, rig, G, pg, visc_of(pg), taug, hqg);
+      for (int a = 0; a < 3; ++a) hq[a] = from_f2(hqg[a]);
 #pragma unroll
-      for (int a = 0; a < 3; ++a) hq[a] = from_pg(hqg[a]);
-#pragma unroll
-      for (int a = 0; a < 6; ++a) tau[a] = from_pg(taug[a]);
+      for (int a = 0; a < 6; ++a) tau[a] = from_f2(taug[a]);
     }
-    physical_flux<d2>(q, u, p, VISC != 0, tau, hq, mom, en);
+    physical_flux<d2>(q, u, p, VISC, tau, hq, mom, en);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       d2 f[5];
@@ -191,14 +197,14 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
     }
   }
   __syncthreads();
-  if constexpr (VISC != 0) {
+  if constexpr (VISC) {
     for (int t = tid; t < 9 * Nf; t += nth) {
       const int jj = t / (3 * Nf), dr = t - jj * 3 * Nf;
       const int d = dr / Nf, r = dr % Nf;
       int base, sd;
       face_line<N>(2 * d, r, base, sd);
       df32 *dst[2][2];
-      TG lj[2];
+      f2 lj[2];
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
         const int f = 2 * d + s;
@@ -208,24 +214,24 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, FP32V, VIS
           const int64_t I = packed >> 4;
           dst[s][l] = Gtr + (I * 2 + ((packed >> 3) & 1)) * 15 * Nf + slot_of(packed & 7, r % N, r / N, N) + jj * 5 * Nf;
         }
-        lj[s] = to_pg<TG>(dup(dph.f.eta) *
+        lj[s] = to_f2(dup(dph.f.eta) *
                           pack(liftfac[((e0 * 6 + f) * 3 + jj) * Nf + r], liftfac[((e1 * 6 + f) * 3 + jj) * Nf + r]));
       }
 #pragma unroll 1
       for (int v = 0; v < 5; ++v) {
-        const TG *sg = sG + (jj * 5 + v) * Np + base;
-        TG x[N];
+        const f2 *sg = sG + (jj * 5 + v) * Np + base;
+        f2 x[N];
 #pragma unroll
         for (int c = 0; c < N; ++c) x[c] = sg[c * sd];
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
-          auto l = [&](int c) { return dup_g<TG>(s ? B.lp[c] : B.lm[c]); };
-          const TG jump = sdQ[((2 * d + s) * 5 + v) * Nf + r];
-          Dot<TG> acc(l(0), x[0]);
+          auto l = [&](int c) { return dup_f2(s ? B.lp[c] : B.lm[c]); };
+          const f2 jump = sdQ[((2 * d + s) * 5 + v) * Nf + r];
+          Dot<f2> acc(l(0), x[0]);
 #pragma unroll
           for (int c = 1; c < N; ++c) acc.add(l(c), x[c]);
           acc.add(lj[s], jump);
-          const d2 g = from_pg(acc.raw());
+          const d2 g = from_f2(acc.raw());
           dst[s][0][v * Nf] = lane0(g);
           dst[s][1][v * Nf] = lane1(g);
         }

@@ -63,6 +63,21 @@ def test_volume_kernels_above_the_small_mesh_limit(p, box, kind, viscous):
             assert_state_parity(g.get_state(), Q1, S, dt, bar)
 
 
+# Odd element counts at which the kernel with two elements per thread runs (FP32 viscous branch, or no viscous branch in
+# double-float), its last block with one.
+@pytest.mark.parametrize("p,box,viscous", [(3, (11, 11, 11), 1), (3, (11, 11, 11), 2), (4, (9, 9, 9), 1), (4, (9, 9, 9), 2),
+                                           (5, (7, 5, 5), 1), (5, (7, 5, 5), 2), (5, (9, 9, 7), 2), (2, (13, 13, 11), 0), (3, (11, 11, 11), 0), (4, (9, 9, 7), 0)])
+def test_two_elements_per_thread(p, box, viscous):
+    d, ph, state = _case("walls" if viscous == 2 else "periodic", box)
+    ph.viscous = viscous
+    ora = HexFR(d, ph, p)
+    Q = np.ascontiguousarray(state(ora.x))
+    ph.precision = fr.FR_PREC_MIXED_VF32 if viscous else fr.FR_PREC_MIXED
+    with fr.Mesh(d, ph, p) as g:
+        g.set_state(Q)
+        assert_residual_parity(g.residual(), ora.residual(Q), ora.residual(Q, magnitude=True), 2e-8 if viscous else 1e-9)
+
+
 @pytest.mark.parametrize("p,box", [(3, (9, 9, 9)), (4, (7, 7, 7))])
 def test_staged_correction_without_source(p, box):
     d, ph, state = _case("periodic", box)
