@@ -9,7 +9,10 @@ One step = one RK44 time step = 4 RK stages (each: residual + stage update); the
 solution points x stages per second.  Inputs are synthetic and seeded; the device working set
 (~18 GB) is far larger than L2, so no flush is needed between iterations.
 
-Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
+Prints one JSON line of at most 1500 characters with the headline, the end-to-end rate and the p = 3..7 rates
+(`headline`); --detail FILE writes everything that was measured.
+
+Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--detail FILE]
 Under torchrun (N > 1) every rank runs an independent replica on its own GPU (weak scaling by
 replicas; the domain-decomposed stage with halo exchange, fr_part_phase, is not timed across GPUs
 here), timing is max over ranks.
@@ -185,10 +188,11 @@ def run_reference(args):
 
 # ------------------------------------------------------------------------------ GPU path
 SWEEP = [(64, 3), (64, 4), (48, 5), (40, 6), (32, 7)]   # (elements per edge, p): 17-33 M points
-# A double-float multiply-add (2 algorithmic flops) is 18 FP32 instructions (7 for the product,
-# 11 for the sum); the FP32 peak in FLOP/s counts an FFMA instruction as 2 flops, so the
-# double-float peak in algorithmic FLOP/s is fp32_peak / 2 instructions/s * 2 / 18 = fp32_peak / 18.
-DF_FP32_FLOPS_PER_FLOP = 18.0
+# A term of a compensated double-float sum (2 algorithmic flops) is 12 FP32 instructions (4 for the
+# product with its error and cross terms, 6 for the sum with its error, 2 to collect the errors); the FP32 peak in
+# FLOP/s counts an FFMA instruction as 2 flops, so the double-float peak in algorithmic FLOP/s is
+# fp32_peak / 2 instructions/s * 2 / 12 = fp32_peak / 12.
+DF_FP32_FLOPS_PER_FLOP = 12.0
 
 
 class Case:
@@ -518,13 +522,13 @@ def run_ours(args):
         dom = max(k, key=lambda n_: k[n_]["share"])
         peak = perfmodel.mixed_alu_peak(ORDER, df_peak, fp32_peak, fp32_viscous) if dom == "volume" else df_peak
         ach = k[dom]["gflops"] * 1e9
-        src = ("measured FP32 FMA rate (fr_probe_fma) / 18 (a double-float multiply-add is 18 FP32 instructions "
-               "for 2 algorithmic flops)")
+        src = ("measured FP32 FMA rate (fr_probe_fma) / 12 (a term of a compensated double-float sum is 12 FP32 "
+               "instructions for 2 algorithmic flops)")
         if fp32_viscous and dom == "volume":
             src = ("the kernel's arithmetic mix at measured rates: the viscous branch's flops at the FP32 FMA rate, "
-                   "the rest at that rate / 18 (times added)")
+                   "the rest at that rate / 12 (times added)")
         return {"bound": "alu", "kernel": dom, "precision": tag, "achieved": ach / 1e12, "peak": peak / 1e12,
-                "unit": "TFLOP/s", "frac": ach / peak, "traffic": TRAFFIC.get((tag, ORDER, N_EDGE, dom)),
+                "unit": "TFLOP/s", "frac": ach / peak, "traffic": None,
                 "peak_source": src, "algorithmic_flops_per_point": fl[dom], "algorithmic_bytes_per_point": by[dom]}
 
     roofline = mixed_roofline(k_mx, False, "mixed")
@@ -534,7 +538,7 @@ def run_ours(args):
     fp64 = {"value": value64, "ms_per_step": ms_64 / args.steps, "kernels": k_64,
             "roofline": {"bound": "alu", "kernel": dom64, "achieved": k_64[dom64]["gflops"] / 1e3,
                          "peak": fp64_peak / 1e12, "unit": "TFLOP/s", "frac": k_64[dom64]["gflops"] * 1e9 / fp64_peak,
-                         "traffic": TRAFFIC.get(("fp64", ORDER, N_EDGE, dom64)),
+                         "traffic": None,
                          "peak_source": "measured FP64 DFMA rate (fr_probe_fma)"}}
     c64.close()
 
@@ -624,7 +628,7 @@ def run_ours(args):
                 ms = c.timed(2)
                 row[prec] = n ** 3 * (p + 1) ** 3 * 4 * 2 / (ms * 1e-3)
                 # Per-kernel CUDA-event times and each kernel's fraction of the arithmetic peak of
-                # its precision (FP64: the DFMA rate; double-float: the FP32 FMA rate / 18; the
+                # its precision (FP64: the DFMA rate; double-float: the FP32 FMA rate / 12; the
                 # volume kernel with the viscous branch in FP32: its arithmetic mix at those rates).
                 peak = fp64_peak if prec == "fp64" else df_peak
                 k = c.kernels(2, p)
@@ -669,14 +673,35 @@ def run_ours(args):
     if world > 1:
         torch.distributed.destroy_process_group()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as fh:
+                json.dump(line, fh)
+        print(json.dumps(headline(line)), flush=True)
     return 0
 
 
-# DRAM traffic per launch of the dominant kernel from ncu captures (precision, p, n_edge, kernel)
-# -> bytes; scaled from a 32^3 capture by the element count.  Only valid for the kernel version
-# that was profiled.
-TRAFFIC = {("fp64", 4, 64, "volume"): 8 * 1.52181e9, ("mixed", 4, 64, "volume"): 8 * 1.51813e9}
+def headline(full):
+    """The printed line: the contract's keys and the rates of every order and precision, in at most 1500
+    characters (records of a run keep the end of its output; a longer line was cut and lost)."""
+    def digits(x, n):
+        return float(f"{x:.{n}g}") if isinstance(x, float) else x
+
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "clocks")
+    out = {k: digits(full[k], 7) for k in keys}
+    out["e2e"] = {k: digits(full["e2e"][k], 7) for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")}
+    out["gpu_launches"] = full["gpu_launches"]
+    out["roofline"] = {k: digits(full["roofline"][k], 4) for k in ("bound", "kernel", "achieved", "peak", "unit", "frac")}
+    out["l2_error_vs_fp64"] = digits(max(full["error_vs_fp64"]["l2_rel"].values()), 3)
+    # [FP64, double-float, FP32 viscous branch]
+    out["updates_per_s"] = {f"p{ORDER}": [digits(v, 4) for v in (full["fp64"]["value"], full["value"],
+                                                               full["fp32_viscous_branch"]["value"])]}
+    for p, row in full["p_sweep_updates_per_s"].items():
+        out["updates_per_s"].setdefault(p, [digits(row[k], 4) for k in ("fp64", "mixed", "mixed_vf32")])
+    if "cpu_baseline" in full:
+        out["cpu_baseline"] = {k: digits(full["cpu_baseline"][k], 5) for k in ("value", "unit", "cores", "kind")}
+        out["cpu_baseline"]["sample"] = "oracle RK44, 8^3 hex p=4 TGV, one replica per core"
+    return out
 
 
 def main():
@@ -685,6 +710,7 @@ def main():
     ap.add_argument("--steps", type=int, default=5)
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
+    ap.add_argument("--detail", default="", help="write everything that was measured to this file (JSON)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-sweep", action="store_true", help="skip the p = 3..7 sweep")
     ap.add_argument("--no-ensemble", action="store_true", help="skip the 64-case batched vortex ensemble")
