@@ -328,9 +328,9 @@ class Mesh:
 
     def set_state(self, Q):
         p, where = _data_ptr(Q)
-        n, have = int(np.prod(self.shape)), Q.size if isinstance(Q, np.ndarray) else Q.numel()
-        if have < n:
-            raise ValueError(f"set_state: {have} values, the mesh's state has {n}")
+        have = Q.size if isinstance(Q, np.ndarray) else Q.numel()
+        if have < 5 * self.n_points:
+            raise ValueError(f"set_state: {have} values, the mesh's state has {5 * self.n_points}")
         self._check(self._lib.fr_set_state(self._h, p, where))
 
     def get_state(self, out=None):
