@@ -356,12 +356,12 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
     for (int c = 0; c < 9; ++c) S[c] = met[c * Np];
     invJ = met[9 * Np];
   }
-  if (active && VISC != 0)
+  // The state goes through shared memory for the gradient only.
+  if (active && viscous)
     for (int t = tid; t < 5 * Np; t += nth) {
       const T x = Q[e * Np * 5 + t];
       sQ[(t % 5) * Np + t / 5] = x;
-      if constexpr (kPert)
-        if (viscous) sQg[(t % 5) * Np + t / 5] = to_g<TG>(x - Q[e * Np * 5 + t % 5]);
+      if constexpr (kPert) sQg[(t % 5) * Np + t / 5] = to_g<TG>(x - Q[e * Np * 5 + t % 5]);
     }
   if (viscous && active) {
     for (int t = tid; t < 6 * Nf; t += nth) {
@@ -391,7 +391,7 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   if (mine) {
     if (pt)
 #pragma unroll
-      for (int v = 0; v < 5; ++v) q[v] = VISC == 0 ? Q[(e * Np + m) * 5 + v] : sQ[v * Np + m];
+      for (int v = 0; v < 5; ++v) q[v] = viscous ? sQ[v * Np + m] : Q[(e * Np + m) * 5 + v];
     if (viscous) {
       // S[d][jj] / |J|.  Double-float transforms the uncorrected and the corrected gradient as the two lanes
       // of packed instructions (their parts wait in shared memory lane by lane: (hi, hi) in sG, (lo, lo) in sGc).
