@@ -104,8 +104,9 @@ __device__ __forceinline__ df32 &operator*=(df32 &x, df32 y) { return x = x * y;
 
 // 1/x by Newton-Raphson iteration from the hardware's approximation: y (FP32, one step), then the
 // correction y (e + e^2) with e = 1 - x y taken from both parts of x.  10 FP32 instructions and no branch
-// (the quotient above: two IEEE divisions with their slow paths); relative error below 2^-47, the
-// rounding of the correction.
+// (the quotient above: two IEEE divisions with their slow paths).  |e| < 2^-23, so the four roundings of the
+// correction (two in e, the sum e + e^2, the product with y) are 2^-48 of 1/x at most each: relative error below
+// 2^-46.  1/0 and 1/inf come out as NaN.
 __device__ __forceinline__ float rcp_newton(float x) {
   float y;
   asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));

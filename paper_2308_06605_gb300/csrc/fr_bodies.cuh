@@ -286,9 +286,8 @@ __host__ __device__ constexpr int volume_threads() { return ((N * N * N + 31) / 
 template <int N>
 constexpr int volume_min_blocks() {
   // Measured on GB300: 16 warps per SM (128 registers) is fastest for the 32- and 64-thread
-  // blocks of p = 2, 3 and, with the per-variable gradient and the contravariant fluxes, for the
-  // 128-thread blocks of p = 4 (4 blocks, no spills in double-float; 3 blocks of 168 registers
-  // were 3 % slower); p = 1 keeps 8 blocks (16 would spill).
+  // blocks of p = 2, 3 and for the 128-thread blocks of p = 4 (4 blocks; 3 blocks of 168 registers were
+  // 3 % slower); p = 1 keeps 8 blocks (16 would spill).
   return N == 2 ? 8 : (N == 5 ? 4 : (volume_threads<N>() <= 128 ? 512 / volume_threads<N>()
                                                                  : (volume_threads<N>() <= 256 ? 2 : 1)));
 }
@@ -337,10 +336,10 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
   const BasisT<T> &B = basis_ref<N, T, VC>(dph);
   // Sums of products end with raw(): the compensated sum renormalised by one fast_two_sum only (an
   // error of the order of 2^-48 of the sum of the terms' magnitudes).  All of them are compensated sums
-  // (Dot).  Summing the gradient and its traces on top of a large offset instead (7 FP32 instructions per term for
-  // 12) took 3 % off this kernel at 48^3 p = 4 (3.13 -> 3.05 ms), but a variable of zero mean lost up to three
-  // bits: at p = 7 and Re 0.1 the momentum residual's error grew from 1.4e-11 to 5.0e-11 on hexahedra and from 2.0e-11 to
-  // 1.8e-10 on prisms.  Transform and traces use packed instructions in double-float (48^3 p = 4 3.09 -> 3.00 ms,
+  // (Dot).  Summing the gradient and its traces on top of a large offset instead (7 FP32 instructions per
+  // term for 12) took 3 % off this kernel at 48^3 p = 4 (3.13 -> 3.05 ms), but a variable of zero mean lost up to
+  // three bits: at p = 7 and Re 0.1 the momentum residual's error grew from 1.4e-11 to 5.0e-11 on hexahedra and
+  // from 2.0e-11 to 1.8e-10 on prisms.  Transform and traces use packed instructions in double-float (48^3 p = 4 3.09 -> 3.00 ms,
   // 28^3 p = 5 1.174 -> 1.154, but 24^3 p = 6 1.30 -> 1.315 with its spills; packing the gradient's and the flux's
   // variables in pairs as well measured 3.03).  The kernel is bound by FP32 issue.
   const bool viscous = VISC == 2 ? dph.viscous != 0 : VISC == 1;
@@ -676,8 +675,8 @@ __device__ __forceinline__ void volume_body(int64_t e, int tid, int nth, bool ac
 
 // Resident blocks per order and arithmetic, each measured (GB300).  p = 5 and 6: 3 blocks of 224 and
 // (double-float) 2 of 352 threads at 80 registers, with some spills, beat the register-limited 2 and
-// 1; FP64 p = 6 keeps 1 block.  Double-float at p = 2, 3, 4: 20, 10 and 5 blocks (96 registers, no
-// spills) beat 16, 8 and 4, since the gradient holds one row of D instead of three: 40^3 p = 2 0.485 -> 0.463
+// 1; FP64 p = 6 keeps 1 block.  Double-float at p = 2, 3, 4: 20, 10 and 5 blocks (96 registers, 8
+// to 24 bytes of spills at p = 2 and 4) beat 16, 8 and 4, since the gradient holds one row of D instead of three: 40^3 p = 2 0.485 -> 0.463
 // ms per launch, 40^3 p = 3 1.023 -> 0.985 ms, 48^3 p = 4 3.27 -> 3.09 ms.  With the viscous branch in FP32 the
 // same counts (6 and 12 at p = 4 and 3 measure the same).
 template <int N, typename T>
@@ -725,8 +724,8 @@ size_t volume_smem(bool viscous, bool closure) {
 // double-float 64 at p = 2 18.5 -> 10.4, 216 at p = 3 18.5 -> 12.3, 64 at p = 4 14.8 -> 14.5.  Limits: where the SMs
 // fill up it costs an extra barrier and the four groups' idle time at the fluxes (FP64 p = 2 18.7 against
 // 28.7 us at 216 elements but 34.3 against 29.2 at 512, p = 3 25.0 against 30.0 and 44.6 against 41.5, p = 4
-// 47.5 against 43.6 at 216), so two elements per SM at p = 2 and 3 and one at p = 4.  p = 1 puts 16 elements in
-// a block, p >= 5 has seven and more warps per element anyway.
+// 47.5 against 43.6 at 216), so two elements per SM at p = 2 and 3 and one at p = 4.  p = 1 has a quarter of a warp
+// per element, p >= 5 seven warps and more.
 template <int N>
 constexpr int64_t volume_split_max() { return N == 3 || N == 4 ? 2 * 152 : (N == 5 ? 152 : 0); }
 
@@ -844,18 +843,19 @@ __device__ __forceinline__ void iface_body(int64_t t, const T *__restrict__ Qtr,
 
 // 5 resident blocks of 128 threads (96 registers, no spills with the Rusanov flux; the Roe flux is an
 // instantiation of its own, which would otherwise set the registers of both), 6 with the FP32 viscous
-// part.  Measured at 5 / 6 blocks: double-float 48^3 p = 4 0.682 / 0.747 ms (0.691 since the FP32 to FP64 conversions moved to the integer pipe), FP64 32^3 p = 4 0.843 / 0.857
-// ms, FP32 viscous 40^3 p = 3 0.231 / 0.220 ms.  Before the viscous flux was formed along the normal and
+// part.  Measured at 5 / 6 blocks: double-float 48^3 p = 4 0.682 / 0.747 ms (0.691 since the FP32 to FP64
+// conversions moved to the integer pipe), FP64 32^3 p = 4 0.843 / 0.857 ms, FP32 viscous 40^3 p = 3 0.231 / 0.220 ms
+// (0.199 with the same conversions).  The double-float Roe instantiations spill 80 to 196 bytes.  Before the viscous flux was formed along the normal and
 // the Roe branch split off: 0.869, 1.072 and 0.232 ms (memory floor 0.48 ms at 48^3; FP64 is bound by its
 // pipe: 185 operations per point instead of 240, Roe 330 instead of 500).
 template <bool FP32V>
 constexpr int iface_blocks() { return FP32V ? 6 : 5; }
 
 template <int N, typename T, bool FP32V, bool ROE>
-__global__ void __launch_bounds__(128, iface_blocks<FP32V>()) k_iface_flux(const T *__restrict__ Qtr, const T *__restrict__ Gtr,
-                             const T *__restrict__ normals, T *__restrict__ FI, int64_t n_if, DevPhys dph,
-                             const int32_t *__restrict__ if_elem, const float *__restrict__ nu,
-                             const int8_t *__restrict__ if_up) {
+__global__ void __launch_bounds__(128, iface_blocks<FP32V>())
+    k_iface_flux(const T *__restrict__ Qtr, const T *__restrict__ Gtr, const T *__restrict__ normals, T *__restrict__ FI,
+                 int64_t n_if, DevPhys dph, const int32_t *__restrict__ if_elem, const float *__restrict__ nu,
+                 const int8_t *__restrict__ if_up) {
   iface_body<N, T, FP32V, ROE>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, Qtr, Gtr, normals, FI, n_if, dph,
                                if_elem, nu, if_up);
 }
@@ -1070,8 +1070,8 @@ __device__ __forceinline__ void correct_body(int64_t t, const T *__restrict__ Rp
 
 // Up to 256 points per SM (one block of the kernel below on each): one thread per point in blocks of one
 // warp, which spreads the chain of loads and FP64 instructions over more schedulers and has no
-// staging barriers.  FP64 8^3 p = 3 12.6 -> 10.6 us per launch, 4^3 p = 2 10.4 -> 8.6, double-float 8^3 p = 3 10.9 -> 9.3;
-// at 64000 points 14.4 against 14.7 us, and at 32^3 p = 4 0.398 ms staged against 0.431.
+// staging barriers.  FP64 8^3 p = 3 12.6 -> 10.6 us per launch, 4^3 p = 2 10.4 -> 8.6, double-float 8^3 p = 3 10.9 ->
+// 9.3; at 64000 points 14.4 against 14.7 us, and at 32^3 p = 4 0.398 ms staged against 0.431.
 constexpr int64_t kCorrectPointMax = 152 * 256;
 
 template <int N, typename T, bool VC>
@@ -1085,11 +1085,11 @@ __global__ void __launch_bounds__(32)
 }
 
 template <int N, typename T, bool VC, bool SRC>
-__global__ void __launch_bounds__(kCorrectThreads, std::is_same<T, double>::value ? 6 : 5) k_correct(const T *__restrict__ Rpart, const T *__restrict__ FI,
-                          const int32_t *__restrict__ ef, const T *__restrict__ metrics, int64_t E,
-                          StageCoef sc, double *__restrict__ Rout, double *__restrict__ Q, T *__restrict__ Qc,
-                          double *__restrict__ Un, T *__restrict__ Unc, double *__restrict__ acc,
-                          int *__restrict__ flag, DevPhys dph) {
+__global__ void __launch_bounds__(kCorrectThreads, std::is_same<T, double>::value ? 6 : 5)
+    k_correct(const T *__restrict__ Rpart, const T *__restrict__ FI, const int32_t *__restrict__ ef,
+              const T *__restrict__ metrics, int64_t E, StageCoef sc, double *__restrict__ Rout, double *__restrict__ Q,
+              T *__restrict__ Qc, double *__restrict__ Un, T *__restrict__ Unc, double *__restrict__ acc,
+              int *__restrict__ flag, DevPhys dph) {
   extern __shared__ double sm_raw[];
   constexpr int Np = N * N * N;
   const CorrectSmem sm(sm_raw);
@@ -1120,10 +1120,10 @@ __device__ __forceinline__ bool unused_tri_slot(int64_t t, int64_t first, int64_
 }
 
 template <int N, typename T, bool ROE>
-__global__ void __launch_bounds__(128, iface_blocks<false>()) k_iface_flux_tri(const T *__restrict__ Qtr, const T *__restrict__ Gtr, const T *__restrict__ normals,
-                                 T *__restrict__ FI, int64_t n_if, DevPhys dph, const int32_t *__restrict__ if_elem,
-                                 const float *__restrict__ nu, const int8_t *__restrict__ if_tri,
-                                 const int8_t *__restrict__ if_up) {
+__global__ void __launch_bounds__(128, iface_blocks<false>())
+    k_iface_flux_tri(const T *__restrict__ Qtr, const T *__restrict__ Gtr, const T *__restrict__ normals,
+                     T *__restrict__ FI, int64_t n_if, DevPhys dph, const int32_t *__restrict__ if_elem,
+                     const float *__restrict__ nu, const int8_t *__restrict__ if_tri, const int8_t *__restrict__ if_up) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (unused_tri_slot<N>(t, 0, n_if, if_tri)) return;
   iface_body<N, T, false, ROE>(t, Qtr, Gtr, normals, FI, n_if, dph, if_elem, nu, if_up);
@@ -1211,8 +1211,9 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const BatchCase 
       const int tid = (int)threadIdx.x % nth;
       const int64_t e = tk.begin + le;
       const bool active = le < epb && e < tk.end;
-      volume_body<N, T, false, false, 2>(e, tid, nth, active, smem + (size_t)(le < epb ? le : 0) * volume_smem_values<N>(), Qin, met,
-                        m.ef, Qtr, lift, Gtr, Rpart, c.ph, m.h, nullptr, m.if_up, m.n_interior, ClosureSpace{nullptr, 0, 0, 0});
+      volume_body<N, T, false, false, 2>(e, tid, nth, active, smem + (size_t)(le < epb ? le : 0) * volume_smem_values<N>(),
+                                         Qin, met, m.ef, Qtr, lift, Gtr, Rpart, c.ph, m.h, nullptr, m.if_up, m.n_interior,
+                                         ClosureSpace{nullptr, 0, 0, 0});
       break;
     }
     case TASK_IFACE:
@@ -1245,8 +1246,9 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const BatchCase 
     }
     case TASK_PRISM_CORRECT:
       prism_correct_body<N, T>(idx, Rpart + pts, FI, m.ef_p, pmet, ptab, m.tri_slot, m.Ep, m.E * m.Np,
-                               stage_coef(MODE_RK, L.stage, L.dts[tk.cs]), nullptr, m.Q, m.mixed ? reinterpret_cast<T *>(m.Qc) : nullptr, m.Un,
-                               reinterpret_cast<T *>(m.Unc), m.acc, &L.sync->nonfinite, c.ph);
+                               stage_coef(MODE_RK, L.stage, L.dts[tk.cs]), nullptr, m.Q,
+                               m.mixed ? reinterpret_cast<T *>(m.Qc) : nullptr, m.Un, reinterpret_cast<T *>(m.Unc), m.acc,
+                               &L.sync->nonfinite, c.ph);
       break;
     case TASK_CORRECT:
       correct_body<N, T>(tk.begin + threadIdx.x < tk.end ? tk.begin + threadIdx.x : (int64_t)1 << 62, Rpart, FI, m.ef,

@@ -207,13 +207,13 @@ static cudaError_t residual_impl(const DevMesh &m, const DevPhys &ph, int mode, 
       if ((err = launch_vcjh_phase(m, ph, 3, mode, stage, dt, Rout, st)) != cudaSuccess) return err;
     } else if (n > 0 && n <= kCorrectPointMax) {
       k_correct_point<N, T, false><<<(unsigned)((n + 31) / 32), 32, 0, st>>>(
-          Rpart, FI, m.ef, met, E, stage_coef(mode, stage, dt), Rout, m.Q, Qc, m.Un, reinterpret_cast<T *>(m.Unc), m.acc,
-          m.flag, ph);
+          Rpart, FI, m.ef, met, E, stage_coef(mode, stage, dt), Rout, m.Q, Qc, m.Un, reinterpret_cast<T *>(m.Unc),
+          m.acc, m.flag, ph);
     } else if (n > 0) {
       auto ck = has_source(ph) ? k_correct<N, T, false, true> : k_correct<N, T, false, false>;
       ck<<<(unsigned)((n + kCorrectThreads - 1) / kCorrectThreads), kCorrectThreads, correct_smem(ph), st>>>(
-          Rpart, FI, m.ef, met, E, stage_coef(mode, stage, dt), Rout, m.Q, Qc, m.Un, reinterpret_cast<T *>(m.Unc), m.acc,
-          m.flag, ph);
+          Rpart, FI, m.ef, met, E, stage_coef(mode, stage, dt), Rout, m.Q, Qc, m.Un, reinterpret_cast<T *>(m.Unc),
+          m.acc, m.flag, ph);
     }
     if ((err = launch_prism_phase(m, ph, 3, mode, stage, dt, Rout, st)) != cudaSuccess) return err;
     FR_EV_END(3);

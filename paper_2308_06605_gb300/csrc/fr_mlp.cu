@@ -35,7 +35,7 @@ __device__ __forceinline__ float sigmoid(float z) { return 1.f / (1.f + expf(-z)
 // FP32 rate, on 128 blocks).  GB300, 4096 samples, loss and gradient: 2.07 ms with one kernel per layer
 // and a thread per weight that read all samples in a chain; with this kernel and its reduction a loss,
 // gradient and optimiser step together take 37 us.
-// Tile: 32 samples fill 128 SMs at the pipeline's batch of 4096, and leave each block's partial row
+// Tile: 32 samples fill 128 SMs at the pipeline's batch of 4096 (the one size it was measured at), and leave each block's partial row
 // (NPAR + 1 floats) within the workspace of its own samples (32 WS).  Each thread owns 4 samples x 4
 // neurons (stride 16), so four k-steps take 8 16-byte shared loads for 64 FMAs; rows are LD = 68 floats
 // apart, so the 16 neuron rows a half-warp reads lie in different banks.

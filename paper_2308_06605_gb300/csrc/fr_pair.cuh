@@ -41,8 +41,8 @@ constexpr int pair_blocks() {
 // Orders it is built for, and what the volume kernel takes per launch against the scalar one (GB300).  It halves the
 // warps of an SM for the same shared memory, so it gains where enough of them remain: FP32 viscous branch
 // 40^3 p = 3 0.638 -> 0.571 ms, 4800 elements p = 4 0.106 -> 0.097, p = 5 0.193 -> 0.170, p = 7 0.562 -> 0.493 (not
-// p = 2: 0.324 -> 0.331 at 40^3, p = 6: 0.912 -> 0.946 at 24^3); inviscid 40^3 p = 2 0.098 -> 0.086, p = 3 0.209 -> 0.191,
-// 4800 elements p = 4 0.042 -> 0.041.  With the viscous branch in double-float it was slower at every size (40^3
+// p = 2: 0.324 -> 0.331 at 40^3, p = 6: 0.912 -> 0.946 at 24^3); inviscid 40^3 p = 2 0.098 -> 0.086, p = 3 0.209 ->
+// 0.191, 4800 elements p = 4 0.042 -> 0.041.  With the viscous branch in double-float it was slower at every size (40^3
 // p = 2 0.445 -> 0.460, p = 3 0.938 -> 0.960, 48^3 p = 4 3.09 -> 3.51).
 template <int N, bool VISC>
 constexpr bool pair_built() {
@@ -73,7 +73,8 @@ template <int N, bool VISC>
 __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, VISC>())
     k_volume_pair(const df32 *__restrict__ Q, const df32 *__restrict__ metrics, const int32_t *__restrict__ ef,
                   const df32 *__restrict__ Qtr, const df32 *__restrict__ liftfac, df32 *__restrict__ Gtr,
-                  df32 *__restrict__ Rpart, DevPhys dph, const int8_t *__restrict__ if_up, int64_t n_interior, int64_t E) {
+                  df32 *__restrict__ Rpart, DevPhys dph, const int8_t *__restrict__ if_up, int64_t n_interior,
+                  int64_t E) {
   extern __shared__ float4 sm_pair[];
   constexpr int Np = N * N * N, Nf = N * N, nth = volume_threads<N>();
   d2 *sH = reinterpret_cast<d2 *>(sm_pair);                    // [15][Np] transformed flux, index d*5+v

@@ -186,8 +186,8 @@ __device__ __forceinline__ void viscous_normal(const T q[5], GetG g, const T n[3
 }
 
 // Viscous stress tau = mu (du_i/dx_j + du_j/dx_i) + delta_ij lambda div u, packed (xx, yy, zz, xy,
-// xz, yz), and heat-flux term hq[j] = kappa dT/dx_j of state q with gradient G[j*5 + v] = dQ_v/dx_j.  Works on rho du_i/dx_j = G[j][1+i] - u_i G[j][0] and puts the factor 1/rho
-// into the coefficients: 40 FP64 operations, 450 FP32 instructions in double-float (57 and 700 with
+// xz, yz), and heat-flux term hq[j] = kappa dT/dx_j of state q with gradient G[j*5 + v] = dQ_v/dx_j.  Works on
+// rho du_i/dx_j = G[j][1+i] - u_i G[j][0] and puts the factor 1/rho into the coefficients: 40 FP64 operations, 450 FP32 instructions in double-float (57 and 700 with
 // du_i/dx_j itself).
 template <typename T>
 __device__ __forceinline__ void viscous_stress(const T q[5], const T u[3], T ri, const T *G, const PhysT<T> &ph,
@@ -469,10 +469,10 @@ __device__ __forceinline__ void finish_point(int64_t t, const T rv[5], T s, cons
 // point replaces its five entries by the residual, and the update runs over the block's values.  With
 // a thread reading its own point's values each 8-byte access of a warp touches ten 128-byte lines.
 // The copies into shared memory (cp.async: partial residual and the stage's two old register values) are in
-// flight while the double-float kernel gathers the fluxes.  Double-float 48^3 p = 4 1.07 -> 0.80 ms per launch (0.757 with to_double on the integer pipe)
-// (0.93 with the partial residual alone staged by plain loads), FP64 32^3 p = 4 0.447 -> 0.398 ms; bound by the
-// FP64 pipe (an addition and an FMA per value, the last stage a split into double-float) beside 3.5 GB of traffic (0.51 ms at
-// 48^3).  FP64 6 blocks per SM (40 registers), double-float 5 (48; 6 measured the same).
+// flight while the double-float kernel gathers the fluxes.  Double-float 48^3 p = 4 1.07 -> 0.80 ms per launch (0.93 with
+// the partial residual alone staged by plain loads; 0.757 since to_double runs on the integer pipe), FP64 32^3 p = 4
+// 0.447 -> 0.398 ms; bound by the FP64 pipe (an addition and an FMA per value, the last stage a split into
+// double-float) beside 3.5 GB of traffic (0.51 ms at 48^3).  FP64 6 blocks per SM (40 registers), double-float 5 (48; 6 measured the same).
 constexpr int kCorrectThreads = 256;
 
 // Shared memory of a block: the partial residual (replaced by the residual), the stage's two old register
@@ -490,7 +490,8 @@ __device__ __forceinline__ void copy_async8(double *dst, const double *src) {
 // Start the copies of everything the block reads by value; the lifted fluxes are gathered meanwhile.  base:
 // first value of the block in the registers, part: of its partial residual, n: points.
 template <typename T>
-__device__ __forceinline__ void stage_begin(const CorrectSmem &sm, const T *part, int64_t base, int n, const StageIn &in) {
+__device__ __forceinline__ void stage_begin(const CorrectSmem &sm, const T *part, int64_t base, int n,
+                                            const StageIn &in) {
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     const int i = threadIdx.x + k * kCorrectThreads;
@@ -516,8 +517,8 @@ template <typename T> constexpr bool kGatherFirst = std::is_same<T, df32>::value
 // null) and s = -1/|J| (used if threadIdx.x < n).
 template <typename T, bool SRC>
 __device__ __forceinline__ void finish_block(int64_t first, int n, const CorrectSmem &sm, Dot<T> rv[5],
-                                             const Dot<T> *last, T s, const StageCoef &c, const StageIn &in, double *__restrict__ Rout,
-                                             double *__restrict__ Q, T *__restrict__ Qc, double *__restrict__ Un,
+                                             const Dot<T> *last, T s, const StageCoef &c, const StageIn &in,
+                                             double *__restrict__ Rout, double *__restrict__ Q, T *__restrict__ Qc, double *__restrict__ Un,
                                              T *__restrict__ Unc, double *__restrict__ acc, int *__restrict__ flag,
                                              const DevPhys &dph) {
   const int me = threadIdx.x;
@@ -547,6 +548,8 @@ __device__ __forceinline__ void finish_block(int64_t first, int n, const Correct
 }
 
 inline bool has_source(const DevPhys &ph) { return ph.src_body || ph.src_sponge; }
-inline size_t correct_smem(const DevPhys &ph) { return sizeof(double) * 5 * kCorrectThreads * (has_source(ph) ? 4 : 3); }
+inline size_t correct_smem(const DevPhys &ph) {
+  return sizeof(double) * 5 * kCorrectThreads * (has_source(ph) ? 4 : 3);
+}
 
 }  // namespace frx

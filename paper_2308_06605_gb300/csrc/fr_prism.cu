@@ -73,7 +73,8 @@ __global__ void __launch_bounds__(kCorrectThreads)
                              kGatherFirst<T> ? nullptr : reinterpret_cast<const T *>(sm.r) + threadIdx.x * 5, r, line);
     s = -metrics[(e * 10 + 9) * Np + m];
   }
-  finish_block<T, SRC>(first_point + first, n, sm, r, kGatherFirst<T> ? line : nullptr, s, sc, in, Rout, Q, Qc, Un, Unc, acc, flag, dph);
+  finish_block<T, SRC>(first_point + first, n, sm, r, kGatherFirst<T> ? line : nullptr, s, sc, in, Rout, Q, Qc, Un, Unc,
+                       acc, flag, dph);
 }
 
 // dt bound per prism: cfl h / ((2p + 1) max(|u| + c)) over its points (FP64 state).

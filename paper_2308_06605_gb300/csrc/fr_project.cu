@@ -76,11 +76,12 @@ constexpr int kProjectThreads = 256;
 // Hexahedra, epb elements per block, one axis after the other through shared memory: out(i, j, k) =
 // sum_c L[k][c] sum_b L[j][b] sum_a L[i][a] in(a, b, c).  Bound by the FP64 pipe and then by memory: the
 // direct triple sum takes 160 operations per target point at p = 2 -> 4, the three passes 30.  GB300, 32^3
-// elements p = 2 -> 4, the whole call: 1.30 ms with the triple sum, device allocations for the operators
-// and the registers set by further copies -> PROJUS.
+// elements p = 2 -> 4, set_state of the source and the call: 1.30 ms with the triple sum, device allocations
+// for the operators and the registers set by further copies, 0.37 ms now, of which this kernel takes 0.30.
 template <int Nd>
 __global__ void __launch_bounds__(kProjectThreads)
-    k_project_hex(const double *__restrict__ src, StateOut out, const __grid_constant__ LineOp op, int64_t E, int Ns, int epb) {
+    k_project_hex(const double *__restrict__ src, StateOut out, const __grid_constant__ LineOp op, int64_t E, int Ns,
+                  int epb) {
   extern __shared__ double sm[];
   __shared__ double L[kMaxN * kMaxN];
   const int n0 = Ns * Ns * Ns * 5, n1 = Nd * Ns * Ns * 5, n2 = Nd * Nd * Ns * 5, n3 = Nd * Nd * Nd * 5;
@@ -142,7 +143,8 @@ static_assert(project_prism_smem_max() <= 48 * 1024, "k_project_prism launches w
 template <int Nd>
 cudaError_t launch_project(const DevMesh &a, const DevMesh &b, const std::vector<double> &L,
                            const std::vector<double> &Tt, cudaStream_t st) {
-  df32 *Qc = b.mixed ? reinterpret_cast<df32 *>(b.Qc) : nullptr, *Unc = b.mixed ? reinterpret_cast<df32 *>(b.Unc) : nullptr;
+  df32 *Qc = b.mixed ? reinterpret_cast<df32 *>(b.Qc) : nullptr;
+  df32 *Unc = b.mixed ? reinterpret_cast<df32 *>(b.Unc) : nullptr;
   if (a.E > 0) {
     LineOp op;
     std::memcpy(op.L, L.data(), L.size() * sizeof(double));
