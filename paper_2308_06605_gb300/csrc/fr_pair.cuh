@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(volume_threads<N>(), pair_blocks<N, VISC>())
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       d2 f[5];
-      transformed_flux<d2>(q, mom, en, S + 3 * d, f);
+      transformed_flux<d2>(q, mom, en, p, S + 3 * d, f);
 #pragma unroll
       for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
     }

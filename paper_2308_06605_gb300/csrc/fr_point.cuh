@@ -217,10 +217,17 @@ __device__ __forceinline__ void viscous_stress(const T q[5], const T u[3], T ri,
 // Physical flux F - Fv of Eq. 1 in the three directions: the momentum part is the symmetric tensor
 // m = rho u u + p I - tau (packed xx, yy, zz, xy, xz, yz), the energy part
 // en_j = (E + p) u_j - sum_i u_i tau_ij - hq_j, the mass part rho u itself.  With its transforms
-// (transformed_flux: 15 three-term products) 105 FP64 operations or 1200 FP32 instructions in
+// (transformed_flux: 15 three-term products) 105 FP64 operations or 1300 FP32 instructions in
 // double-float, where the contravariant form (U_d = S_d . u, then S_d tau and S_d hq for each direction d)
 // takes 150 and 1900 with the stress.  Volume kernel, GB300, double-float 48^3 p = 4: 3.80 -> 3.43 ms;
 // FP64 32^3 p = 4: 4.16 -> 3.79 ms.
+//
+// FP64 holds the pressure in the tensor's diagonal.  The double-float forms leave it out, and their transforms add
+// S p by itself: with the pressure in the tensor it is rounded there and again in the transform, and at low Mach
+// number it is much the largest part (momentum residual's error at Ma 0.1 3 to 8 % larger on hexahedra of p = 2 to 7;
+// volume launch 48^3 p = 4 3.134 ms for 3.184).
+template <typename T> constexpr bool kPressureInTensor = std::is_same<T, double>::value;
+
 template <typename T>
 __device__ __forceinline__ void physical_flux(const T q[5], const T u[3], T p, bool viscous, const T tau[6],
                                               const T hq[3], T m[6], T en[3]) {
@@ -228,7 +235,10 @@ __device__ __forceinline__ void physical_flux(const T q[5], const T u[3], T p, b
   if (!viscous) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      m[i] = muladd(p, q[1 + i], u[i]);
+      if constexpr (kPressureInTensor<T>)
+        m[i] = muladd(p, q[1 + i], u[i]);
+      else
+        m[i] = q[1 + i] * u[i];
       en[i] = H * u[i];
     }
     m[3] = q[1] * u[1];
@@ -238,10 +248,14 @@ __device__ __forceinline__ void physical_flux(const T q[5], const T u[3], T p, b
   }
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    Dot<T> d(p);
-    d.add(q[1 + i], u[i]);
-    d.plus(-tau[i]);
-    m[i] = d.raw();
+    if constexpr (kPressureInTensor<T>) {
+      Dot<T> d(p);
+      d.add(q[1 + i], u[i]);
+      d.plus(-tau[i]);
+      m[i] = d.raw();
+    } else {
+      m[i] = muladd(-tau[i], q[1 + i], u[i]);
+    }
   }
   m[3] = muladd(-tau[3], q[1], u[1]);
   m[4] = muladd(-tau[4], q[1], u[2]);
@@ -272,12 +286,15 @@ __device__ __forceinline__ void inviscid_transformed(const double q[5], const do
 
 // Transformed flux of reference direction d, F^_d = sum_j S[d][j] (F - Fv)_j (Eq. 1); Sd = S[d][0..2].
 template <typename T>
-__device__ __forceinline__ void transformed_flux(const T q[5], const T m[6], const T en[3], const T Sd[3], T f[5]) {
+__device__ __forceinline__ void transformed_flux(const T q[5], const T m[6], const T en[3], T p, const T Sd[3], T f[5]) {
   f[0] = dot3(Sd[0], q[1], Sd[1], q[2], Sd[2], q[3]);
   f[1] = dot3(Sd[0], m[0], Sd[1], m[3], Sd[2], m[4]);
   f[2] = dot3(Sd[0], m[3], Sd[1], m[1], Sd[2], m[5]);
   f[3] = dot3(Sd[0], m[4], Sd[1], m[5], Sd[2], m[2]);
   f[4] = dot3(Sd[0], en[0], Sd[1], en[1], Sd[2], en[2]);
+  if constexpr (!kPressureInTensor<T>)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) f[1 + i] = muladd(f[1 + i], Sd[i], p);
 }
 
 // ------------------------------------------------------------------------------------------

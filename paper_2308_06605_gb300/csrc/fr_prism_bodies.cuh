@@ -285,7 +285,7 @@ __device__ __forceinline__ void prism_volume_body(int64_t e, int tid, int nth, b
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
           T f[5];
-          transformed_flux<T>(qv, mom, en, S + 3 * d, f);
+          transformed_flux<T>(qv, mom, en, p, S + 3 * d, f);
 #pragma unroll
           for (int v = 0; v < 5; ++v) sH[(d * 5 + v) * Np + m] = f[v];
         }

@@ -39,3 +39,11 @@ def test_inviscid_share_of_prisms(p, n, bar):
     """Re 400, Ma 0.1: the sums carry a pressure that cancels; along the prisms' axis (z) the flow's momentum is small."""
     err = _momentum_error(p, n, "all", 400.0)
     assert (err <= bar).all(), err
+
+
+@pytest.mark.parametrize("p,n,bar", [(2, 8, (1.18e-11, 1.20e-11, 2.26e-11)), (4, 8, (6.03e-11, 6.08e-11, 8.52e-11))])
+def test_pressure_rounded_once(p, n, bar):
+    """At Ma 0.1 the pressure is 99 % of the momentum flux: one more rounding of it on the way to the transformed
+    flux raises these errors by 3 to 8 %.  The bars are 1 to 3 % above those without it (the arithmetic is deterministic)."""
+    err = _momentum_error(p, n, None, 10.0)
+    assert (err <= bar).all(), err
