@@ -111,7 +111,7 @@ __device__ __forceinline__ void prism_interp_body(int64_t t, const T *__restrict
 // Bound by FP32 issue (double-float) or the FP64 pipe.  Operator entries are read with consecutive
 // threads on consecutive addresses and once for the five variables (row-major tables cost 15 L1
 // wavefronts per load at p = 4, and were read per variable).  On the cascade passage (72 case: 25 200
-// hexahedra, 10 080 prisms, p = 4) the two volume kernels together 1.505 -> 1.260 ms in double-float, 5.06 ->
+// hexahedra, 10 080 prisms, p = 4) the two volume kernels together 1.505 -> 1.279 ms in double-float, 5.06 ->
 // 4.60 ms in FP64.
 // ------------------------------------------------------------------------------------------
 // One prism e handled by `nth` threads of the block (thread index tid in [0, nth)); every thread
